@@ -56,11 +56,10 @@ struct DevGeom {
 // compute in FP32 (GB300's FP64 rate is a small fraction of its FP32 rate, so
 // converting them per thread is not free).
 struct CoefF32 {
-  float rho0, T0, s_nu, s_b, s3, s4, l1, l2;
+  float rho0, T0;
   float rgb;  // rho0 * g beta
   float Fvx, Fvy, Q, hQ, cT2;
   float vhc;  // viscous source: 3 s_nu^2 (1/s_nu - 1/2), 0 when off
-  float pad;
 };
 
 // The collision's rates combined with the exact power-of-two scalings of the
@@ -69,13 +68,13 @@ struct CoefF32 {
 // the host in FP64, and rounded once for the FP32 kernels.
 template <typename T>
 struct CollideK {
-  T hFx;                     // Fvx / 2
+  T hFx, hFy, hrgb;          // Fvx / 2, Fvy / 2, rho0 g beta / 2
   T al, be;                  // -(s_b + s_nu) / 4, (s_nu - s_b) / 4 (the k~20, k~02 block)
-  T snu4, snur4;             // (1 - s_nu) / 4, s_nu rho0 / 4
-  T s3m4, s3r4, hs3q;        // (1 - s3) / 4, s3 rho0 / 4, (1 - s3 / 2) / 12
-  T s4m4, s4r4, s4n, s4r9;   // (1 - s4) / 4, s4 rho0 / 4, s4 / 36, s4 rho0 / 36
-  T l1m2, l1T2, l2m2, l2T2;  // (1 - l1) / 2, l1 T0 / 2, (1 - l2) / 2, l2 T0 / 2
-  T srcq2, srct2;            // (1 - l2 / 2) cT2 / 2, l2 cT2 / 2
+  T snu4, nsnur4;            // (1 - s_nu) / 4, -s_nu rho0 / 4
+  T s3m4, s3r4, s3f, s3Fx;   // (1 - s3) / 4, s3 rho0 / 4, (1 - s3 / 2) / 6, (1 - s3 / 2) / 12 Fvx
+  T s4m4, ns4r4, s4n;        // (1 - s4) / 4, -s4 rho0 / 4, s4 / 36
+  T l1m2, l1T2, l2m2, nl2T2; // (1 - l1) / 2, l1 T0 / 2, (1 - l2) / 2, -l2 T0 / 2
+  T srcq2, srct2, srcQ;      // (1 - l2 / 2) cT2 / 2, l2 cT2 / 2, srcq2 Q
 };
 
 struct DevCoef {
@@ -93,51 +92,51 @@ struct DevCoef {
 inline void fill_f32(DevCoef& k) {
   CollideK<double>& d = k.kd;
   d.hFx = 0.5 * k.Fvx;
+  d.hFy = 0.5 * k.Fvy;
+  d.hrgb = 0.5 * k.rho0 * k.gbeta;
   d.al = -0.25 * (k.s_b + k.s_nu);
   d.be = 0.25 * (k.s_nu - k.s_b);
   d.snu4 = 0.25 * (1.0 - k.s_nu);
-  d.snur4 = 0.25 * k.s_nu * k.rho0;
+  d.nsnur4 = -0.25 * k.s_nu * k.rho0;
   d.s3m4 = 0.25 * (1.0 - k.s3);
   d.s3r4 = 0.25 * k.s3 * k.rho0;
-  d.hs3q = (1.0 - 0.5 * k.s3) / 12.0;
+  d.s3f = (1.0 - 0.5 * k.s3) / 6.0;
+  d.s3Fx = (1.0 - 0.5 * k.s3) / 12.0 * k.Fvx;
   d.s4m4 = 0.25 * (1.0 - k.s4);
-  d.s4r4 = 0.25 * k.s4 * k.rho0;
+  d.ns4r4 = -0.25 * k.s4 * k.rho0;
   d.s4n = k.s4 / 36.0;
-  d.s4r9 = k.s4 * k.rho0 / 36.0;
   d.l1m2 = 0.5 * (1.0 - k.l1);
   d.l1T2 = 0.5 * k.l1 * k.T0;
   d.l2m2 = 0.5 * (1.0 - k.l2);
-  d.l2T2 = 0.5 * k.l2 * k.T0;
+  d.nl2T2 = -0.5 * k.l2 * k.T0;
   d.srcq2 = 0.5 * (1.0 - 0.5 * k.l2) * k.cT2;
   d.srct2 = 0.5 * k.l2 * k.cT2;
+  d.srcQ = d.srcq2 * k.Q;
   CollideK<float>& e = k.kf;
   e.hFx = (float)d.hFx;
+  e.hFy = (float)d.hFy;
+  e.hrgb = (float)d.hrgb;
   e.al = (float)d.al;
   e.be = (float)d.be;
   e.snu4 = (float)d.snu4;
-  e.snur4 = (float)d.snur4;
+  e.nsnur4 = (float)d.nsnur4;
   e.s3m4 = (float)d.s3m4;
   e.s3r4 = (float)d.s3r4;
-  e.hs3q = (float)d.hs3q;
+  e.s3f = (float)d.s3f;
+  e.s3Fx = (float)d.s3Fx;
   e.s4m4 = (float)d.s4m4;
-  e.s4r4 = (float)d.s4r4;
+  e.ns4r4 = (float)d.ns4r4;
   e.s4n = (float)d.s4n;
-  e.s4r9 = (float)d.s4r9;
   e.l1m2 = (float)d.l1m2;
   e.l1T2 = (float)d.l1T2;
   e.l2m2 = (float)d.l2m2;
-  e.l2T2 = (float)d.l2T2;
+  e.nl2T2 = (float)d.nl2T2;
   e.srcq2 = (float)d.srcq2;
   e.srct2 = (float)d.srct2;
+  e.srcQ = (float)d.srcQ;
   CoefF32& o = k.f;
   o.rho0 = (float)k.rho0;
   o.T0 = (float)k.T0;
-  o.s_nu = (float)k.s_nu;
-  o.s_b = (float)k.s_b;
-  o.s3 = (float)k.s3;
-  o.s4 = (float)k.s4;
-  o.l1 = (float)k.l1;
-  o.l2 = (float)k.l2;
   o.rgb = (float)(k.rho0 * k.gbeta);
   o.Fvx = (float)k.Fvx;
   o.Fvy = (float)k.Fvy;
@@ -145,7 +144,6 @@ inline void fill_f32(DevCoef& k) {
   o.hQ = (float)(0.5 * k.Q);
   o.cT2 = (float)k.cT2;
   o.vhc = (float)(k.vh ? 3.0 * k.s_nu * k.s_nu * (1.0 / k.s_nu - 0.5) : 0.0);
-  o.pad = 0.0f;
 }
 
 struct StepArgs {

@@ -37,6 +37,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "clbm_internal.h"
@@ -223,11 +224,45 @@ __device__ __forceinline__ void sr_words(uint32_t key, int q, uint32_t& r0, uint
 }
 
 // ---------------------------------------------------------------------------
+// Arithmetic with the rounding points written out.  The same node update is
+// compiled into several kernels (plane tiles, boundary nodes, batches, lattices
+// resident in shared memory); left to itself the compiler contracts a * b + c
+// differently in each, and a lattice would then depend on the kernel that
+// advanced it.  With every multiply-add explicit they agree bit for bit.
+// ---------------------------------------------------------------------------
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
+#else
+inline float fma_(float a, float b, float c) { return std::fma(a, b, c); }
+inline double fma_(double a, double b, double c) { return std::fma(a, b, c); }
+template <typename R> inline R mul_(R a, R b) { return a * b; }
+template <typename R> inline R add_(R a, R b) { return a + b; }
+template <typename R> inline R sub_(R a, R b) { return a - b; }
+#endif
+// 1 / rho.  FP32: to within 2 ulp (hardware approximation), which the FP32
+// parity bound leaves ample room for; FP64: the exact quotient.
+__host__ __device__ __forceinline__ double rcp_(double v) { return 1.0 / v; }
+__host__ __device__ __forceinline__ float rcp_(float v) {
+#ifdef __CUDA_ARCH__
+  return __fdividef(1.0f, v);
+#else
+  return 1.0f / v;
+#endif
+}
+
+// ---------------------------------------------------------------------------
 // Constants in the compute type
 // ---------------------------------------------------------------------------
 template <typename R>
 struct Co {
-  R rho0, T0, s_nu, s_b, s3, s4, l1, l2;
+  R rho0, T0;
   R rgb;   // rho0 * g beta
   R Fvx, Fvy, Q, hQ, cT2;
   R vhc;   // viscous source: Q_v = vhc (k~11^2 + (k~20 - k~02)^2 / 4) / rho^2
@@ -242,12 +277,6 @@ __host__ __device__ __forceinline__ Co<R> make_co(const DevCoef& c) {
     const CoefF32& f = c.f;
     o.rho0 = f.rho0;
     o.T0 = f.T0;
-    o.s_nu = f.s_nu;
-    o.s_b = f.s_b;
-    o.s3 = f.s3;
-    o.s4 = f.s4;
-    o.l1 = f.l1;
-    o.l2 = f.l2;
     o.rgb = f.rgb;
     o.Fvx = f.Fvx;
     o.Fvy = f.Fvy;
@@ -259,12 +288,6 @@ __host__ __device__ __forceinline__ Co<R> make_co(const DevCoef& c) {
     o.k = c.kd;
     o.rho0 = (R)c.rho0;
     o.T0 = (R)c.T0;
-    o.s_nu = (R)c.s_nu;
-    o.s_b = (R)c.s_b;
-    o.s3 = (R)c.s3;
-    o.s4 = (R)c.s4;
-    o.l1 = (R)c.l1;
-    o.l2 = (R)c.l2;
     o.rgb = (R)(c.rho0 * c.gbeta);
     o.Fvx = (R)c.Fvx;
     o.Fvy = (R)c.Fvy;
@@ -280,27 +303,19 @@ __host__ __device__ __forceinline__ Co<R> make_co(const DevCoef& c) {
 // ---------------------------------------------------------------------------
 // 1-D central-moment transform over the velocities {-1, 0, +1} and back
 // ---------------------------------------------------------------------------
+// First and second order from the row's sum c0, difference s = a+ - a- and
+// sum q = a+ + a-; n2u = -2 u, uu = u^2.
 template <typename R>
-__host__ __device__ __forceinline__ void fwd1(R am, R a0, R ap, R u, R& c0, R& c1, R& c2) {
-  c0 = am + a0 + ap;
-  const R s = ap - am;
-  c1 = s - u * c0;
-  c2 = (ap + am) - (u + u) * s + u * u * c0;
+__host__ __device__ __forceinline__ void fwd1p(R c0, R s, R q, R u, R n2u, R uu, R& c1, R& c2) {
+  c1 = fma_(-u, c0, s);
+  c2 = fma_(uu, c0, fma_(n2u, s, q));
 }
-// The same with c0 formed from the pair sum ap + am (one add fewer).
+// The same from the three populations.
 template <typename R>
-__host__ __device__ __forceinline__ void fwd1q(R am, R a0, R ap, R u, R& c0, R& c1, R& c2) {
-  const R q = ap + am;
-  c0 = q + a0;
-  const R s = ap - am;
-  c1 = s - u * c0;
-  c2 = q - (u + u) * s + u * u * c0;
-}
-// The same from the row's sum c0, difference ap - am and sum ap + am.
-template <typename R>
-__host__ __device__ __forceinline__ void fwd1p(R c0, R s, R q, R u, R& c1, R& c2) {
-  c1 = s - u * c0;
-  c2 = q - (u + u) * s + u * u * c0;
+__host__ __device__ __forceinline__ void fwd1(R am, R a0, R ap, R u, R n2u, R uu, R& c0, R& c1, R& c2) {
+  const R q = add_(ap, am), s = sub_(ap, am);
+  c0 = add_(q, a0);
+  fwd1p(c0, s, q, u, n2u, uu, c1, c2);
 }
 template <typename R>
 __host__ __device__ __forceinline__ void inv1(R c0, R c1, R c2, R u, R& am, R& a0, R& ap) {
@@ -317,11 +332,11 @@ __host__ __device__ __forceinline__ void inv1(R c0, R c1, R c2, R u, R& am, R& a
 template <typename R>
 __host__ __device__ __forceinline__ void inv1h(R c0, R c1h, R c2h, R u2, R hu, R hu2, R& am, R& a0,
                                                R& ap) {
-  const R h1 = c1h + hu * c0;
-  const R h2 = c2h + u2 * c1h + hu2 * c0;
-  a0 = c0 - R(2) * h2;
-  ap = h2 + h1;
-  am = h2 - h1;
+  const R h1 = fma_(hu, c0, c1h);
+  const R h2 = fma_(hu2, c0, fma_(u2, c1h, c2h));
+  a0 = fma_(R(-2), h2, c0);
+  ap = add_(h2, h1);
+  am = sub_(h2, h1);
 }
 
 // ---------------------------------------------------------------------------
@@ -331,188 +346,120 @@ __host__ __device__ __forceinline__ void inv1h(R c0, R c1h, R c2h, R u2, R hu, R
 // VH: add the viscous dissipation source Q_v (Sec. 3.2), read from the
 // pre-collision non-equilibrium central moments; it is returned in qv.  The
 // Boussinesq force uses T without Q_v/2 (Q_v needs u, which needs the force).
-// The combined constants: from the host (HK), or formed here from the rates.
-// The FP32-storage kernels, memory-bound, run 1-1.4 % faster as compiled with
-// the latter and with the (k~20, k~02) block and the first thermal moments
-// grouped as plain relaxations; the 16-bit and FP64 ones, bound by issue or by
-// the FP64 pipe, with the former and the regrouped sums, which take fewer
-// operations (measured A/B on one GB300).
-template <typename R, bool HK>
-__host__ __device__ __forceinline__ CollideK<R> collide_k(const Co<R>& c) {
-  if constexpr (HK) {
-    return c.k;
-  } else {
-    const R q4 = R(0.25), h = R(0.5), third = R(1.0 / 3.0);
-    CollideK<R> k;
-    k.hFx = h * c.Fvx;
-    k.al = -(c.s_b + c.s_nu) * q4;
-    k.be = (c.s_nu - c.s_b) * q4;
-    k.snu4 = (R(1) - c.s_nu) * q4;
-    k.snur4 = c.s_nu * c.rho0 * q4;
-    k.s3m4 = (R(1) - c.s3) * q4;
-    k.s3r4 = c.s3 * c.rho0 * q4;
-    k.hs3q = (R(1) - h * c.s3) * third * q4;
-    k.s4m4 = (R(1) - c.s4) * q4;
-    k.s4r4 = c.s4 * c.rho0 * q4;
-    k.s4n = c.s4 * R(1.0 / 36.0);
-    k.s4r9 = c.s4 * c.rho0 * R(1.0 / 36.0);
-    k.l1m2 = (R(1) - c.l1) * h;
-    k.l1T2 = c.l1 * c.T0 * h;
-    k.l2m2 = (R(1) - c.l2) * h;
-    k.l2T2 = c.l2 * c.T0 * h;
-    k.srcq2 = (R(1) - h * c.l2) * c.cT2 * h;
-    k.srct2 = c.l2 * c.cT2 * h;
-    return k;
-  }
-}
-
-template <typename R, bool VH = false, bool HK = true>
+template <typename R, bool VH = false>
 __host__ __device__ __forceinline__ void collide(const Co<R>& c, R (&d)[9], R (&h)[5], R& qv) {
-  const R third = R(1.0 / 3.0);
-  // Eq. 25 (T - T0 = sum h + Q/2) and Eq. 2
-  const R k20 = h[1] + h[3], k02 = h[2] + h[4];
-  const R sh = (h[0] + k20) + k02;
-  const R dT = sh + c.hQ;
-  const R Fx = c.Fvx;
-  const R Fy = c.Fvy + c.rgb * dT;
+  const CollideK<R>& k = c.k;
+  // Eq. 25 (T - T0 = sum h + Q/2) and half of the force of Eq. 2
+  const R k20 = add_(h[1], h[3]), k02 = add_(h[2], h[4]);
+  const R sh = add_(add_(h[0], k20), k02);
+  const R dT = add_(sh, c.hQ);
+  const R hFy = fma_(k.hrgb, dT, k.hFy);
   // Eq. 12 (sum_i w_i e_i = 0, so the rest state adds nothing to j), from the
   // sums and differences of each velocity row, which the x-pass below reuses
-  const R ms = d[8] - d[7], mq = d[8] + d[7];  // e_y = -1
-  const R zs = d[1] - d[3], zq = d[1] + d[3];  // e_y =  0
-  const R ps = d[5] - d[6], pq = d[5] + d[6];  // e_y = +1
-  // row sums: from the pair sums (one add fewer each) where the kernels are
-  // bound by issue, in the grouping the FP32-storage kernels run fastest with otherwise
-  const R m0 = HK ? mq + d[4] : (d[7] + d[4]) + d[8];
-  const R z0 = HK ? zq + d[0] : (d[3] + d[0]) + d[1];
-  const R p0 = HK ? pq + d[2] : (d[6] + d[2]) + d[5];
-  const R drho = (m0 + z0) + p0;
-  const R rho = c.rho0 + drho;
-  const R jx = (ms + zs) + ps;
-  const R jy = p0 - m0;
-  // FP32: the reciprocal to within 2 ulp (hardware approximation), which the
-  // FP32 parity bound leaves ample room for; FP64: the exact quotient
-  R inv_rho = R(1) / rho;
-#ifdef __CUDA_ARCH__
-  if constexpr (std::is_same<R, float>::value) inv_rho = __fdividef(1.0f, rho);
-#endif
-  const R hFx = R(0.5) * Fx, hFy = R(0.5) * Fy;
-  const R ux = (jx + hFx) * inv_rho;
-  const R uy = (jy + hFy) * inv_rho;
+  const R ms = sub_(d[8], d[7]), mq = add_(d[8], d[7]);  // e_y = -1
+  const R zs = sub_(d[1], d[3]), zq = add_(d[1], d[3]);  // e_y =  0
+  const R ps = sub_(d[5], d[6]), pq = add_(d[5], d[6]);  // e_y = +1
+  const R m0 = add_(mq, d[4]), z0 = add_(zq, d[0]), p0 = add_(pq, d[2]);
+  const R yq = add_(p0, m0), jy = sub_(p0, m0);
+  const R drho = add_(yq, z0);
+  const R jx = add_(add_(ms, zs), ps);
+  const R inv_rho = rcp_(add_(c.rho0, drho));
+  const R ux = mul_(add_(jx, k.hFx), inv_rho);
+  const R uy = mul_(add_(jy, hFy), inv_rho);
+  const R ux2 = mul_(ux, ux), uy2 = mul_(uy, uy);
+  const R n2ux = mul_(R(-2), ux), n2uy = mul_(R(-2), uy);
 
   // central moments of the deviations: x-pass per velocity row, then y-pass
   R xm1, xm2, xz1, xz2, xp1, xp2;
-  fwd1p(m0, ms, mq, ux, xm1, xm2);  // e_y = -1
-  fwd1p(z0, zs, zq, ux, xz1, xz2);  // e_y =  0
-  fwd1p(p0, ps, pq, ux, xp1, xp2);  // e_y = +1
+  fwd1p(m0, ms, mq, ux, n2ux, ux2, xm1, xm2);  // e_y = -1
+  fwd1p(z0, zs, zq, ux, n2ux, ux2, xz1, xz2);  // e_y =  0
+  fwd1p(p0, ps, pq, ux, n2ux, ux2, xp1, xp2);  // e_y = +1
   R b01, b02, b10, b11, b12, b20, b21, b22;
-  const R b00 = drho;
-  fwd1p(drho, jy, p0 + m0, uy, b01, b02);
-  if constexpr (HK) {
-    fwd1q(xm1, xz1, xp1, uy, b10, b11, b12);
-    fwd1q(xm2, xz2, xp2, uy, b20, b21, b22);
-  } else {
-    fwd1(xm1, xz1, xp1, uy, b10, b11, b12);
-    fwd1(xm2, xz2, xp2, uy, b20, b21, b22);
-  }
+  fwd1p(drho, jy, yq, uy, n2uy, uy2, b01, b02);
+  fwd1(xm1, xz1, xp1, uy, n2uy, uy2, b10, b11, b12);
+  fwd1(xm2, xz2, xp2, uy, n2uy, uy2, b20, b21, b22);
 
   // Eq. 7-10, minus the rest-state moments rho0 kappa_m(ux) kappa_n(uy),
   // kappa = (1, -u, 1/3 + u^2).  Each post-collision moment D_mn is formed
   // scaled by 2^-[m > 0] 2^-[n > 0] (H_mn; exact scalings folded into the
   // rates), the form the back-transformation inv1h takes on both passes.
-  const R ux2 = ux * ux, uy2 = uy * uy;
-  const R r0 = c.rho0;
-  const CollideK<R> k = collide_k<R, HK>(c);
-  const R H00 = b00;
-  const R H10 = R(0.5) * b10 + k.hFx;  // D10 / 2, D10 = b10 + Fx
-  const R H01 = R(0.5) * b01 + hFy;    // D01 / 2, D01 = b01 + Fy
+  const R third = R(1.0 / 3.0);
+  const R H10 = fma_(R(0.5), b10, k.hFx);  // D10 / 2, D10 = b10 + Fx
+  const R H01 = fma_(R(0.5), b01, hFy);    // D01 / 2, D01 = b01 + Fy
   // the (k~20, k~02) block: with a = k~ - its equilibrium (a20, a02 below),
   // D20 = k~20 - a20 + ((1 - s_b)(a20 + a02) + (1 - s_nu)(a20 - a02)) / 2, so
   // D20 / 2 = b20 / 2 + al a20 + be a02 and D02 / 2 = b02 / 2 + be a20 + al a02
-  const R tdr = third * drho;
-  const R a20 = r0 * ux2 + b20 - tdr;
-  const R a02 = r0 * uy2 + b02 - tdr;
-  R H20, H02;  // D20 / 2, D02 / 2
-  if constexpr (HK) {
-    H20 = R(0.5) * b20 + k.al * a20 + k.be * a02;
-    H02 = R(0.5) * b02 + k.be * a20 + k.al * a02;
-  } else {  // the same sums grouped as the FP32-storage kernels run fastest
-    const R sum = (R(1) - c.s_b) * R(0.25) * (a20 + a02);
-    const R dif = k.snu4 * (a20 - a02);
-    const R htdr = R(0.5) * tdr, hr0 = R(0.5) * r0;
-    H20 = htdr - hr0 * ux2 + (sum + dif);
-    H02 = htdr - hr0 * uy2 + (sum - dif);
-  }
-  const R H11 = k.snu4 * b11 - k.snur4 * (ux * uy);  // D11 / 4
-  const R tx = third + ux2, ty = third + uy2;
-  const R H21 = k.s3m4 * b21 + k.s3r4 * (tx * uy) + k.hs3q * Fy;  // D21 / 4
-  const R H12 = k.s3m4 * b12 + k.s3r4 * (ux * ty) + k.hs3q * Fx;  // D12 / 4
-  const R H22 = k.s4m4 * b22 - k.s4r4 * (third * (ux2 + uy2) + ux2 * uy2) + k.s4n * drho;  // D22 / 4
-  R Qt = c.Q;
+  const R a20 = fma_(c.rho0, ux2, fma_(-third, drho, b20));
+  const R a02 = fma_(c.rho0, uy2, fma_(-third, drho, b02));
+  const R H20 = fma_(k.be, a02, fma_(k.al, a20, mul_(R(0.5), b20)));
+  const R H02 = fma_(k.be, a20, fma_(k.al, a02, mul_(R(0.5), b02)));
+  const R uxy = mul_(ux, uy);
+  const R H11 = fma_(k.nsnur4, uxy, mul_(k.snu4, b11));  // D11 / 4
+  const R tx = add_(third, ux2), ty = add_(third, uy2);
+  const R H21 = fma_(k.s3f, hFy, fma_(k.s3r4, mul_(tx, uy), mul_(k.s3m4, b21)));  // D21 / 4
+  const R H12 = fma_(k.s3r4, mul_(ux, ty), fma_(k.s3m4, b12, k.s3Fx));            // D12 / 4
+  const R w22 = fma_(ux2, ty, mul_(third, uy2));  // (ux^2 + uy^2) / 3 + ux^2 uy^2
+  const R H22 = fma_(k.ns4r4, w22, fma_(k.s4n, drho, mul_(k.s4m4, b22)));  // D22 / 4
   qv = R(0);
   if constexpr (VH) {
-    const R k11 = r0 * ux * uy + b11;
-    const R kd = r0 * (ux2 - uy2) + (b20 - b02);
-    qv = c.vhc * inv_rho * inv_rho * (k11 * k11 + R(0.25) * kd * kd);
-    Qt = c.Q + qv;
+    const R k11 = fma_(c.rho0, uxy, b11);
+    const R kd = fma_(c.rho0, sub_(ux2, uy2), sub_(b20, b02));
+    const R k2 = fma_(mul_(R(0.25), kd), kd, mul_(k11, k11));
+    qv = mul_(mul_(c.vhc, mul_(inv_rho, inv_rho)), k2);
   }
 
   // back-transformation: y-pass inverse per x-order (rows m = 1, 2 come out
   // halved, as the x-pass wants them), then x-pass inverse per row
-  const R ux2x = ux + ux, uy2x = uy + uy;
-  const R hux = R(0.5) * ux, huy = R(0.5) * uy;
-  const R hux2 = hux * ux, huy2 = huy * uy;
+  const R hux = mul_(R(0.5), ux), huy = mul_(R(0.5), uy);
+  const R hux2 = mul_(R(0.5), ux2), huy2 = mul_(R(0.5), uy2);
   R ym0, yz0, yp0, ym1, yz1, yp1, ym2, yz2, yp2;
-  inv1h(H00, H01, H02, uy2x, huy, huy2, ym0, yz0, yp0);
-  inv1h(H10, H11, H12, uy2x, huy, huy2, ym1, yz1, yp1);
-  inv1h(H20, H21, H22, uy2x, huy, huy2, ym2, yz2, yp2);
-  inv1h(ym0, ym1, ym2, ux2x, hux, hux2, d[7], d[4], d[8]);
-  inv1h(yz0, yz1, yz2, ux2x, hux, hux2, d[3], d[0], d[1]);
-  inv1h(yp0, yp1, yp2, ux2x, hux, hux2, d[6], d[2], d[5]);
+  inv1h(drho, H01, H02, -n2uy, huy, huy2, ym0, yz0, yp0);
+  inv1h(H10, H11, H12, -n2uy, huy, huy2, ym1, yz1, yp1);
+  inv1h(H20, H21, H22, -n2uy, huy, huy2, ym2, yz2, yp2);
+  inv1h(ym0, ym1, ym2, -n2ux, hux, hux2, d[7], d[4], d[8]);
+  inv1h(yz0, yz1, yz2, -n2ux, hux, hux2, d[3], d[0], d[1]);
+  inv1h(yp0, yp1, yp2, -n2ux, hux, hux2, d[6], d[2], d[5]);
 
   // thermal (Eq. 15-20, 23-24) on deviations from w^T T0; kappa^T = (1, -u, cT2 + u^2)
-  const R k10 = h[1] - h[3], k01 = h[2] - h[4];
+  const R k10 = sub_(h[1], h[3]), k01 = sub_(h[2], h[4]);
   // (1 - l1)(k10 - ux sh) / 2 + l1 T0 ux / 2 = l1m2 k10 + ux (l1T2 - l1m2 sh)
-  const R w1 = HK ? k.l1T2 - k.l1m2 * sh : R(0);
-  const R t20 = k20 - (ux + ux) * k10 + ux2 * sh;
-  const R t02 = k02 - (uy + uy) * k01 + uy2 * sh;
-  const R dTt = VH ? sh + R(0.5) * Qt : dT;  // Eq. 25 with the total source
+  const R w1 = fma_(-k.l1m2, sh, k.l1T2);
+  const R t20 = fma_(ux2, sh, fma_(n2ux, k10, k20));
+  const R t02 = fma_(uy2, sh, fma_(n2uy, k01, k02));
   // post-collision thermal moments, first and second order halved (G = E / 2)
   // so that the back-transformation needs no halving of its own
-  const R E00 = sh + Qt;
-  R G10, G01;
-  if constexpr (HK) {
-    G10 = k.l1m2 * k10 + ux * w1;
-    G01 = k.l1m2 * k01 + uy * w1;
+  R E00, src2h;
+  if constexpr (VH) {
+    const R Qt = add_(c.Q, qv);
+    E00 = add_(sh, Qt);
+    src2h = fma_(k.srct2, fma_(R(0.5), Qt, sh), mul_(k.srcq2, Qt));  // Eq. 25 with the total source
   } else {
-    G10 = k.l1m2 * (k10 - ux * sh) + k.l1T2 * ux;
-    G01 = k.l1m2 * (k01 - uy * sh) + k.l1T2 * uy;
+    E00 = add_(sh, c.Q);
+    src2h = fma_(k.srct2, dT, k.srcQ);
   }
-  const R src2h = k.srcq2 * Qt + k.srct2 * dTt;
-  const R G20 = k.l2m2 * t20 - k.l2T2 * ux2 + src2h;
-  const R G02 = k.l2m2 * t02 - k.l2T2 * uy2 + src2h;
-  const R q10 = G10 + hux * E00, q01 = G01 + huy * E00;  // halves of the raw moments
-  const R q20 = G20 + ux2x * G10 + hux2 * E00;
-  const R q02 = G02 + uy2x * G01 + huy2 * E00;
-  h[0] = E00 - R(2) * (q20 + q02);
-  h[1] = q20 + q10;
-  h[3] = q20 - q10;
-  h[2] = q02 + q01;
-  h[4] = q02 - q01;
+  const R G10 = fma_(ux, w1, mul_(k.l1m2, k10));
+  const R G01 = fma_(uy, w1, mul_(k.l1m2, k01));
+  const R G20 = fma_(k.l2m2, t20, fma_(k.nl2T2, ux2, src2h));
+  const R G02 = fma_(k.l2m2, t02, fma_(k.nl2T2, uy2, src2h));
+  const R q10 = fma_(hux, E00, G10), q01 = fma_(huy, E00, G01);  // halves of the raw moments
+  const R q20 = fma_(hux2, E00, fma_(-n2ux, G10, G20));
+  const R q02 = fma_(huy2, E00, fma_(-n2uy, G01, G02));
+  h[0] = fma_(R(-2), add_(q20, q02), E00);
+  h[1] = add_(q20, q10);
+  h[3] = sub_(q20, q10);
+  h[2] = add_(q02, q01);
+  h[4] = sub_(q02, q01);
 }
 
+// HK is of no effect: every storage type takes the same constants.
 template <typename R, bool HK = true>
 __host__ __device__ __forceinline__ void collide_any(const Co<R>& c, bool vh, R (&d)[9], R (&h)[5],
                                                      R& qv) {
   if (vh)
-    collide<R, true, HK>(c, d, h, qv);
+    collide<R, true>(c, d, h, qv);
   else
-    collide<R, false, HK>(c, d, h, qv);
+    collide<R, false>(c, d, h, qv);
 }
-
-// Which constants the kernels of storage type S take (the same in every
-// kernel of one storage type, so that they all compute the same numbers).
-template <typename S>
-constexpr bool kHostK = !std::is_same<S, float>::value;
 
 // Pre-collision equilibrium deviations (central moments Eq. 9 and Eq. 19 minus
 // the rest-state moments) at (rho, u, T).
@@ -552,8 +499,11 @@ __host__ __device__ __forceinline__ void equilibrium(const Co<R>& c, R rho, R ux
 // ---------------------------------------------------------------------------
 template <typename R>
 __host__ __device__ __forceinline__ R wall_temperature(R b1, R b2, R b3, R ne, R T1, R T2, bool have2) {
-  if (have2) return (R(9) * b1 * T1 - b1 * T2 + R(3) * ne * b3) / (R(8) * b1 + R(3) * ne * b2);
-  return (R(2) * b1 * T1 + ne * b3) / (R(2) * b1 + ne * b2);
+  const R n3 = mul_(ne, b3);
+  if (have2)
+    return fma_(mul_(R(9), b1), T1, fma_(R(3), n3, -mul_(b1, T2))) /
+           fma_(R(8), b1, mul_(R(3), mul_(ne, b2)));
+  return fma_(mul_(R(2), b1), T1, n3) / fma_(R(2), b1, mul_(ne, b2));
 }
 
 // Walls at the fraction q of a link (no counterpart in the paper; q = 1/2 is
@@ -564,11 +514,13 @@ __host__ __device__ __forceinline__ R wall_temperature(R b1, R b2, R b3, R ne, R
 // through (0, T_w), (q, T1) when T2 is missing).
 template <typename R>
 __host__ __device__ __forceinline__ R wall_temperature_q(R b1, R b2, R b3, R ne, R q, R T1, R T2, bool have2) {
+  const R qn = mul_(q, ne);
   if (have2) {
-    const R qq = q * (R(1) + q), p = R(1) + q;
-    return (b3 * qq * ne + b1 * (p * p * T1 - q * q * T2)) / (b1 * (R(1) + R(2) * q) + b2 * qq * ne);
+    const R p = add_(R(1), q), qqn = mul_(qn, p);
+    const R e = fma_(mul_(p, p), T1, -mul_(mul_(q, q), T2));
+    return fma_(b1, e, mul_(b3, qqn)) / fma_(b1, fma_(R(2), q, R(1)), mul_(b2, qqn));
   }
-  return (b3 * q * ne + b1 * T1) / (b1 + b2 * q * ne);
+  return fma_(b1, T1, mul_(b3, qn)) / fma_(b2, qn, b1);
 }
 
 // dT/dn at such a wall from the same profile.
@@ -591,17 +543,19 @@ __host__ __device__ __forceinline__ R wall_gradient_q(R ne, R q, R Tw, R T1, R T
 template <typename R>
 __host__ __device__ __forceinline__ R midpoint_temperature_q(R q, R Tw, R T1, R T2, bool have2, R T3,
                                                              bool have3, bool dirichlet) {
-  const R m = R(2) * q - R(1);  // 2 (q - 1/2)
+  const R m = fma_(R(2), q, R(-1));  // 2 (q - 1/2)
+  const R p1 = add_(R(1), q);
   if (q >= R(0.5) || !dirichlet) {
-    if (!have2) return Tw + (T1 - Tw) * m / (R(2) * q);
-    const R p = R(1) + q;
-    return R(3) / (R(4) * q * p) * Tw + R(3) * m / (R(4) * q) * T1 - m / (R(4) * p) * T2;
+    if (!have2) return fma_(sub_(T1, Tw), m / mul_(R(2), q), Tw);
+    return fma_(R(3) / mul_(R(4), mul_(q, p1)), Tw,
+                fma_(mul_(R(3), m) / mul_(R(4), q), T1, mul_(-(m / mul_(R(4), p1)), T2)));
   }
   if (have2 && have3) {
-    const R p1 = R(1) + q, p2 = R(2) + q;
-    return R(15) / (R(4) * p1 * p2) * Tw + R(5) * m / (R(4) * p1) * T2 - R(3) * m / (R(4) * p2) * T3;
+    const R p2 = add_(R(2), q);
+    return fma_(R(15) / mul_(R(4), mul_(p1, p2)), Tw,
+                fma_(mul_(R(5), m) / mul_(R(4), p1), T2, mul_(-(mul_(R(3), m) / mul_(R(4), p2)), T3)));
   }
-  if (have2) return Tw + (T2 - Tw) * m / (R(2) * (R(1) + q));
+  if (have2) return fma_(sub_(T2, Tw), m / mul_(R(2), p1), Tw);
   return Tw;
 }
 
@@ -614,7 +568,7 @@ __device__ __forceinline__ R node_T(const S* __restrict__ src, long long plane, 
 #pragma unroll
   for (int q = 10; q < 14; ++q) s += to_r(src[q * plane + idx]);
   R t = c.T0 + s - c.hQ;
-  if (c.vhc != R(0)) t -= R(0.5) * to_r(src[14 * plane + idx]);
+  if (c.vhc != R(0)) t = fma_(R(-0.5), to_r(src[14 * plane + idx]), t);
   return t;
 }
 
@@ -678,12 +632,14 @@ __device__ __forceinline__ void fixup(const DevGeom& g, const Co<R>& c, const S*
             uwy = (R)g.side_u[sd][1];
           }
           const R w6 = j <= 4 ? R(6.0 / 9.0) : R(6.0 / 36.0);
-          d[j] += w6 * c.rho0 * (R(ex) * uwx + R(ey) * uwy);
+          d[j] = fma_(mul_(w6, c.rho0), add_(mul_(R(ex), uwx), mul_(R(ey), uwy)), d[j]);
         }
       } else if (q < R(0.5)) {  // f_i* interpolated to the point 1 - 2q behind x_f
-        d[j] = R(2) * q * fi + (R(1) - R(2) * q) * to_r(src[i * plane + i2]);
+        const R q2 = mul_(R(2), q);
+        d[j] = fma_(q2, fi, mul_(sub_(R(1), q2), to_r(src[i * plane + i2])));
       } else {  // the reflected value, 2q - 1 beyond x_f, interpolated with f_j* at x_f
-        d[j] = fi / (R(2) * q) + (R(2) * q - R(1)) / (R(2) * q) * to_r(src[j * plane + own]);
+        const R q2 = mul_(R(2), q);
+        d[j] = fma_(sub_(q2, R(1)) / q2, to_r(src[j * plane + own]), fi / q2);
       }
       if (j <= 4) {
         R ne, b1, b2, b3;
@@ -737,7 +693,7 @@ __device__ __forceinline__ void fixup(const DevGeom& g, const Co<R>& c, const S*
           }
           Tm = midpoint_temperature_q(q, Tw, T1, T2, have2, T3, have3, dirichlet);
         }
-        h[j] = -to_r(src[(9 + i) * plane + own]) + c.cT2 * (Tm - c.T0);  // Eq. 26
+        h[j] = fma_(c.cT2, sub_(Tm, c.T0), -to_r(src[(9 + i) * plane + own]));  // Eq. 26
       }
     } else if (outx || outy) {  // periodic seam
       if (outx) sx = sx < 0 ? sx + g.nx : sx - g.nx;
@@ -843,7 +799,7 @@ __device__ __forceinline__ void step_tile(const DevGeom& g, const Co<typename Tr
     for (int q = 0; q < 9; ++q) d[q] = v[q][k];
 #pragma unroll
     for (int q = 0; q < 5; ++q) h[q] = v[9 + q][k];
-    collide<R, VH, kHostK<S>>(c, d, h, qv[k]);
+    collide<R, VH>(c, d, h, qv[k]);
 #pragma unroll
     for (int q = 0; q < 9; ++q) v[q][k] = d[q];
 #pragma unroll
@@ -945,7 +901,7 @@ __device__ __forceinline__ void step_node(const DevGeom& g, const Co<typename Tr
   fixup<S, MASK>(g, c, src, x, y, fl, d, h);
   R qv;
   const bool vh = c.vhc != R(0);
-  collide_any<R, kHostK<S>>(c, vh, d, h, qv);
+  collide_any<R>(c, vh, d, h, qv);
   if (vh) dst[14 * plane + i] = from_r<S, R>(qv);
   // global node index of the group of four (the pitch is a multiple of 4)
   const uint32_t key = sr_key(seed, i + (long long)g.yoff * g.pitch - (x & 3));
@@ -1063,7 +1019,7 @@ __global__ void init_kernel(const DevGeom g, const DevCoef cf, S* __restrict__ d
       const R t = T ? (R)T[k] : c.T0;
       equilibrium(c, r, u, w, t, d, h);
       R qv;
-      collide_any<R, kHostK<S>>(c, cf.vh != 0, d, h, qv);
+      collide_any<R>(c, cf.vh != 0, d, h, qv);
       if (cf.vh) dst[14 * g.plane + i] = from_r<S, R>(qv);
     } else {
       if (cf.vh) dst[14 * g.plane + i] = from_r<S, R>(R(0));
