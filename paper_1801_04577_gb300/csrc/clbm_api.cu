@@ -18,6 +18,7 @@
 
 #include "../../include/clbm.h"
 #include "clbm_internal.h"
+#include "clbm_walls.h"
 
 using namespace clbm;
 
@@ -57,19 +58,17 @@ struct clbm_ctx {
   // masked-lattice tables
   uint16_t* d_flags = nullptr;
   int32_t* d_slot = nullptr;
-  double* d_lk_ne = nullptr;
-  int32_t* d_lk_tbc = nullptr;
-  double* d_lk_q = nullptr;
+  void* d_lk_t = nullptr;
+  void* d_lk_f = nullptr;
   uint8_t* d_tile_fluid = nullptr;  // masked lattices: which interior warp tiles hold fluid
   int tiles_per_row = 0;
-  double* d_tbc = nullptr;
   std::vector<int32_t> h_bnodes;  // nodes the boundary kernel recomputes (pitch layout)
   int32_t* d_bnodes = nullptr;
   std::vector<uint8_t> h_solid;    // [p.ny][nx] over the stored rows (empty: no mask)
   std::vector<clbm_tbc> h_tbc;
   std::vector<clbm_link> h_links;  // links of own-row nodes, node = stored row * nx + x
   int side_tbc[4] = {-1, -1, -1, -1};
-  double side_b[4][3] = {};
+  double side_k[4][2][3] = {};  // link_heat of the box sides without / with a second node
   double side_u[4][2] = {};  // moving box sides (clbm_set_wall_velocity)
   // scratch
   double* d_fields = nullptr;  // 4 * nx * ny doubles, allocated on first use
@@ -132,16 +131,15 @@ static DevGeom make_geom(const clbm_ctx* c) {
   g.plane = c->plane;
   g.flags = c->d_flags;
   g.slot = c->d_slot;
-  g.lk_ne = c->d_lk_ne;
-  g.lk_tbc = c->d_lk_tbc;
-  g.lk_q = c->d_lk_q;
+  g.lk_t = c->d_lk_t;
+  g.lk_f = c->d_lk_f;
   g.tile_fluid = c->d_tile_fluid;
   g.tiles_per_row = c->tiles_per_row;
   g.pad_tiles = 0;
-  g.tbc = c->d_tbc;
-  std::memcpy(g.side_b, c->side_b, sizeof(g.side_b));
+  std::memcpy(g.side_k, c->side_k, sizeof(g.side_k));
   for (int sd = 0; sd < 4; ++sd)
-    for (int k = 0; k < 3; ++k) g.side_bf[sd][k] = (float)c->side_b[sd][k];
+    for (int two = 0; two < 2; ++two)
+      for (int m = 0; m < 3; ++m) g.side_kf[sd][two][m] = (float)c->side_k[sd][two][m];
   g.moving = 0;
   g.pad_moving = 0;
   for (int sd = 0; sd < 4; ++sd)
@@ -178,21 +176,17 @@ static DevCoef make_coef(const clbm_ctx* c) {
 static void free_tables(clbm_ctx* c) {
   cudaFree(c->d_flags);
   cudaFree(c->d_slot);
-  cudaFree(c->d_lk_ne);
-  cudaFree(c->d_lk_tbc);
-  cudaFree(c->d_lk_q);
+  cudaFree(c->d_lk_t);
+  cudaFree(c->d_lk_f);
   cudaFree(c->d_tile_fluid);
-  cudaFree(c->d_tbc);
   cudaFree(c->d_bnodes);
   c->d_bnodes = nullptr;
   c->d_flags = nullptr;
   c->d_slot = nullptr;
-  c->d_lk_ne = nullptr;
-  c->d_lk_tbc = nullptr;
-  c->d_lk_q = nullptr;
+  c->d_lk_t = nullptr;
+  c->d_lk_f = nullptr;
   c->d_tile_fluid = nullptr;
   c->tiles_per_row = 0;
-  c->d_tbc = nullptr;
   for (auto& kv : c->nu_lists) cudaFree(kv.second.first);
   c->nu_lists.clear();
 }
@@ -223,6 +217,16 @@ static cudaError_t upload_boundary_list(clbm_ctx* c, const std::vector<uint16_t>
   cudaError_t e = cudaMalloc(&c->d_bnodes, v.size() * sizeof(int32_t));
   if (e != cudaSuccess) return e;
   return cudaMemcpy(c->d_bnodes, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+}
+
+// A table of wall coefficients in the lattice's compute type.
+static cudaError_t upload_coefficients(const clbm_ctx* c, const std::vector<double>& v, void** out) {
+  const std::vector<float> f(v.begin(), v.end());
+  const bool wide = c->p.precision == CLBM_F64;
+  const size_t bytes = std::max<size_t>(v.size(), 1) * (wide ? sizeof(double) : sizeof(float));
+  cudaError_t e = cudaMalloc(out, bytes);
+  if (e != cudaSuccess || v.empty()) return e;
+  return cudaMemcpy(*out, wide ? (const void*)v.data() : (const void*)f.data(), bytes, cudaMemcpyHostToDevice);
 }
 
 extern "C" {
@@ -319,8 +323,6 @@ static clbm_status create_impl(const clbm_params* params, void* stream, void* bu
   c->plane = (long long)p.ny * c->pitch;
   c->buf_bytes = (size_t)planes_of(p.viscous_heating) * (size_t)c->plane * L->elem_bytes;
   c->have_walls = p.periodic_x && c->gpy;
-  for (int s = 0; s < 4; ++s)
-    for (int k = 0; k < 3; ++k) c->side_b[s][k] = 0.0;
   cudaError_t e;
   if (stream) {
     c->stream = static_cast<cudaStream_t>(stream);
@@ -465,8 +467,22 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
       kk.node = y * nx + x;
       kept.push_back(kk);
     }
+    // whether (x, y) is a stored fluid node (around the seams; rows: stored rows)
+    auto fluid_at = [&](int x, int y) {
+      if (x < 0 || x >= nx) {
+        if (!px) return false;
+        x = (x + 2 * nx) % nx;
+      }
+      if (y < c->ylo || y >= c->yhi) {
+        if (y < c->ylo ? c->ywlo : c->ywhi) return false;
+        if (!c->slab) y = (y + 2 * ny) % ny;
+        if (y < 0 || y >= ny) return false;  // beyond the ghost row (refused above where it is read)
+      }
+      return !is_solid(x, y);
+    };
     std::vector<uint16_t> flags;
     std::vector<int32_t> slot_pitch;
+    std::vector<double> lk_t(lk_tbc.size() * 4, 0.0), lk_f(lk_tbc.size() * 6, 0.0);
     if (masked) {
       flags.assign((size_t)ny * c->pitch, 0);
       slot_pitch.assign((size_t)ny * c->pitch, -1);
@@ -492,6 +508,7 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
               else if (!c->slab)
                 sy = (sy + ny) % ny;  // periodic seam (slabs read their ghost row)
             }
+            const bool box = wall;
             if (!wall && is_solid(sx, sy)) {
               wall = true;
               // a D2Q5 link into a solid needs a listed condition: link dir i = opp(j)
@@ -505,6 +522,7 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
             }
             if (wall) f |= (uint16_t)(1u << (j - 1));
             else ++fluid_nb;
+            if (box && j <= 4 && !fluid_at(x + kEX[j], y + kEY[j])) f |= (uint16_t)(1u << (kFlagSecond + j - 1));
           }
           if (fluid_nb == 0 && n > 1)
             return fail(c, CLBM_EINVAL, "isolated fluid node " + std::to_string((long long)grow(y) * nx + x));
@@ -512,6 +530,22 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
           if (s >= 0) {
             f |= kFlagLinks;
             slot_pitch[ip] = s;
+            for (int i = 1; i < 9; ++i) {
+              const int dx = -kEX[i], dy = -kEY[i];
+              const bool have2 = fluid_at(x + dx, y + dy);
+              const double q = lk_q[8 * s + i - 1];
+              double kf[3];
+              link_bounce(q, have2, kf);
+              for (int m = 0; m < 3; ++m) lk_f[(size_t)24 * s + 3 * (i - 1) + m] = kf[m];
+              if (kf[0] != 1.0) f |= kFlagOffMid;
+              if (i <= 4 && lk_tbc[4 * s + i - 1] >= 0) {
+                const clbm_tbc& b = tbc[lk_tbc[4 * s + i - 1]];
+                double kt[4];
+                link_heat(b.b1, b.b2, b.b3, lk_ne[4 * s + i - 1], q, have2, fluid_at(x + 2 * dx, y + 2 * dy),
+                          c->p.T0, 0.5 * c->p.Q, c->p.cT2, kt);
+                for (int m = 0; m < 4; ++m) lk_t[(size_t)16 * s + 4 * (i - 1) + m] = kt[m];
+              }
+            }
           }
           flags[ip] = f;
         }
@@ -526,16 +560,8 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
       CLBM_CUDA(c, cudaMalloc(&c->d_slot, np * sizeof(int32_t)));
       CLBM_CUDA(c, cudaMemcpy(c->d_flags, flags.data(), np * sizeof(uint16_t), cudaMemcpyHostToDevice));
       CLBM_CUDA(c, cudaMemcpy(c->d_slot, slot_pitch.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice));
-      const size_t ns = std::max<size_t>(lk_tbc.size(), 4);
-      lk_ne.resize(ns, 0.0);
-      lk_tbc.resize(ns, -1);
-      lk_q.resize(2 * ns, 0.5);
-      CLBM_CUDA(c, cudaMalloc(&c->d_lk_ne, ns * sizeof(double)));
-      CLBM_CUDA(c, cudaMalloc(&c->d_lk_tbc, ns * sizeof(int32_t)));
-      CLBM_CUDA(c, cudaMalloc(&c->d_lk_q, 2 * ns * sizeof(double)));
-      CLBM_CUDA(c, cudaMemcpy(c->d_lk_ne, lk_ne.data(), ns * sizeof(double), cudaMemcpyHostToDevice));
-      CLBM_CUDA(c, cudaMemcpy(c->d_lk_tbc, lk_tbc.data(), ns * sizeof(int32_t), cudaMemcpyHostToDevice));
-      CLBM_CUDA(c, cudaMemcpy(c->d_lk_q, lk_q.data(), 2 * ns * sizeof(double), cudaMemcpyHostToDevice));
+      CLBM_CUDA(c, upload_coefficients(c, lk_t, &c->d_lk_t));
+      CLBM_CUDA(c, upload_coefficients(c, lk_f, &c->d_lk_f));
       {  // classes of the interior kernel's warp tiles (32 vec nodes of a row): 0 = no
          // fluid node (skipped), 1 = fluid nodes only, none flagged, 2 = holds a
          // flagged node (solid, or fluid next to a wall) whose store it leaves out
@@ -556,21 +582,17 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
         c->tiles_per_row = tpr;
       }
     }
-    {
-      std::vector<double> t3((size_t)std::max(n_tbc, 1) * 3, 0.0);
-      for (int k = 0; k < n_tbc; ++k) {
-        t3[3 * k] = tbc[k].b1;
-        t3[3 * k + 1] = tbc[k].b2;
-        t3[3 * k + 2] = tbc[k].b3;
-      }
-      CLBM_CUDA(c, cudaMalloc(&c->d_tbc, t3.size() * sizeof(double)));
-      CLBM_CUDA(c, cudaMemcpy(c->d_tbc, t3.data(), t3.size() * sizeof(double), cudaMemcpyHostToDevice));
-    }
     CLBM_CUDA(c, upload_boundary_list(c, flags));
     for (int s = 0; s < 4; ++s) {
       c->side_tbc[s] = sides[s];
-      for (int k = 0; k < 3; ++k)
-        c->side_b[s][k] = sides[s] >= 0 ? (&tbc[sides[s]].b1)[k] : 0.0;
+      for (int two = 0; two < 2; ++two) {
+        double k[4] = {0, 0, 0, 0};
+        if (sides[s] >= 0) {
+          const clbm_tbc& b = tbc[sides[s]];
+          link_heat(b.b1, b.b2, b.b3, 1.0, 0.5, two != 0, false, c->p.T0, 0.5 * c->p.Q, c->p.cT2, k);
+        }
+        std::copy(k, k + 3, c->side_k[s][two]);
+      }
     }
     c->h_solid = std::move(sol);
     c->h_tbc.assign(tbc, tbc + n_tbc);

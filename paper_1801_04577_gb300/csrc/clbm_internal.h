@@ -14,8 +14,12 @@ namespace clbm {
 //               (a solid node or a non-periodic box side)
 //   bit 8     : the node itself is solid
 //   bit 9     : the node has listed (curved / obstacle) thermal wall links
+//   bits 10..13 : box wall in D2Q5 direction j = bit - 9, and no fluid node behind this one (x + e_j)
+//   bit 14    : a listed link's wall is off the link midpoint
 constexpr uint16_t kFlagSolid = 1u << 8;
 constexpr uint16_t kFlagLinks = 1u << 9;
+constexpr int kFlagSecond = 10;
+constexpr uint16_t kFlagOffMid = 1u << 14;
 
 // Planes per buffer: 14 distributions, plus the viscous source Q_v when enabled.
 inline int planes_of(int vh) { return vh ? 15 : 14; }
@@ -34,15 +38,13 @@ struct DevGeom {
   long long plane;             // elements per plane = ny * pitch
   const uint16_t* flags;       // [ny][pitch] or nullptr (box walls only)
   const int32_t* slot;         // [ny][pitch] link slot, -1 = none (masked lattices)
-  const double* lk_ne;         // [nslots][4] n.e_i per link direction i = 1..4
-  const int32_t* lk_tbc;       // [nslots][4] condition index, -1 = no link
-  const double* lk_q;          // [nslots][8] wall fraction q per link direction i = 1..8 (0.5 = half-way)
-  const double* tbc;           // [ntbc][3] (b1, b2, b3)
+  const void* lk_t;            // [nslots][4][4] link_heat coefficients per link direction i = 1..4, and
+  const void* lk_f;            // [nslots][8][3] link_bounce coefficients, i = 1..8; both in the compute type
   const uint8_t* tile_fluid;   // [ny][tiles_per_row] class of each warp tile (32 V nodes of a row): 0 = no
                                // fluid node, 1 = no flagged node, 2 = holds flagged nodes; nullptr = box lattice
   int tiles_per_row, pad_tiles;
-  double side_b[4][3];         // conditions of the box sides x0, x1, y0, y1
-  float side_bf[4][3];         // the same rounded to FP32 (for FP32 arithmetic)
+  double side_k[4][2][3];      // link_heat of the box sides x0, x1, y0, y1 without / with a second node
+  float side_kf[4][2][3];      // the same rounded to FP32 (for FP32 arithmetic)
   // moving box sides (not in the paper): wall velocity of each side, and the
   // same rounded to FP32; moving = 0 when every side is at rest
   double side_u[4][2];

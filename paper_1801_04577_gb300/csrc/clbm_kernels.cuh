@@ -41,6 +41,7 @@
 #include <type_traits>
 
 #include "clbm_internal.h"
+#include "clbm_walls.h"
 
 namespace clbm {
 
@@ -224,28 +225,6 @@ __device__ __forceinline__ void sr_words(uint32_t key, int q, uint32_t& r0, uint
 }
 
 // ---------------------------------------------------------------------------
-// Arithmetic with the rounding points written out.  The same node update is
-// compiled into several kernels (plane tiles, boundary nodes, batches, lattices
-// resident in shared memory); left to itself the compiler contracts a * b + c
-// differently in each, and a lattice would then depend on the kernel that
-// advanced it.  With every multiply-add explicit they agree bit for bit.
-// ---------------------------------------------------------------------------
-#ifdef __CUDA_ARCH__
-__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
-#else
-inline float fma_(float a, float b, float c) { return std::fma(a, b, c); }
-inline double fma_(double a, double b, double c) { return std::fma(a, b, c); }
-template <typename R> inline R mul_(R a, R b) { return a * b; }
-template <typename R> inline R add_(R a, R b) { return a + b; }
-template <typename R> inline R sub_(R a, R b) { return a - b; }
-#endif
 // 1 / rho.  FP32: to within 2 ulp (hardware approximation), which the FP32
 // parity bound leaves ample room for; FP64: the exact quotient.
 __host__ __device__ __forceinline__ double rcp_(double v) { return 1.0 / v; }
@@ -494,215 +473,157 @@ __host__ __device__ __forceinline__ void equilibrium(const Co<R>& c, R rho, R ux
   h[4] = R(0.5) * (q02 - q01);
 }
 
-// ---------------------------------------------------------------------------
-// Wall temperature (Eq. 28), one-sided when the second node is missing
-// ---------------------------------------------------------------------------
-template <typename R>
-__host__ __device__ __forceinline__ R wall_temperature(R b1, R b2, R b3, R ne, R T1, R T2, bool have2) {
-  const R n3 = mul_(ne, b3);
-  if (have2)
-    return fma_(mul_(R(9), b1), T1, fma_(R(3), n3, -mul_(b1, T2))) /
-           fma_(R(8), b1, mul_(R(3), mul_(ne, b2)));
-  return fma_(mul_(R(2), b1), T1, n3) / fma_(R(2), b1, mul_(ne, b2));
-}
-
-// Walls at the fraction q of a link (no counterpart in the paper; q = 1/2 is
-// its half-way wall).  s = distance from the wall along the link into the
-// fluid; the wall profile is the quadratic through (0, T_w), (q, T1),
-// (1 + q, T2), i.e. q(1+q) dT/ds(0) = -(1+2q) T_w + (1+q)^2 T1 - q^2 T2, and
-// dT/dn = -dT/ds(0) / (n.e).  T_w solves b1 dT/dn + b2 T_w = b3 (the line
-// through (0, T_w), (q, T1) when T2 is missing).
-template <typename R>
-__host__ __device__ __forceinline__ R wall_temperature_q(R b1, R b2, R b3, R ne, R q, R T1, R T2, bool have2) {
-  const R qn = mul_(q, ne);
-  if (have2) {
-    const R p = add_(R(1), q), qqn = mul_(qn, p);
-    const R e = fma_(mul_(p, p), T1, -mul_(mul_(q, q), T2));
-    return fma_(b1, e, mul_(b3, qqn)) / fma_(b1, fma_(R(2), q, R(1)), mul_(b2, qqn));
-  }
-  return fma_(b1, T1, mul_(b3, qn)) / fma_(b2, qn, b1);
-}
-
-// dT/dn at such a wall from the same profile.
-template <typename R>
-__host__ __device__ __forceinline__ R wall_gradient_q(R ne, R q, R Tw, R T1, R T2, bool have2) {
-  if (have2) {
-    const R p = R(1) + q;
-    return ((R(1) + R(2) * q) * Tw - p * p * T1 + q * q * T2) / (q * p * ne);
-  }
-  return (Tw - T1) / (q * ne);
-}
-
-// The profile's value at the link midpoint s = q - 1/2, which Eq. 26 then
-// imposes there.  q >= 1/2 or a wall with a flux term (b1 > 0): interpolation
-// weights of the quadratic through the wall and the nodes at q and 1 + q.
-// q < 1/2 at a Dirichlet wall: the quadratic through the wall and the nodes
-// at 1 + q and 2 + q instead (bounded weights as q -> 0, none on the node's
-// own T1, which would feed back into the node).  Both exact for quadratic
-// profiles; lines through the available points in thin fluid layers.
-template <typename R>
-__host__ __device__ __forceinline__ R midpoint_temperature_q(R q, R Tw, R T1, R T2, bool have2, R T3,
-                                                             bool have3, bool dirichlet) {
-  const R m = fma_(R(2), q, R(-1));  // 2 (q - 1/2)
-  const R p1 = add_(R(1), q);
-  if (q >= R(0.5) || !dirichlet) {
-    if (!have2) return fma_(sub_(T1, Tw), m / mul_(R(2), q), Tw);
-    return fma_(R(3) / mul_(R(4), mul_(q, p1)), Tw,
-                fma_(mul_(R(3), m) / mul_(R(4), q), T1, mul_(-(m / mul_(R(4), p1)), T2)));
-  }
-  if (have2 && have3) {
-    const R p2 = add_(R(2), q);
-    return fma_(R(15) / mul_(R(4), mul_(p1, p2)), Tw,
-                fma_(mul_(R(5), m) / mul_(R(4), p1), T2, mul_(-(mul_(R(3), m) / mul_(R(4), p2)), T3)));
-  }
-  if (have2) return fma_(sub_(T2, Tw), m / mul_(R(2), p1), Tw);
-  return Tw;
-}
-
+// The stored state as the boundary nodes read it.
+template <typename S>
+struct PlaneSrc {
+  using Idx = long long;
+  const S* __restrict__ p;
+  long long plane;
+  __device__ __forceinline__ S at(int q, long long i) const { return p[q * plane + i]; }
+};
 // T at a node from its post-collision thermal deviations: T = T0 + sum h* - Q/2,
 // Q including the node's stored viscous source when that is enabled.
-template <typename S, typename R>
-__device__ __forceinline__ R node_T(const S* __restrict__ src, long long plane, long long idx,
-                                    const Co<R>& c) {
-  R s = to_r(src[9 * plane + idx]);
+template <class Src, typename R, typename Idx>
+__device__ __forceinline__ R node_T(const Src& src, Idx idx, const Co<R>& c) {
+  R s = to_r(src.at(9, idx));
 #pragma unroll
-  for (int q = 10; q < 14; ++q) s += to_r(src[q * plane + idx]);
+  for (int q = 10; q < 14; ++q) s += to_r(src.at(q, idx));
   R t = c.T0 + s - c.hQ;
-  if (c.vhc != R(0)) t = fma_(R(-0.5), to_r(src[14 * plane + idx]), t);
+  if (c.vhc != R(0)) t = fma_(R(-0.5), to_r(src.at(14, idx)), t);
   return t;
 }
 
-// Fix-up of one node that touches a wall, a periodic seam or a solid.
-template <typename S, bool MASK, typename R>
-__device__ __forceinline__ void fixup(const DevGeom& g, const Co<R>& c, const S* __restrict__ src,
-                                      int x, int y, uint16_t fl, R (&d)[9], R (&h)[5]) {
-  const long long plane = g.plane;
-  const long long own = (long long)y * g.pitch + x;
-  const R T1 = node_T(src, plane, own, c);
+// T - T0 + Q/2 at a node (the wall rules' constants absorb T0 - Q/2).
+template <class Src, typename R, typename Idx>
+__device__ __forceinline__ R node_heat(const Src& src, Idx idx, const Co<R>& c) {
+  R s = to_r(src.at(9, idx));
+#pragma unroll
+  for (int q = 10; q < 14; ++q) s = add_(s, to_r(src.at(q, idx)));
+  if (c.vhc != R(0)) s = fma_(R(-0.5), to_r(src.at(14, idx)), s);
+  return s;
+}
+
+// A pair of constants for the compute type (FP32 arithmetic has its own copies).
+template <typename R>
+__device__ __forceinline__ const R* side_wall(const DevGeom& g, int sd, bool have2) {
+  if constexpr (std::is_same<R, float>::value)
+    return g.side_kf[sd][have2 ? 1 : 0];
+  else
+    return g.side_k[sd][have2 ? 1 : 0];
+}
+
+// New state of node (x, y) next to a wall, a solid or a periodic seam: pull,
+// bounce-back, Eq. 26-28, collision.  src: the stored state, indexed
+// y * g.pitch + x; fl, slot: its flags and its entry of the link tables
+// (masked lattices).
+//
+// What bounds this is the length of its dependent chain, not its bytes: a
+// block of boundary nodes that took 3 us held up every small step.  So a
+// population that comes from a wall is the opposite one of the node itself,
+// chosen by its address (no branch), and the wall temperature, linear in the
+// temperatures along the link, is three or four host-made coefficients (no
+// division, no branch on the kind of wall).
+template <class Src, bool MASK, typename R>
+__device__ __forceinline__ void node_update(const DevGeom& g, const Co<R>& c, const Src& src, int x, int y,
+                                            uint32_t fl, int slot, R (&d)[9], R (&h)[5], R& qv) {
+  using Idx = typename Src::Idx;
+  const Idx own = (Idx)y * g.pitch + x;
+  const bool x_lo = x == 0, x_hi = x == g.nx - 1;
+  const bool y_lo = y == g.ylo, y_hi = y == g.yhi - 1;
+  d[0] = to_r(src.at(0, own));
+  h[0] = to_r(src.at(9, own));
+  uint32_t wall = MASK ? (fl & 0xFFu) : 0u;  // bit j - 1: population j comes from a wall ...
+  uint32_t box = 0;                          // ... of the box
 #pragma unroll
   for (int j = 1; j < 9; ++j) {
     const int ex = ex_of(j), ey = ey_of(j);
-    int sx = x - ex, sy = y - ey;
-    const bool outx = sx < 0 || sx >= g.nx;
-    const bool ylow = sy < g.ylo, yhigh = sy >= g.yhi;
-    // beyond the own rows: a box wall, the periodic seam, or a ghost row (read as is)
-    const bool outy = (ylow || yhigh) && g.py;
-    const bool boxwall = (outx && !g.px) || (ylow && g.ywlo) || (yhigh && g.ywhi);
-    bool wall = boxwall;
-    if (MASK) wall = wall || ((fl >> (j - 1)) & 1u);
-    if (wall) {
-      const int i = opp_of(j);
-      // listed link of a masked lattice: its slot and wall fraction (1/2 otherwise)
-      int slot = -1;
-      R q = R(0.5);
-      if (MASK && !boxwall && (fl & kFlagLinks)) {
-        slot = g.slot[own];
-        q = (R)g.lk_q[8 * slot + (i - 1)];
-      }
-      // second node x_f - e_i = x + e_j, away from the wall
-      int x2 = x + ex, y2 = y + ey;
-      bool have2 = true;
-      if (x2 < 0 || x2 >= g.nx) {
-        if (g.px)
-          x2 = x2 < 0 ? x2 + g.nx : x2 - g.nx;
+    const bool outx = ex > 0 ? x_lo : (ex < 0 ? x_hi : false);
+    const bool outl = ey > 0 && y_lo, outh = ey < 0 && y_hi;
+    if ((outx && !g.px) || (outl && g.ywlo) || (outh && g.ywhi)) box |= 1u << (j - 1);
+  }
+  wall |= box;
+#pragma unroll
+  for (int j = 1; j < 9; ++j) {
+    const int ex = ex_of(j), ey = ey_of(j);
+    int sx = x - ex, sy = y - ey;  // within the storage, around the seam, or unused (a wall)
+    if (ex != 0 && g.px) sx = sx < 0 ? g.nx - 1 : (sx >= g.nx ? 0 : sx);
+    if (ey != 0 && g.py) sy = sy < 0 ? g.ny - 1 : (sy >= g.ny ? 0 : sy);
+    const bool w = (wall >> (j - 1)) & 1u;
+    const Idx from = w ? own : (Idx)sy * g.pitch + sx;
+    d[j] = to_r(src.at(w ? opp_of(j) : j, from));
+    if (j < 5) h[j] = to_r(src.at(w ? 9 + opp_of(j) : 9 + j, from));
+  }
+  // the node one further along the link, x_f - e_i = x + e_j
+  auto ahead = [&](int ex, int ey, int n) -> Idx {
+    int x2 = x + n * ex, y2 = y + n * ey;
+    if (g.px) x2 = x2 < 0 ? x2 + g.nx : (x2 >= g.nx ? x2 - g.nx : x2);
+    if (g.py) y2 = y2 < 0 ? y2 + g.ny : (y2 >= g.ny ? y2 - g.ny : y2);
+    return (Idx)y2 * g.pitch + x2;
+  };
+  if (wall & 0xFu) {
+    const R s1 = node_heat(src, own, c);
+#pragma unroll
+    for (int j = 1; j < 5; ++j) {
+      if (!((wall >> (j - 1)) & 1u)) continue;
+      const int ex = ex_of(j), ey = ey_of(j);
+      R ka, kb, kc, kd = R(0);
+      if ((box >> (j - 1)) & 1u) {
+        bool have2;
+        if (MASK)
+          have2 = !((fl >> (kFlagSecond + j - 1)) & 1u);
         else
-          have2 = false;
+          have2 = ex != 0 ? g.nx > 1 : !(ey > 0 ? (y_hi && g.ywhi) : (y_lo && g.ywlo));
+        const R* k = side_wall<R>(g, side_of(j), have2);
+        ka = k[0];
+        kb = k[1];
+        kc = k[2];
+      } else {
+        const R* k = static_cast<const R*>(g.lk_t) + 16 * slot + 4 * (opp_of(j) - 1);
+        ka = __ldg(k);
+        kb = __ldg(k + 1);
+        kc = __ldg(k + 2);
+        kd = __ldg(k + 3);
       }
-      if (y2 < g.ylo || y2 >= g.yhi) {
-        if (g.py)
-          y2 = y2 < 0 ? y2 + g.ny : y2 - g.ny;
-        else if (y2 < g.ylo ? g.ywlo : g.ywhi)
-          have2 = false;  // beyond a box wall (else: a ghost row)
-      }
-      const long long i2 = (long long)y2 * g.pitch + x2;
-      if (MASK && have2) have2 = (g.flags[i2] & kFlagSolid) == 0;
-      const R fi = to_r(src[i * plane + own]);
-      if (q == R(0.5) || (q < R(0.5) && !have2)) {
-        d[j] = fi;  // half-way bounce-back
-        if (boxwall && g.moving) {
-          // a moving box side (not in the paper; Ladd's bounce-back): the
-          // reflected population gains -6 w_i rho0 (e_i . u_w), e_i = -e_j
-          const int sd = (outx && !g.px) ? (sx < 0 ? 0 : 1) : (ylow ? 2 : 3);
-          R uwx, uwy;
-          if constexpr (std::is_same<R, float>::value) {
-            uwx = g.side_uf[sd][0];
-            uwy = g.side_uf[sd][1];
-          } else {
-            uwx = (R)g.side_u[sd][0];
-            uwy = (R)g.side_u[sd][1];
-          }
-          const R w6 = j <= 4 ? R(6.0 / 9.0) : R(6.0 / 36.0);
-          d[j] = fma_(mul_(w6, c.rho0), add_(mul_(R(ex), uwx), mul_(R(ey), uwy)), d[j]);
-        }
-      } else if (q < R(0.5)) {  // f_i* interpolated to the point 1 - 2q behind x_f
-        const R q2 = mul_(R(2), q);
-        d[j] = fma_(q2, fi, mul_(sub_(R(1), q2), to_r(src[i * plane + i2])));
-      } else {  // the reflected value, 2q - 1 beyond x_f, interpolated with f_j* at x_f
-        const R q2 = mul_(R(2), q);
-        d[j] = fma_(sub_(q2, R(1)) / q2, to_r(src[j * plane + own]), fi / q2);
-      }
-      if (j <= 4) {
-        R ne, b1, b2, b3;
-        if (boxwall) {
-          const int sd = side_of(j);
-          ne = R(1);
-          if constexpr (std::is_same<R, float>::value) {
-            b1 = g.side_bf[sd][0];
-            b2 = g.side_bf[sd][1];
-            b3 = g.side_bf[sd][2];
-          } else {
-            b1 = (R)g.side_b[sd][0];
-            b2 = (R)g.side_b[sd][1];
-            b3 = (R)g.side_b[sd][2];
-          }
-        } else {
-          const int s = slot >= 0 ? slot : g.slot[own];
-          const int t = g.lk_tbc[4 * s + (i - 1)];
-          ne = (R)g.lk_ne[4 * s + (i - 1)];
-          b1 = (R)g.tbc[3 * t + 0];
-          b2 = (R)g.tbc[3 * t + 1];
-          b3 = (R)g.tbc[3 * t + 2];
-        }
-        const R T2 = have2 ? node_T(src, plane, i2, c) : R(0);
-        R Tm;
-        if (q == R(0.5)) {
-          Tm = wall_temperature(b1, b2, b3, ne, T1, T2, have2);  // Eq. 28
-        } else {
-          const R Tw = wall_temperature_q(b1, b2, b3, ne, q, T1, T2, have2);
-          const bool dirichlet = b1 == R(0);
-          bool have3 = false;
-          R T3 = R(0);
-          if (q < R(0.5) && dirichlet && have2) {  // third node x + 2 e_j
-            int x3 = x2 + ex, y3 = y2 + ey;
-            have3 = true;
-            if (x3 < 0 || x3 >= g.nx) {
-              if (g.px)
-                x3 = x3 < 0 ? x3 + g.nx : x3 - g.nx;
-              else
-                have3 = false;
-            }
-            if (y3 < g.ylo || y3 >= g.yhi) {
-              if (g.py)
-                y3 = y3 < 0 ? y3 + g.ny : y3 - g.ny;
-              else if ((y3 < g.ylo ? g.ywlo : g.ywhi) || y3 < 0 || y3 >= g.ny)
-                have3 = false;  // beyond a box wall (slabs reject links whose third node is not stored)
-            }
-            const long long i3 = (long long)y3 * g.pitch + x3;
-            if (MASK && have3) have3 = (g.flags[i3] & kFlagSolid) == 0;
-            if (have3) T3 = node_T(src, plane, i3, c);
-          }
-          Tm = midpoint_temperature_q(q, Tw, T1, T2, have2, T3, have3, dirichlet);
-        }
-        h[j] = fma_(c.cT2, sub_(Tm, c.T0), -to_r(src[(9 + i) * plane + own]));  // Eq. 26
-      }
-    } else if (outx || outy) {  // periodic seam
-      if (outx) sx = sx < 0 ? sx + g.nx : sx - g.nx;
-      if (outy) sy = sy < 0 ? sy + g.ny : sy - g.ny;
-      const long long s = (long long)sy * g.pitch + sx;
-      d[j] = to_r(src[j * plane + s]);
-      if (j <= 4) h[j] = to_r(src[(9 + j) * plane + s]);
+      R e = kc;
+      if (kd != R(0)) e = fma_(kd, node_heat(src, ahead(ex, ey, 2), c), e);
+      if (kb != R(0)) e = fma_(kb, node_heat(src, ahead(ex, ey, 1), c), e);
+      h[j] = sub_(fma_(ka, s1, e), h[j]);  // Eq. 26
     }
   }
+  if (MASK && (fl & kFlagOffMid)) {  // walls off the link midpoint: interpolated bounce-back
+#pragma unroll
+    for (int j = 1; j < 9; ++j) {
+      if (!(((wall & ~box) >> (j - 1)) & 1u)) continue;
+      const int i = opp_of(j);
+      const R* k = static_cast<const R*>(g.lk_f) + 24 * slot + 3 * (i - 1);
+      const R k0 = __ldg(k), k1 = __ldg(k + 1), k2 = __ldg(k + 2);
+      R v = mul_(k2, to_r(src.at(j, own)));
+      if (k1 != R(0)) v = fma_(k1, to_r(src.at(i, ahead(ex_of(j), ey_of(j), 1))), v);
+      d[j] = fma_(k0, d[j], v);
+    }
+  }
+  if (g.moving && box) {
+    // moving box sides (not in the paper; Ladd's bounce-back): the reflected
+    // population gains -6 w_i rho0 (e_i . u_w), e_i = -e_j
+#pragma unroll
+    for (int j = 1; j < 9; ++j) {
+      if (!((box >> (j - 1)) & 1u)) continue;
+      const int ex = ex_of(j), ey = ey_of(j);
+      const bool outx = ex > 0 ? x_lo : (ex < 0 ? x_hi : false);
+      const int sd = (outx && !g.px) ? (ex > 0 ? 0 : 1) : (ey > 0 ? 2 : 3);
+      R uwx, uwy;
+      if constexpr (std::is_same<R, float>::value) {
+        uwx = g.side_uf[sd][0];
+        uwy = g.side_uf[sd][1];
+      } else {
+        uwx = (R)g.side_u[sd][0];
+        uwy = (R)g.side_u[sd][1];
+      }
+      const R w6 = j <= 4 ? R(6.0 / 9.0) : R(6.0 / 36.0);
+      d[j] = fma_(mul_(w6, c.rho0), add_(mul_(R(ex), uwx), mul_(R(ey), uwy)), d[j]);
+    }
+  }
+  collide_any<R>(c, c.vhc != R(0), d, h, qv);
 }
 
 // ---------------------------------------------------------------------------
@@ -875,8 +796,7 @@ __device__ __forceinline__ void step_tile(const DevGeom& g, const Co<typename Tr
   for (int q = 0; q < 14; ++q) stv<S, V>(out + q * plane, v[q]);
 }
 
-// Boundary update of node index i (pitch layout): pull with clamped indices,
-// then the fix-up applies bounce-back, Eq. 26-28 and periodic wrapping.
+// Boundary update of node index i (pitch layout).
 template <typename S, bool MASK>
 __device__ __forceinline__ void step_node(const DevGeom& g, const Co<typename Traits<S>::R>& c,
                                           const S* __restrict__ src, S* __restrict__ dst,
@@ -884,25 +804,11 @@ __device__ __forceinline__ void step_node(const DevGeom& g, const Co<typename Tr
   using R = typename Traits<S>::R;
   const int y = (int)(i / g.pitch), x = (int)(i - (long long)y * g.pitch);
   const long long plane = g.plane;
-  R d[9], h[5];
-#pragma unroll
-  for (int q = 0; q < 14; ++q) {
-    const int dir = q < 9 ? q : q - 9;
-    int sx = x - ex_of(dir), sy = y - ey_of(dir);
-    sx = sx < 0 ? 0 : (sx >= g.nx ? g.nx - 1 : sx);
-    sy = sy < 0 ? 0 : (sy >= g.ny ? g.ny - 1 : sy);
-    const R val = to_r(src[q * plane + (long long)sy * g.pitch + sx]);
-    if (q < 9)
-      d[q] = val;
-    else
-      h[q - 9] = val;
-  }
-  const uint16_t fl = MASK ? g.flags[i] : (uint16_t)0;
-  fixup<S, MASK>(g, c, src, x, y, fl, d, h);
-  R qv;
-  const bool vh = c.vhc != R(0);
-  collide_any<R>(c, vh, d, h, qv);
-  if (vh) dst[14 * plane + i] = from_r<S, R>(qv);
+  R d[9], h[5], qv;
+  const uint32_t fl = MASK ? (uint32_t)g.flags[i] : 0u;
+  const int slot = MASK && (fl & kFlagLinks) ? g.slot[i] : 0;
+  node_update<PlaneSrc<S>, MASK>(g, c, PlaneSrc<S>{src, plane}, x, y, fl, slot, d, h, qv);
+  if (c.vhc != R(0)) dst[14 * plane + i] = from_r<S, R>(qv);
   // global node index of the group of four (the pitch is a multiple of 4)
   const uint32_t key = sr_key(seed, i + (long long)g.yoff * g.pitch - (x & 3));
 #pragma unroll
@@ -1321,11 +1227,12 @@ __global__ void __launch_bounds__(kRedThreads)
                    const NuLink* __restrict__ links, int nlinks, double* __restrict__ partials) {
   double acc[2] = {0, 0};
   const Co<double> cd = make_co<double>(c);
+  const PlaneSrc<S> src{b, g.plane};
   for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlinks; l += gridDim.x * blockDim.x) {
     const NuLink L = links[l];
-    const double T1 = node_T(b, g.plane, L.own, cd);
+    const double T1 = node_T(src, L.own, cd);
     const bool have2 = L.second >= 0;
-    const double T2 = have2 ? node_T(b, g.plane, L.second, cd) : 0.0;
+    const double T2 = have2 ? node_T(src, L.second, cd) : 0.0;
     double grad;
     if (L.q == 0.5) {
       const double Tw = wall_temperature(L.b1, L.b2, L.b3, L.ne, T1, T2, have2);
