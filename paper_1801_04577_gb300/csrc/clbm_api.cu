@@ -77,6 +77,7 @@ struct clbm_ctx {
   // captured step graphs of 2, 4, ..., kGraphSteps steps, keyed by (current buffer, step parity)
   long long* d_t = nullptr;
   cudaGraphExec_t step_graph[4][kGraphLevels] = {};
+  ResPlan res;  // steps in shared memory (planned on first use for the current walls)
   std::string err;
 };
 
@@ -174,6 +175,7 @@ static DevCoef make_coef(const clbm_ctx* c) {
 }
 
 static void free_tables(clbm_ctx* c) {
+  c->res = ResPlan{};
   cudaFree(c->d_flags);
   cudaFree(c->d_slot);
   cudaFree(c->d_lk_t);
@@ -702,9 +704,48 @@ static clbm_status capture_steps(clbm_ctx* c, int cur, int par, int len, cudaGra
   return CLBM_OK;
 }
 
+// Steps of one resident launch (about 4 ms).
+constexpr int kResidentSteps = 4096;
+
+// Plan the resident steps of a single lattice: the most blocks a cluster can
+// have, so that each has the fewest nodes (a step's time is a block's latency).
+// FP64 stays with the plane kernels beyond 128 nodes a block: its arithmetic
+// needs the FP64 pipes of every multiprocessor.
+static bool resident_ready(clbm_ctx* c) {
+  if (c->res.cl < 0) {
+    ResPlan best;
+    best.cl = 0;
+    for (int cl = kMaxCluster; cl >= 1 && best.cl == 0; cl /= 2) {
+      if (c->p.precision == CLBM_F64 && (long long)c->p.nx * c->p.ny > 128LL * cl) break;
+      ResPlan p;
+      if (resident_plan(c, cl, kMaxResidentSmem, kMaxResidentThreads, &p, nullptr) &&
+          c->L->resident_clusters(cl, p.threads, p.smem, c->p.viscous_heating) > 0)
+        best = p;
+    }
+    c->res = best;
+  }
+  return c->res.cl > 0;
+}
+
 clbm_status clbm_step(clbm_ctx* c, int64_t nsteps) {
   if (!c || nsteps < 0) return fail(c, CLBM_EINVAL, "bad step count");
   if (!c->have_walls) return fail(c, CLBM_EINVAL, "non-periodic lattice: call clbm_set_boundaries first");
+  if (nsteps >= 2 && resident_ready(c)) {
+    ResArgs a{};
+    resident_plan(c, c->res.cl, kMaxResidentSmem, kMaxResidentThreads, &c->res, &a.one);
+    a.cl = c->res.cl;
+    a.stochastic = c->p.rounding;
+    while (nsteps > 0) {
+      a.steps = (int)std::min<int64_t>(nsteps, kResidentSteps);
+      a.t0 = c->t;
+      a.cur = c->cur;
+      CLBM_CUDA(c, c->L->resident_step(a, 1, c->res.threads, c->res.smem, c->p.viscous_heating, c->stream));
+      c->t += a.steps;
+      c->cur ^= a.steps & 1;
+      nsteps -= a.steps;
+    }
+    return CLBM_OK;
+  }
   // Runs of two or more steps replay captured graphs of 32, 16, ..., 2 steps
   // (the binary digits of nsteps; fewer launch gaps), with the step count on
   // the device.  Every graph length is even, so the buffer/parity key stays the
@@ -1161,6 +1202,42 @@ ViewInfo describe_view(const clbm_ctx* c) {
   v.bnodes_host = c->h_bnodes.data();
   v.nb = (int)c->h_bnodes.size();
   return v;
+}
+
+bool resident_plan(const clbm_ctx* c, int cl, size_t max_smem, int max_threads, ResPlan* plan, ResLat* lat) {
+  const int nx = c->p.nx, ny = c->p.ny;
+  if (c->slab || (cl > 1 && ny / cl < 2)) return false;
+  const int rows = (ny + cl - 1) / cl;
+  if (cl > 1)  // the off-midpoint Dirichlet rule reads two nodes beyond its own: a ghost row holds one
+    for (const clbm_link& k : c->h_links)
+      if (k.dir <= 4 && k.q < 0.5 && c->h_tbc[k.tbc].b1 == 0.0) return false;
+  int off[kMaxCluster + 1], most = 0;
+  const std::vector<int32_t>& v = c->h_bnodes;  // ascending
+  for (int r = 0; r <= cl; ++r)
+    off[r] = (int)(std::lower_bound(v.begin(), v.end(), (long long)r * ny / cl * c->pitch) - v.begin());
+  for (int r = 0; r < cl; ++r) most = std::max(most, off[r + 1] - off[r]);
+  if (nx > 65535 || rows + 2 > 65535) return false;  // 16-bit coordinates of the boundary nodes
+  const size_t smem = c->L->resident_smem(nx, rows, most, c->p.viscous_heating);
+  if (smem > max_smem) return false;
+  const int items = (most + 31) / 32 * 32 + rows * nx;
+  // whole passes over the items: as few threads as take the same number of passes
+  const int passes = (items + max_threads - 1) / max_threads;
+  plan->cl = cl;
+  plan->threads = std::max(64, ((items + passes - 1) / passes + 31) / 32 * 32);
+  plan->smem = smem;
+  if (lat) {
+    const ViewInfo w = describe_view(c);
+    lat->L.g = w.g;
+    lat->L.c = w.c;
+    lat->L.buf[0] = w.buf[0];
+    lat->L.buf[1] = w.buf[1];
+    lat->L.snap = nullptr;
+    lat->bnodes = c->d_bnodes;
+    std::copy(off, off + cl + 1, lat->bn_off);
+    lat->bn_most = most;
+    lat->lat = 0;
+  }
+  return true;
 }
 
 void set_view_time(clbm_ctx* c, int64_t t, int cur) {

@@ -109,6 +109,16 @@ struct clbm_batch {
   std::vector<int> nx, ny, py, masked, width, group;
   std::vector<long long> nodes;
   std::vector<int> grid;  // per group
+  // lattices that take their steps in shared memory: launches by cluster size, and per lattice its
+  // cluster size (0: the tile kernels)
+  struct Resident {
+    ResPlan plan;
+    int n = 0;
+    ResLat* d_lats = nullptr;
+  };
+  std::vector<Resident> resident;
+  std::vector<int> res_cl;
+  bool tiled = true;  // some lattice takes the tile kernels
   std::vector<long long> group_base = std::vector<long long>(kBatchGroups, 0);  // tile-list offsets
   BatchLat* d_lats = nullptr;
   int* d_active = nullptr;
@@ -147,6 +157,7 @@ static clbm_status bfail(clbm_batch* b, clbm_status s, const std::string& m) {
 // Rows that get interior tiles: all rows of a periodic y axis, else all but the
 // first and last (boundary rows).
 static int interior_rows(const clbm_batch* b, int i) {
+  if (b->res_cl[i]) return 0;  // no tiles
   return b->py[i] ? b->ny[i] : std::max(b->ny[i] - 2, 0);
 }
 
@@ -199,7 +210,8 @@ static clbm_status build_tiles(clbm_batch* b) {
 // (which, next to solids, replace the provisional values the tiles wrote).
 static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
   std::vector<int> used(kBatchGroups, 0);
-  for (int i = 0; i < b->n; ++i) used[b->group[i]] = 1;
+  for (int i = 0; i < b->n; ++i)
+    if (!b->res_cl[i]) used[b->group[i]] = 1;
   const std::vector<long long>& base = b->group_base;  // as in upload_layout
   for (int g = 0; g < kBatchGroups; ++g) {
     if (!used[g]) continue;
@@ -210,6 +222,82 @@ static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
   }
   BCUDA(b, b->L->batch_boundary(b->d_lats, b->d_bent, b->nbent, b->d_active, parity, &b->d_ctl->t,
                                 tstep, b->rounding, b->stream));
+  return CLBM_OK;
+}
+
+// K steps of the resident lattices, from buffer 0 (K even: back to it).
+static clbm_status launch_resident(clbm_batch* b, int K) {
+  for (const clbm_batch::Resident& r : b->resident) {
+    ResArgs a{};
+    a.lats = r.d_lats;
+    a.active = b->d_active;
+    a.tptr = &b->d_ctl->t;
+    a.cl = r.plan.cl;
+    a.steps = K;
+    a.stochastic = b->rounding;
+    BCUDA(b, b->L->resident_step(a, r.n, r.plan.threads, r.plan.smem, 0, b->stream));
+  }
+  return CLBM_OK;
+}
+
+// Which lattices take their steps in shared memory.  A cluster per lattice, as
+// few blocks as leave two blocks to a multiprocessor (their barriers then
+// overlap); more blocks while the batch does not fill the device.
+static clbm_status plan_resident(clbm_batch* b) {
+  const int n = b->n;
+  b->res_cl.assign(n, 0);
+  if (b->precision == CLBM_F64) return CLBM_OK;  // bound by the FP64 pipes of every multiprocessor
+  int dev = 0, sms = 0;
+  BCUDA(b, cudaGetDevice(&dev));
+  BCUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  std::vector<int> cl(n, 0);
+  long long blocks = 0;
+  for (int i = 0; i < n; ++i) {
+    for (int c = 1; c <= kMaxCluster && !cl[i]; c *= 2) {
+      ResPlan p;
+      if (resident_plan(b->views[i], c, kMaxResidentSmem / 2 - 1024, kMaxResidentThreads / 2, &p, nullptr)) cl[i] = c;
+    }
+    blocks += cl[i];
+  }
+  if (blocks == 0) return CLBM_OK;
+  for (bool grown = true; grown;) {  // double the bands while every block still has its own slot
+    grown = false;
+    for (int i = 0; i < n; ++i) {
+      ResPlan p;
+      if (cl[i] && cl[i] < kMaxCluster && blocks + cl[i] <= 2 * sms &&
+          resident_plan(b->views[i], 2 * cl[i], kMaxResidentSmem / 2 - 1024, kMaxResidentThreads / 2, &p, nullptr)) {
+        blocks += cl[i];
+        cl[i] *= 2;
+        grown = true;
+      }
+    }
+  }
+  for (int c = 1; c <= kMaxCluster; c *= 2) {
+    clbm_batch::Resident r;
+    std::vector<ResLat> lats;
+    for (int i = 0; i < n; ++i) {
+      if (cl[i] != c) continue;
+      ResPlan p;
+      ResLat l;
+      resident_plan(b->views[i], c, kMaxResidentSmem / 2 - 1024, kMaxResidentThreads / 2, &p, &l);
+      l.L.snap = nullptr;
+      l.lat = i;
+      lats.push_back(l);
+      r.plan.cl = c;
+      r.plan.threads = std::max(r.plan.threads, p.threads);
+      r.plan.smem = std::max(r.plan.smem, p.smem);
+    }
+    if (lats.empty() || b->L->resident_clusters(c, r.plan.threads, r.plan.smem, 0) < 1) continue;
+    r.n = (int)lats.size();
+    if (cudaMalloc(&r.d_lats, lats.size() * sizeof(ResLat)) != cudaSuccess) {
+      cudaGetLastError();
+      return CLBM_ENOMEM;
+    }
+    b->resident.push_back(r);
+    BCUDA(b, cudaMemcpy(r.d_lats, lats.data(), lats.size() * sizeof(ResLat), cudaMemcpyHostToDevice));
+    for (const ResLat& l : lats) b->res_cl[l.lat] = c;
+  }
+  b->tiled = std::count(b->res_cl.begin(), b->res_cl.end(), 0) > 0;
   return CLBM_OK;
 }
 
@@ -233,6 +321,7 @@ static void release(clbm_batch* b) {
   cudaFree(b->d_rpart);
   cudaFree(b->d_snap);
   cudaFree(b->d_snap_valid);
+  for (auto& r : b->resident) cudaFree(r.d_lats);
   if (b->h_ctl) cudaFreeHost(b->h_ctl);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
 }
@@ -258,7 +347,7 @@ static clbm_status autotune(clbm_batch* b) {
     std::vector<int> active(n, 0);
     long long nodes = 0;
     for (int i = 0; i < n; ++i)
-      if (width_class(b->nx[i]) == cls) {
+      if (width_class(b->nx[i]) == cls && !b->res_cl[i]) {
         active[i] = 1;
         nodes += b->nodes[i];
       }
@@ -371,6 +460,10 @@ clbm_status clbm_batch_create(const clbm_batch_item* items, int32_t n, int32_t a
     cudaGetLastError();
     return bail(CLBM_ENOMEM);
   }
+  {
+    const clbm_status st = plan_resident(b);
+    if (st != CLBM_OK) return bail(st);
+  }
   std::vector<BatchLat> lats(n);
   std::vector<int2> bent;
   long long snap_off = 0;
@@ -384,7 +477,7 @@ clbm_status clbm_batch_create(const clbm_batch_item* items, int32_t n, int32_t a
     lats[i].snap = b->d_snap + snap_off;
     snap_off += 3 * b->nodes[i];
     b->masked[i] = v.g.flags != nullptr;
-    for (int k = 0; k < v.nb; ++k) bent.push_back(make_int2(i, v.bnodes_host[k]));
+    for (int k = 0; k < v.nb && !b->res_cl[i]; ++k) bent.push_back(make_int2(i, v.bnodes_host[k]));
   }
   b->nbent = (int)bent.size();
   if (!bent.empty()) {
@@ -478,8 +571,8 @@ clbm_status clbm_batch_solve(clbm_batch* b, double tol, int64_t max_steps, int32
     }
     cudaGraph_t graph;
     BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    clbm_status cst = CLBM_OK;
-    for (int j = 0; j < K && cst == CLBM_OK; ++j) cst = launch_steps(b, j & 1, j);
+    clbm_status cst = launch_resident(b, K);
+    for (int j = 0; j < K && cst == CLBM_OK && b->tiled; ++j) cst = launch_steps(b, j & 1, j);
     if (cst == CLBM_OK && b->L->batch_residual(b->d_lats, b->d_active, b->d_snap_valid, b->d_res, n, K,
                                                b->d_rpart, b->res_chunks, b->stream) != cudaSuccess)
       cst = CLBM_ECUDA;

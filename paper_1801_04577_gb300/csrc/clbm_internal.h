@@ -191,6 +191,29 @@ struct BatchCtl {
   int count[kBatchGroups];     // tiles per launch group
 };
 
+// One lattice of the resident kernel: a cluster of blocks, each with a band of
+// rows; its boundary nodes bnodes[bn_off[r]] .. bnodes[bn_off[r + 1]) are block r's.
+constexpr int kMaxCluster = 16;
+constexpr int kMaxResidentThreads = 512;        // of a block (128 registers each)
+constexpr size_t kMaxResidentSmem = 232448;     // 227 KB: the most dynamic shared memory of a block
+struct ResLat {
+  BatchLat L;
+  const int32_t* bnodes;
+  int bn_off[kMaxCluster + 1];
+  int bn_most;  // boundary nodes of the block that has most of them
+  int lat;      // index in the batch (its `active` entry)
+  int pad;
+};
+
+struct ResArgs {
+  const ResLat* lats;      // one per cluster, or nullptr: `one`
+  const int* active;       // or nullptr: all
+  const long long* tptr;   // device step counter, or nullptr: t0
+  long long t0;
+  int cl, steps, cur, stochastic;  // blocks per cluster; buffer `cur` holds the current state
+  ResLat one;
+};
+
 // Launchers implemented once per storage type (S = double, float, __half,
 // __nv_bfloat16).  All enqueue on `stream` and return cudaGetLastError().
 struct Launchers {
@@ -231,6 +254,12 @@ struct Launchers {
                                 double* res, int n, int K, double* part, int maxchunks,
                                 cudaStream_t s);
   int residual_chunk;  // nodes per residual chunk
+
+  // resident steps: shared memory of a block with `rows` rows and nb boundary nodes, clusters of `cl`
+  // such blocks that the device holds at once (0: none), and the launch of n lattices
+  size_t (*resident_smem)(int nx, int rows, int nb, int vh);
+  int (*resident_clusters)(int cl, int threads, size_t smem, int vh);
+  cudaError_t (*resident_step)(const ResArgs& a, int n, int threads, size_t smem, int vh, cudaStream_t s);
 };
 
 extern const Launchers kLaunchF64;
@@ -255,6 +284,12 @@ clbm_status create_view(const clbm_params* p, cudaStream_t s, void* buf_a, void*
                         clbm_ctx** out);
 ViewInfo describe_view(const clbm_ctx* c);
 void set_view_time(clbm_ctx* c, int64_t t, int cur);
+// A lattice's launch on clusters of `cl` resident blocks: false if its bands do not fit.
+struct ResPlan {
+  int cl = -1, threads = 0;  // cl: -1 not planned yet, 0 the lattice is not resident
+  size_t smem = 0;
+};
+bool resident_plan(const clbm_ctx* c, int cl, size_t max_smem, int max_threads, ResPlan* plan, ResLat* lat);
 
 // *t += k on the device (advances the step counter of a captured step graph)
 cudaError_t launch_advance(long long* t, int k, cudaStream_t s);

@@ -473,7 +473,7 @@ __host__ __device__ __forceinline__ void equilibrium(const Co<R>& c, R rho, R ux
   h[4] = R(0.5) * (q02 - q01);
 }
 
-// The stored state as the boundary nodes read it.
+// The stored state as the boundary nodes read it: planes in device memory ...
 template <typename S>
 struct PlaneSrc {
   using Idx = long long;
@@ -481,6 +481,14 @@ struct PlaneSrc {
   long long plane;
   __device__ __forceinline__ S at(int q, long long i) const { return p[q * plane + i]; }
 };
+// ... or whole nodes in shared memory, ST values apart.
+template <typename S, int ST>
+struct NodeSrc {
+  using Idx = int;
+  const S* p;
+  __device__ __forceinline__ S at(int q, int i) const { return p[i * ST + q]; }
+};
+
 // T at a node from its post-collision thermal deviations: T = T0 + sum h* - Q/2,
 // Q including the node's stored viscous source when that is enabled.
 template <class Src, typename R, typename Idx>
@@ -1421,6 +1429,12 @@ __global__ void average_state_kernel(S* __restrict__ a, const S* __restrict__ b,
   }
 }
 
+}  // namespace clbm
+
+#include "clbm_resident.cuh"
+
+namespace clbm {
+
 // ---------------------------------------------------------------------------
 // Launchers for one storage type
 // ---------------------------------------------------------------------------
@@ -1586,8 +1600,57 @@ struct LaunchImpl {
     return cudaGetLastError();
   }
 
+  static size_t resident_smem(int nx, int rows, int nb, int vh) {
+    return resident_bytes<S>(nx, rows, nb, vh != 0);
+  }
+
+
+  static cudaLaunchConfig_t resident_config(int cl, int n, int threads, size_t smem, cudaStream_t s,
+                                            cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cl * n));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)cl;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+  }
+
+  // the kernel with the limits that its launches may need
+  static cudaError_t resident_prepare(int vh) {
+    auto k = vh ? resident_kernel<S, true> : resident_kernel<S, false>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxResidentSmem);
+    return e ? e : cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
+
+  static int resident_clusters(int cl, int threads, size_t smem, int vh) {
+    int n = 0;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = resident_config(cl, 1, threads, smem, nullptr, &attr);
+    if (resident_prepare(vh) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, vh ? resident_kernel<S, true> : resident_kernel<S, false>, &cfg) !=
+            cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return n;
+  }
+
+  static cudaError_t resident_step(const ResArgs& a, int n, int threads, size_t smem, int vh, cudaStream_t s) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = resident_config(a.cl, n, threads, smem, s, &attr);
+    return cudaLaunchKernelEx(&cfg, vh ? resident_kernel<S, true> : resident_kernel<S, false>, a);
+  }
+
   static Launchers table() {
     Launchers L;
+    L.resident_smem = &resident_smem;
+    L.resident_clusters = &resident_clusters;
+    L.resident_step = &resident_step;
     L.average = &average;
     L.batch_step = &batch_step;
     L.batch_boundary = &batch_boundary;
