@@ -520,6 +520,17 @@ __device__ __forceinline__ const R* side_wall(const DevGeom& g, int sd, bool hav
     return g.side_k[sd][have2 ? 1 : 0];
 }
 
+// Eq. 26's cT2 (T_m - T0) at box side sd for the node `own` with `next` behind it.
+template <class Src, typename R, typename Idx>
+__device__ __forceinline__ R side_heat(const Src& src, const DevGeom& g, const Co<R>& c, int sd, bool have2,
+                                       Idx own, Idx next) {
+  const R* k = side_wall<R>(g, sd, have2);
+  R e = k[2];
+  if (k[1] != R(0)) e = fma_(k[1], node_heat(src, next, c), e);
+  if (k[0] != R(0)) e = fma_(k[0], node_heat(src, own, c), e);
+  return e;
+}
+
 // New state of node (x, y) next to a wall, a solid or a periodic seam: pull,
 // bounce-back, Eq. 26-28, collision.  src: the stored state, indexed
 // y * g.pitch + x; fl, slot: its flags and its entry of the link tables
@@ -595,7 +606,8 @@ __device__ __forceinline__ void node_update(const DevGeom& g, const Co<R>& c, co
       R e = kc;
       if (kd != R(0)) e = fma_(kd, node_heat(src, ahead(ex, ey, 2), c), e);
       if (kb != R(0)) e = fma_(kb, node_heat(src, ahead(ex, ey, 1), c), e);
-      h[j] = sub_(fma_(ka, s1, e), h[j]);  // Eq. 26
+      if (ka != R(0)) e = fma_(ka, s1, e);
+      h[j] = sub_(e, h[j]);  // Eq. 26
     }
   }
   if (MASK && (fl & kFlagOffMid)) {  // walls off the link midpoint: interpolated bounce-back
@@ -804,6 +816,158 @@ __device__ __forceinline__ void step_tile(const DevGeom& g, const Co<typename Tr
   for (int q = 0; q < 14; ++q) stv<S, V>(out + q * plane, v[q]);
 }
 
+// Interior and walls in one: the tile for a lattice without a mask or moving
+// sides, every node final.  The walls of a box need no list: a row next to a
+// y wall pulls the opposite populations of its own row instead of the row
+// beyond, and the lanes of the first and last column take the one value that
+// an interior lane gets from the neighbouring tile from the opposite
+// population of the edge node, or from around a periodic seam.
+// EDGE: the tile touches a wall or seam.  It is a second copy of the code, and
+// every choice in it is a select of an address or a value: a branch between
+// the loads would keep them from being issued together (branches instead of
+// selects took the FP32 4096 x 2048 step from 0.14 to 0.19 ms).
+template <typename S, int V, bool VH, bool SKIP_DEAD, bool EDGE>
+__device__ __forceinline__ void box_tile(const DevGeom& g, const Co<typename Traits<S>::R>& c,
+                                            const S* __restrict__ src, S* __restrict__ dst, int y, int xw,
+                                            int lane, uint32_t seed, int stochastic) {
+  using R = typename Traits<S>::R;
+  const int x0 = xw + lane * V;
+  const long long plane = g.plane;
+  const bool lo = EDGE && g.ywlo && y == g.ylo, hi = EDGE && g.ywhi && y == g.yhi - 1;
+  int ym = y - 1, yp = y + 1;  // rows the e_y = +1 / -1 populations come from
+  if (g.py) {
+    ym = ym < 0 ? g.ny - 1 : ym;
+    yp = yp >= g.ny ? 0 : yp;
+  }
+  const int lastx = g.nx - 1;
+  const bool live = !SKIP_DEAD || x0 < g.nx;
+  const bool first = EDGE && x0 == 0, last = EDGE && x0 <= lastx && lastx < x0 + V;
+  const bool wall_l = first && !g.px, wall_r = last && !g.px;
+  const long long row_y = (long long)y * g.pitch;
+  // columns beyond the tile that lanes 0 and 31 (and the edge lanes) read: the
+  // neighbouring tile's, the other end of a periodic row, the edge node's own
+  const int xl = x0 > 0 ? x0 - 1 : (g.px ? lastx : 0);
+  const int xr = last ? (g.px ? 0 : lastx) : (x0 + V < g.pitch ? x0 + V : g.pitch - 1);
+  const bool get_l = lane == 0, get_r = (lane == 31 || last) && live;
+
+  R v[14][V];
+#pragma unroll
+  for (int q = 0; q < 14; ++q) {
+    const int dir = q < 9 ? q : q - 9, opp = q - dir + opp_of(dir);
+    const int ex = ex_of(dir), ey = ey_of(dir);
+    const bool w = ey > 0 ? lo : (ey < 0 ? hi : false);
+    const int row = w ? y : (ey > 0 ? ym : (ey < 0 ? yp : y));
+    const S* base = src + (w ? opp : q) * plane + (long long)row * g.pitch;
+    R t[V];
+    if (live) {
+      ldv<S, V>(base + x0, t);
+    } else {
+#pragma unroll
+      for (int k = 0; k < V; ++k) t[k] = R(0);
+    }
+    if (ex == 0) {
+#pragma unroll
+      for (int k = 0; k < V; ++k) v[q][k] = t[k];
+    } else if (ex > 0) {  // value from x - 1
+      const S* at = EDGE && wall_l ? src + opp * plane + row_y : base;
+      R left = __shfl_up_sync(0xffffffffu, t[V - 1], 1);
+      if (get_l) left = to_r(at[xl]);
+      v[q][0] = w ? t[0] : left;
+#pragma unroll
+      for (int k = 1; k < V; ++k) v[q][k] = w ? t[k] : t[k - 1];
+    } else {  // value from x + 1
+      const S* at = EDGE && wall_r ? src + opp * plane + row_y : base;
+      R right = __shfl_down_sync(0xffffffffu, t[0], 1);
+      if (get_r) right = to_r(at[xr]);
+      // the last column may lie inside the vector
+#pragma unroll
+      for (int k = 0; k < V - 1; ++k) v[q][k] = w ? t[k] : (EDGE && x0 + k == lastx ? right : t[k + 1]);
+      v[q][V - 1] = w ? t[V - 1] : right;
+    }
+  }
+  if (!g.px && (first || last)) {  // Eq. 26 at the x walls
+    const PlaneSrc<S> ps{src, plane};
+    if (first) v[10][0] = sub_(side_heat(ps, g, c, 0, g.nx > 1, row_y, row_y + 1), v[10][0]);
+    if (last) {
+      const R e = side_heat(ps, g, c, 1, g.nx > 1, row_y + lastx, row_y + lastx - 1);
+#pragma unroll
+      for (int k = 0; k < V; ++k)
+        if (x0 + k == lastx) v[12][k] = sub_(e, v[12][k]);
+    }
+  }
+  if ((lo || hi) && live) {  // rows next to a y wall: Eq. 26 for the whole row
+    auto heat = [&](int row, R(&o)[V]) {
+      const S* b = src + (long long)row * g.pitch + x0;
+      R t[V];
+      ldv<S, V>(b + 9 * plane, o);
+#pragma unroll
+      for (int q = 10; q < 14; ++q) {
+        ldv<S, V>(b + q * plane, t);
+#pragma unroll
+        for (int k = 0; k < V; ++k) o[k] = add_(o[k], t[k]);
+      }
+      if (VH) {
+        ldv<S, V>(b + 14 * plane, t);
+#pragma unroll
+        for (int k = 0; k < V; ++k) o[k] = fma_(R(-0.5), t[k], o[k]);
+      }
+    };
+    auto wall = [&](int sd, int y2, bool have2, R(&h)[V]) {
+      const R* k = side_wall<R>(g, sd, have2);
+      R e[V], t[V];
+#pragma unroll
+      for (int m = 0; m < V; ++m) e[m] = k[2];
+      if (k[1] != R(0)) {
+        heat(y2, t);
+#pragma unroll
+        for (int m = 0; m < V; ++m) e[m] = fma_(k[1], t[m], e[m]);
+      }
+      if (k[0] != R(0)) {
+        heat(y, t);
+#pragma unroll
+        for (int m = 0; m < V; ++m) e[m] = fma_(k[0], t[m], e[m]);
+      }
+#pragma unroll
+      for (int m = 0; m < V; ++m) h[m] = sub_(e[m], h[m]);
+    };
+    if (lo) wall(2, y + 1, !hi, v[11]);
+    if (hi) wall(3, y - 1, !lo, v[13]);
+  }
+
+  R qv[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    R d[9], h[5];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) d[q] = v[q][k];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) h[q] = v[9 + q][k];
+    collide<R, VH>(c, d, h, qv[k]);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) v[q][k] = d[q];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) v[9 + q][k] = h[q];
+  }
+  if (!live) return;
+  S* out = dst + row_y + x0;
+  if constexpr (VH) stv<S, V>(out + 14 * plane, qv);
+  if constexpr (sizeof(S) == 2) {
+    if (stochastic) {
+      // x0 is a multiple of V (tiles start at multiples of 32 V nodes)
+      const uint32_t key = sr_key(seed, (long long)(y + g.yoff) * g.pitch + (x0 & ~3));
+#pragma unroll
+      for (int q = 0; q < 14; ++q) {
+        uint32_t r0, r1;
+        sr_words(key, q, r0, r1);
+        stv_sr<S, V>(out + q * plane, v[q], r0, r1, x0 & 3);
+      }
+      return;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 14; ++q) stv<S, V>(out + q * plane, v[q]);
+}
+
 // Boundary update of node index i (pitch layout).
 template <typename S, bool MASK>
 __device__ __forceinline__ void step_node(const DevGeom& g, const Co<typename Traits<S>::R>& c,
@@ -832,41 +996,6 @@ __device__ __forceinline__ uint32_t step_seed(const StepArgs& a) {
   return (uint32_t)(t * 0x9E3779B1ull) ^ (uint32_t)(t >> 32);
 }
 
-// One launch = the interior update of one time step of one lattice.
-template <typename S, bool VH>
-__global__ void __launch_bounds__(kStepThreads) step_kernel(const StepArgs a) {
-  using R = typename Traits<S>::R;
-  constexpr int V = Traits<S>::V;
-  const int lane = threadIdx.x & 31;
-  const int warp = blockIdx.x * (kStepThreads / 32) + (threadIdx.x >> 5);
-  const int xw = warp * 32 * V;
-  if (xw >= a.g.nx) return;  // whole warps only: the shuffles need all 32 lanes
-  const int y = a.g.ylo + (a.reverse ? (int)gridDim.y - 1 - (int)blockIdx.y : (int)blockIdx.y);
-  // a tile of solid nodes only: nothing reads them, so neither load nor store
-  if (a.g.tile_fluid && !a.g.tile_fluid[(long long)y * a.g.tiles_per_row + warp]) return;
-  const Co<R> c = make_co<R>(a.c);
-  step_tile<S, V, false, VH, sizeof(S) != 2>(a.g, c, static_cast<const S*>(a.src),
-                                             static_cast<S*>(a.dst), y, xw, lane, step_seed(a),
-                                             a.stochastic);
-}
-
-// The boundary nodes of the same step (launched after step_kernel).
-template <typename S, bool MASK>
-__global__ void __launch_bounds__(kRedThreads) boundary_kernel(const StepArgs a) {
-  using R = typename Traits<S>::R;
-  const Co<R> c = make_co<R>(a.c);
-  const uint32_t seed = step_seed(a);
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.nb; k += gridDim.x * blockDim.x)
-    step_node<S, MASK>(a.g, c, static_cast<const S*>(a.src), static_cast<S*>(a.dst), a.bnodes[k],
-                       seed, a.stochastic);
-}
-
-// Box lattices (no mask): interior and boundary nodes are disjoint, so one
-// launch does both.  The first nbb blocks update the boundary list (first and
-// last column, first and last row of a non-periodic y axis); the others are
-// interior tiles of rows that are not boundary rows, which skip the first and
-// last column.  The latency-bound boundary work then overlaps the streaming
-// interior work instead of following it.
 // Blocks per SM the register budget is cut for: five (96 registers) where the
 // step is memory-bound (FP32, FP64 storage); six (80 registers, a 44-byte
 // spill) for 16-bit storage, which is bound by issue and memory latency and
@@ -874,7 +1003,35 @@ __global__ void __launch_bounds__(kRedThreads) boundary_kernel(const StepArgs a)
 template <typename S>
 constexpr int kStepBlocks = sizeof(S) == 2 ? 6 : 5;
 
-template <typename S, bool VH, bool MASKED = false>
+// Lattices without a mask or moving sides: blocks of up to four tiles of one
+// row, in row order.  The row, and which copy of the tile runs, depend on
+// blockIdx alone, so that the inner tiles keep their addresses in uniform
+// registers (rows from threadIdx, or a choice per warp, cost the 16-bit step
+// 15 %; edge tiles in blocks of their own, out of row order, the FP32 step 6 %).
+template <typename S, int V, bool VH>
+__global__ void __launch_bounds__(kStepThreads, kStepBlocks<S>) step_box_kernel(const StepArgs a, int xblocks,
+                                                                              int rows) {
+  using R = typename Traits<S>::R;
+  const Co<R> c = make_co<R>(a.c);
+  const S* src = static_cast<const S*>(a.src);
+  S* dst = static_cast<S*>(a.dst);
+  const int b = blockIdx.x, row = b / xblocks, xb = b - row * xblocks;
+  const int xw = (xb * blockDim.x + (threadIdx.x & ~31)) * V;
+  if (xw >= a.g.nx) return;  // whole warps only
+  const int y = a.g.ylo + (a.reverse ? rows - 1 - row : row);
+  const bool edge = xb == 0 || xb == xblocks - 1 || (a.g.ywlo && y == a.g.ylo) || (a.g.ywhi && y == a.g.yhi - 1);
+  if (edge)
+    box_tile<S, V, VH, sizeof(S) != 2, true>(a.g, c, src, dst, y, xw, threadIdx.x & 31, step_seed(a), a.stochastic);
+  else
+    box_tile<S, V, VH, sizeof(S) != 2, false>(a.g, c, src, dst, y, xw, threadIdx.x & 31, step_seed(a), a.stochastic);
+}
+
+// Lattices with a mask or moving sides: interior and boundary nodes are
+// disjoint, so one launch does both.  The first nbb blocks update the boundary
+// list; the others are interior tiles, which leave those nodes out.  The
+// latency-bound boundary work then overlaps the streaming interior work
+// instead of following it.
+template <typename S, bool VH, bool MASKED>
 __global__ void __launch_bounds__(kStepThreads, kStepBlocks<S>) step_fused_kernel(const StepArgs a, int nbb,
                                                                                 int xblocks, int y0, int rows) {
   using R = typename Traits<S>::R;
@@ -1442,46 +1599,59 @@ template <typename S>
 struct LaunchImpl {
   static constexpr int V = Traits<S>::V;
 
-  static cudaError_t step(const StepArgs& a, cudaStream_t s) {
-    const int nodes_per_block = kStepThreads * V;
-    const int xblocks = (a.g.nx + nodes_per_block - 1) / nodes_per_block;
-    // one fused launch: boundary nodes in the first blocks, interior tiles in the
-    // rest (box lattices; masked ones with their tile classes, whose interior
-    // tiles leave the listed nodes out)
-    if (!a.g.flags || a.g.tile_fluid) {
-      // interior tiles: the own rows that are not next to a box wall (those are
-      // boundary rows, in the node list)
-      const int y0 = a.g.ylo + a.g.ywlo;
-      const int rows = std::max(0, a.g.yhi - a.g.ywhi - y0);
-      const int nbb = (a.nb + kStepThreads - 1) / kStepThreads;
-      const long long blocks = (long long)nbb + (long long)xblocks * rows;
-      if (blocks > 0 && blocks < (1LL << 31)) {
-        const unsigned nblk = (unsigned)blocks;
-        if (a.g.flags) {
-          if (a.c.vh)
-            step_fused_kernel<S, true, true><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-          else
-            step_fused_kernel<S, false, true><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-        } else {
-          if (a.c.vh)
-            step_fused_kernel<S, true><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-          else
-            step_fused_kernel<S, false><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-        }
-        return cudaGetLastError();
-      }
-    }
-    dim3 grid(xblocks, a.g.yhi - a.g.ylo);
+  template <int VV>
+  static cudaError_t box_step(const StepArgs& a, cudaStream_t s) {
+    const int tiles = (a.g.nx + 32 * VV - 1) / (32 * VV), rows = a.g.yhi - a.g.ylo;
+    const int wx = std::min(tiles, kStepThreads / 32), xblocks = wx > 0 ? (tiles + wx - 1) / wx : 0;
+    if (xblocks <= 0 || rows <= 0) return cudaSuccess;
+    const unsigned nblk = (unsigned)xblocks * (unsigned)rows;
     if (a.c.vh)
-      step_kernel<S, true><<<grid, kStepThreads, 0, s>>>(a);
+      step_box_kernel<S, VV, true><<<nblk, 32 * wx, 0, s>>>(a, xblocks, rows);
     else
-      step_kernel<S, false><<<grid, kStepThreads, 0, s>>>(a);
-    if (a.nb > 0) {
-      const int blocks = (a.nb + kRedThreads - 1) / kRedThreads;
-      if (a.g.flags)
-        boundary_kernel<S, true><<<blocks, kRedThreads, 0, s>>>(a);
+      step_box_kernel<S, VV, false><<<nblk, 32 * wx, 0, s>>>(a, xblocks, rows);
+    return cudaGetLastError();
+  }
+
+  static int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+      sms = 152;
+    return sms;
+  }
+
+  static cudaError_t step(const StepArgs& a, cudaStream_t s) {
+    if (!a.g.flags && !a.g.moving) {
+      // FP64: an FP64 instruction holds a warp's quarter of the multiprocessor for 64 cycles, so a
+      // step is as long as the most nodes that one lane of a quarter updates; tiles of one node a
+      // lane where that number is then smaller (48^2: 12.1 -> 9 us a step)
+      if constexpr (sizeof(S) == 8) {
+        const long long quarters = 4LL * sm_count(), rows = a.g.yhi - a.g.ylo;
+        const long long w1 = rows * ((a.g.nx + 31) / 32), w2 = rows * ((a.g.nx + 63) / 64);
+        if ((w1 + quarters - 1) / quarters < 2 * ((w2 + quarters - 1) / quarters)) return box_step<1>(a, s);
+      }
+      return box_step<V>(a, s);
+    }
+    const int tiles = (a.g.nx + 32 * V - 1) / (32 * V);  // of a row
+    // interior tiles: the own rows that are not next to a box wall (those are
+    // boundary rows, in the node list).  Fewer than 2^31 blocks: a lattice has
+    // at most 2^31 nodes, and each block updates more than one.
+    const int xblocks = (tiles + kStepThreads / 32 - 1) / (kStepThreads / 32);
+    const int y0 = a.g.ylo + a.g.ywlo;
+    const int rows = std::max(0, a.g.yhi - a.g.ywhi - y0);
+    const int nbb = (a.nb + kStepThreads - 1) / kStepThreads;
+    const unsigned nblk = (unsigned)nbb + (unsigned)xblocks * (unsigned)rows;
+    if (nblk == 0) return cudaSuccess;
+    if (a.g.flags) {
+      if (a.c.vh)
+        step_fused_kernel<S, true, true><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
       else
-        boundary_kernel<S, false><<<blocks, kRedThreads, 0, s>>>(a);
+        step_fused_kernel<S, false, true><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
+    } else {
+      if (a.c.vh)
+        step_fused_kernel<S, true, false><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
+      else
+        step_fused_kernel<S, false, false><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
     }
     return cudaGetLastError();
   }
