@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "../../include/clbm.h"
+#include "clbm_conv.cuh"
 #include "clbm_tc.cuh"
 
 namespace {
@@ -319,17 +320,38 @@ struct GatherRows {
 };
 
 struct TStoreAct {  // D(m = pixel, n = channel)
+  static constexpr bool kRow = false;
   StoreAct s;
   __device__ __forceinline__ void operator()(int m, int n, float v, int) const { s(n, m, v); }
 };
 struct TStoreSplit {  // D(m = pixel, n = channel) of split z -> part[z][n][m]
+  static constexpr bool kRow = false;
   float* part;
   int M, N;
   __device__ __forceinline__ void operator()(int m, int n, float v, int z) const {
     part[((long long)z * N + n) * M + m] = v;
   }
 };
+// D(m = pixel, n = channel) through the epilogue of the operand-layout convolutions
+struct TStoreOp {
+  static constexpr bool kRow = true;
+  conv::Epilogue e;
+  __device__ __forceinline__ void row(int m, int n0, const float (&v)[16]) const {
+    const int hw = e.H * e.W, n = m / hw, p = m - n * hw, y = p / e.W, x = p - y * e.W;
+    const int Wp = e.W + 2, Pn = ((e.H + 2) * Wp + 15) / 16 * 16;
+    const int pos = n * Pn + (y + 1) * Wp + x + 1;
+#pragma unroll
+    for (int h = 0; h < 16; h += 8) {
+      if (n0 + h >= e.channels) continue;
+      float u[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) u[k] = v[h + k];
+      e.apply(pos, n, p, n0 + h, u, e.bias + n0 + h);
+    }
+  }
+};
 struct TStorePartial {  // D(m = (ci, tap), n = co) of split z
+  static constexpr bool kRow = false;
   StorePartial s;
   __device__ __forceinline__ void operator()(int m, int n, float v, int z) const { s(n, m, v, z); }
 };
@@ -343,6 +365,7 @@ struct PackDesc {
   long long dst_off;  // first element of this layer's packed buffer
   int co, ci, kk;     // output / input channels, taps
   int transpose;      // 0: forward, 1: input gradient
+  int groups;         // channel groups of K in the chunk order of conv::conv_kernel; 0: K in order
   int N, K, bn, slices;
   long long size;     // packed elements (N tiles x slices x bn x 64)
 };
@@ -358,7 +381,10 @@ __global__ void pack_weights_kernel(const PackDesc* __restrict__ descs, const __
     const int nt = (int)(tile / d.slices), ks = (int)(tile - (long long)nt * d.slices);
     // inverse of chunk_off: 512 elements per 8-row group, 64 per K chunk, 8 per row
     const int rg = within >> 9, kc = (within >> 6) & 7, r7 = (within >> 3) & 7, e = within & 7;
-    const int n = nt * d.bn + rg * 8 + r7, k = ks * tc::kBK + kc * 8 + e;
+    const int n = nt * d.bn + rg * 8 + r7;
+    int chunk = ks * (tc::kBK / 8) + kc;
+    if (d.groups && conv::pair_swapped(chunk & ~1, d.groups, d.K / 8)) chunk ^= 1;
+    const int k = chunk * 8 + e;
     __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
     if (n < d.N && k < d.K) {
       if (!d.transpose) {  // n = co, k = t * ci + c
@@ -732,6 +758,11 @@ struct clbm_net {
     int N = 0;
   };
   Captured grad_pass, fwd_pass;
+  // Operand-layout convolutions (clbm_conv.cuh): the tensor-core network whose widths are multiples
+  // of eight.  Operands of the activations and of their gradients, per buffer (base nullptr: none).
+  bool direct = false;
+  std::vector<conv::Op> aop, gop;
+  std::vector<void*> op_mem;
   double* h_loss = nullptr;  // page-locked copy of the loss partials and mask sums
   float *tgt = nullptr, *msk = nullptr;  // the caller's target and mask, copied in before a pass
 };
@@ -851,6 +882,267 @@ long long dw_kper(int sms, bool tensor, long long Np, int Kd, int co) {
   return ((per + tc::kBK - 1) / tc::kBK) * tc::kBK;
 }
 
+// ---------------------------------------------------------------------------
+// Operand-layout passes (net->direct)
+// ---------------------------------------------------------------------------
+constexpr int kMaxSmem = 232448;  // 227 KB
+
+// Stages of weights beside the input tile (0: the tile does not fit).
+int conv_stages(int C, int taps, int W, int bn) {
+  for (int s = 4; s >= 2; --s)
+    if (conv::conv_smem(C, taps, W + 2, bn, s) <= kMaxSmem) return s;
+  return 0;
+}
+
+struct ConvSplit {
+  int splits, kper;  // ranges of K, 64-wide slices per range
+};
+// The ranges of the gathering GEMM (the partial sums, and so the results, are the same).
+ConvSplit conv_ranges(int sms, int pixels, int N, int K) {
+  const int slices = (K + tc::kBK - 1) / tc::kBK;
+  const int s = conv_splits(sms, pixels, N, K);
+  if (s <= 1) return {1, slices};
+  const int kper = ((K + s - 1) / s + tc::kBK - 1) / tc::kBK;
+  return {(slices + kper - 1) / kper, kper};
+}
+
+long long op_positions(const conv::Op& o, int N) { return (long long)N * o.Pn(); }
+long long split_stride(const conv::Op& o, int N) {
+  return (op_positions(o, N) + tc::kBM - 1) / tc::kBM * tc::kBM;
+}
+
+// D = conv(a, packed weights of `layer`) for N samples through the epilogue.
+cudaError_t conv_direct(clbm_net* net, const conv::Op& a, int layer, int transpose, int taps, int N,
+                        conv::Epilogue e) {
+  const PackDesc& d = net->pack[2 * layer + transpose];
+  const ConvSplit r = conv_ranges(net->sms, N * a.H * a.W, d.N, d.K);
+  e.H = a.H;
+  e.W = a.W;
+  e.N = N;
+  e.channels = d.N;
+  conv::ConvArgs c{};
+  c.a = a;
+  c.w = net->packed + d.dst_off;
+  c.taps = taps;
+  c.bn = d.bn;
+  c.slices = d.slices;
+  c.kper = r.kper;
+  c.stages = std::min(conv_stages(a.C, taps, a.W, d.bn), std::max(2, r.kper));
+  c.M = (int)op_positions(a, N);
+  c.Mst = split_stride(a, N);
+  c.part = r.splits > 1 ? net->part : nullptr;
+  c.epi = e;
+  c.err = net->d_tflag;
+  if (r.splits > 1 && (long long)r.splits * d.N * c.Mst > net->part_cap) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)(c.Mst / tc::kBM), (unsigned)((d.N + d.bn - 1) / d.bn), (unsigned)r.splits);
+  conv::conv_kernel<<<grid, conv::kThreads, conv::conv_smem(a.C, taps, a.W + 2, d.bn, c.stages), net->stream>>>(c);
+  if (r.splits > 1)
+    conv::conv_finish_kernel<<<dim3((unsigned)((c.M + 127) / 128), (unsigned)((d.N + 7) / 8)), 128, 0, net->stream>>>(
+        net->part, r.splits, c.M, c.Mst, e);
+  return cudaGetLastError();
+}
+
+// Launch shape of a weight gradient.
+struct DwShape {
+  int group_set, group_sets, tap_set, tap_sets, mtiles, kper, ranges, stages, smem;
+};
+DwShape dw_shape(int sms, const conv::Op& x, int co_groups, int taps, int N) {
+  DwShape s{};
+  const int groups = x.C / 8;
+  // at most 256 columns an MMA, and two stages that fit shared memory
+  for (s.group_sets = (groups + 31) / 32;; ++s.group_sets) {
+    s.group_set = (groups + s.group_sets - 1) / s.group_sets;
+    if (s.group_set == 1 || conv::dw_smem(std::min(16, co_groups), s.group_set, taps, x.W + 2, 2) <= kMaxSmem) break;
+  }
+  const int cols = conv::dw_cols(s.group_set);
+  s.tap_set = std::min(taps, 512 / cols);
+  s.tap_sets = (taps + s.tap_set - 1) / s.tap_set;
+  s.tap_set = (taps + s.tap_sets - 1) / s.tap_sets;
+  s.mtiles = (co_groups + 15) / 16;
+  const int gg = std::min(16, co_groups);
+  for (s.stages = 4; s.stages >= 2; --s.stages) {
+    s.smem = conv::dw_smem(gg, s.group_set, taps, x.W + 2, s.stages);
+    if (s.smem <= kMaxSmem / 2 || (s.stages == 2 && s.smem <= kMaxSmem)) break;
+  }
+  // about one block per multiprocessor, at least two stages of positions each
+  const long long K = (long long)N * x.Pn(), per_range = (long long)s.group_sets * s.tap_sets * s.mtiles;
+  const long long want = std::max<long long>(1, (sms + per_range - 1) / per_range);
+  const long long most = std::max<long long>(1, K / (2 * conv::kKP));
+  const long long r = std::min(want, most);
+  s.kper = (int)(((K + r - 1) / r + conv::kKP - 1) / conv::kKP * conv::kKP);
+  s.ranges = (int)((K + s.kper - 1) / s.kper);
+  return s;
+}
+
+// dW, db of a layer from its input operand x and output gradient operand g (and FP32 view gy).
+cudaError_t dw_direct(clbm_net* net, const Conv& cv, const conv::Op& x, const conv::Op& g, Act gy, int N) {
+  const int taps = cv.ks * cv.ks;
+  const DwShape s = dw_shape(net->sms, x, g.C / 8, taps, N);
+  conv::DwArgs a{};
+  a.x = x;
+  a.g = g;
+  a.taps = taps;
+  a.tap_set = s.tap_set;
+  a.tap_sets = s.tap_sets;
+  a.group_set = s.group_set;
+  a.K = (int)op_positions(x, N);
+  a.kper = s.kper;
+  a.stages = s.stages;
+  a.ci = cv.ci;
+  a.co = cv.co;
+  a.part = net->part;
+  a.err = net->d_tflag;
+  const long long n = (long long)taps * cv.ci * cv.co;
+  if (s.ranges * n > net->part_cap) return cudaErrorInvalidValue;
+  conv::dw_kernel<<<dim3((unsigned)s.ranges, (unsigned)(s.tap_sets * s.group_sets), (unsigned)s.mtiles),
+                    conv::kThreads, s.smem, net->stream>>>(a);
+  const long long want = std::max<long long>(1, (net->sms * 2048LL) / n);
+  int R = 1;
+  while (2 * R <= std::min(s.ranges, 32) && 2 * R <= want) R *= 2;
+  conv::dw_sum_kernel<<<(unsigned)std::min<long long>((n + 31) / 32, 65535), dim3(32, R), 0, net->stream>>>(
+      net->part, s.ranges, taps, cv.ci, cv.co, net->g + cv.w_off);
+  // bias: the partial sums are consumed, so part holds the chunk sums next
+  const int Np = N * cv.H * cv.W, chunks = (Np + kBiasChunk - 1) / kBiasChunk;
+  if ((long long)chunks * cv.co > net->part_cap) return cudaErrorInvalidValue;
+  bias_partial_kernel<<<dim3(chunks, cv.co), GT, 0, net->stream>>>(gy, N, net->part);
+  sum_splits(net->part, chunks, cv.co, net->g + cv.b_off, net->sms, net->stream);
+  return cudaGetLastError();
+}
+
+dim3 op_grid(long long pixels, int groups) {
+  return dim3((unsigned)std::max<long long>(1, std::min<long long>((pixels + 127) / 128, 4096)), (unsigned)groups);
+}
+
+// forward() on operands: FP32 copies only of the skip connections (pooled in FP32) and the output.
+cudaError_t forward_direct(clbm_net* net, const Plan& P, int N) {
+  const int L = net->cfg.levels, B = net->cfg.base;
+  cudaError_t e;
+  int li = 0;
+  auto conv_into = [&](const conv::Op& x, int out_id, int group, int taps, int relu, float* f32, int cs) {
+    const Conv& cv = net->convs[li];
+    conv::Epilogue ep{};
+    ep.bias = net->p + cv.b_off;
+    ep.relu = relu;
+    ep.op = net->aop[out_id];
+    ep.op_group = group;
+    ep.f32 = f32;
+    ep.cs = cs;
+    return conv_direct(net, x, li++, 0, taps, N, ep);
+  };
+  for (int l = 0; l < L - 1; ++l) {
+    const int c = B << l, up = (B << (l + 1)) / 8;
+    if (l == 0) {  // five (or any number of) input channels: the gathering GEMM
+      const Conv& cv = net->convs[li];
+      conv::Epilogue ep{};
+      ep.bias = net->p + cv.b_off;
+      ep.relu = 1;
+      ep.op = net->aop[P.a1[0]];
+      ep.H = ep.W = cv.H;
+      ep.N = N;
+      ep.channels = cv.co;
+      const int K = cv.ci * 9;
+      if ((e = tc_gemm(net, GatherIm2col<3>{view(net, P.in, 0, cv.ci)}, packed_of(net, 0, 0), TStoreOp{ep},
+                       N * cv.H * cv.W, cv.co, K, K))) return e;
+      ++li;
+    } else {
+      if ((e = conv_into(net->aop[P.pool[l - 1]], P.a1[l], 0, 9, 1, nullptr, 0))) return e;
+    }
+    if ((e = conv_into(net->aop[P.a1[l]], P.cat[l], up, 9, 1, net->act[P.cat[l]], c))) return e;
+    const conv::Op& o = net->aop[P.pool[l]];
+    conv::pool_op_kernel<<<op_grid((long long)N * o.H * o.W, c / 8), 128, 0, net->stream>>>(net->act[P.cat[l]], c, 0, N, o);
+  }
+  if ((e = conv_into(net->aop[P.pool[L - 2]], P.b1, 0, 9, 1, nullptr, 0))) return e;
+  if ((e = conv_into(net->aop[P.b1], P.b2, 0, 9, 1, nullptr, 0))) return e;
+  int prev = P.b2;
+  for (int l = L - 2; l >= 0; --l) {
+    const conv::Op& in = net->aop[prev];
+    conv::up_op_kernel<<<op_grid((long long)N * in.H * in.W, in.C / 8), 128, 0, net->stream>>>(in, N, net->aop[P.cat[l]]);
+    if ((e = conv_into(net->aop[P.cat[l]], P.d1[l], 0, 9, 1, nullptr, 0))) return e;
+    if ((e = conv_into(net->aop[P.d1[l]], P.d2[l], 0, 9, 1, nullptr, 0))) return e;
+    prev = P.d2[l];
+  }
+  if ((e = conv_into(net->aop[prev], P.out, 0, 1, 0, net->act[P.out], net->cfg.out_ch))) return e;
+  return cudaGetLastError();
+}
+
+// backward() on operands: every gradient is stored once, complete.
+cudaError_t backward_direct(clbm_net* net, const Plan& P, int N) {
+  const int L = net->cfg.levels, B = net->cfg.base;
+  cudaError_t e;
+  int li = (int)net->convs.size() - 1;
+  // the epilogue of a gradient that the ReLU of `id` masks: operand and FP32 copies
+  auto masked = [&](int id) {
+    conv::Epilogue ep{};
+    ep.mask = net->aop[id];
+    ep.op = net->gop[id];
+    ep.f32 = net->gact[id];
+    ep.cs = net->act_c[id];
+    ep.H = ep.W = net->act_hw[id];
+    ep.N = N;
+    ep.channels = net->act_c[id];
+    return ep;
+  };
+  auto plain = [&](int id) {  // FP32 only
+    conv::Epilogue ep{};
+    ep.f32 = net->gact[id];
+    ep.cs = net->act_c[id];
+    return ep;
+  };
+  auto grad = [&](int id) { return view(net, id, 0, net->act_c[id], true); };
+  {  // head (1x1): its input gradient has K = out_ch, the gathering GEMM
+    const Conv& cv = net->convs[li];
+    const conv::Op& o = net->gop[P.out];
+    conv::to_op_kernel<<<op_grid((long long)N * o.H * o.W, 1), 128, 0, net->stream>>>(net->gact[P.out], cv.co, N, o);
+    const conv::Op& in = net->aop[P.in];
+    conv::to_op_kernel<<<op_grid((long long)N * o.H * o.W, 1), 128, 0, net->stream>>>(net->act[P.in], net->cfg.in_ch, N, in);
+    if ((e = tc_gemm(net, GatherIm2col<1>{grad(P.out)}, packed_of(net, li, 1), TStoreOp{masked(P.d2[0])},
+                     N * cv.H * cv.W, cv.ci, cv.co, cv.co))) return e;
+    if ((e = dw_direct(net, cv, net->aop[P.d2[0]], o, grad(P.out), N))) return e;
+    --li;
+  }
+  for (int l = 0; l <= L - 2; ++l) {
+    const int c2 = li--, c1 = li--;
+    if ((e = conv_direct(net, net->gop[P.d2[l]], c2, 1, 9, N, masked(P.d1[l])))) return e;
+    if ((e = conv_direct(net, net->gop[P.d1[l]], c1, 1, 9, N, plain(P.cat[l])))) return e;
+    const int below = l + 1 <= L - 2 ? P.d2[l + 1] : P.b2;
+    const conv::Epilogue ep = masked(below);
+    conv::up_back_op_kernel<<<op_grid((long long)N * ep.H * ep.W, ep.channels / 8), 128, 0, net->stream>>>(
+        net->gact[P.cat[l]], net->act_c[P.cat[l]], 0, ep);
+    if ((e = dw_direct(net, net->convs[c2], net->aop[P.d1[l]], net->gop[P.d2[l]], grad(P.d2[l]), N))) return e;
+    if ((e = dw_direct(net, net->convs[c1], net->aop[P.cat[l]], net->gop[P.d1[l]], grad(P.d1[l]), N))) return e;
+  }
+  {  // bottleneck
+    const int c2 = li--, c1 = li--;
+    if ((e = conv_direct(net, net->gop[P.b2], c2, 1, 9, N, masked(P.b1)))) return e;
+    if ((e = conv_direct(net, net->gop[P.b1], c1, 1, 9, N, plain(P.pool[L - 2])))) return e;
+    if ((e = dw_direct(net, net->convs[c2], net->aop[P.b1], net->gop[P.b2], grad(P.b2), N))) return e;
+    if ((e = dw_direct(net, net->convs[c1], net->aop[P.pool[L - 2]], net->gop[P.b1], grad(P.b1), N))) return e;
+  }
+  for (int l = L - 2; l >= 0; --l) {
+    const int c = B << l, cup = B << (l + 1), cat = P.cat[l];
+    const int c2 = li--, c1 = li--;
+    // the skip connection's gradient: from the decoder (in gact[cat]) and through the pooling
+    conv::Epilogue ep{};
+    ep.mask = net->aop[cat];
+    ep.mask_group = cup / 8;
+    ep.op = net->gop[cat];
+    ep.f32 = net->gact[cat];
+    ep.cs = cup + c;
+    ep.coff = cup;
+    ep.H = ep.W = net->act_hw[cat];
+    ep.N = N;
+    ep.channels = c;
+    conv::pool_back_op_kernel<<<op_grid((long long)N * ep.H * ep.W, c / 8), 128, 0, net->stream>>>(
+        net->gact[cat], cup + c, cup, net->gact[P.pool[l]], c, ep);
+    if ((e = conv_direct(net, net->gop[cat], c2, 1, 9, N, masked(P.a1[l])))) return e;
+    if (l > 0)
+      if ((e = conv_direct(net, net->gop[P.a1[l]], c1, 1, 9, N, plain(P.pool[l - 1])))) return e;
+    if ((e = dw_direct(net, net->convs[c2], net->aop[P.a1[l]], net->gop[cat], view(net, cat, cup, c, true), N))) return e;
+    if ((e = dw_direct(net, net->convs[c1], net->aop[l > 0 ? P.pool[l - 1] : P.in], net->gop[P.a1[l]], grad(P.a1[l]), N))) return e;
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t conv_forward(clbm_net* net, const Conv& cv, Act x, int out_id, int out_coff, int relu,
                          int N) {
   const int M = cv.co, Kd = cv.ci * cv.ks * cv.ks, Np = N * cv.H * cv.W;
@@ -923,6 +1215,7 @@ cudaError_t conv_backward(clbm_net* net, const Conv& cv, Act x, Act gy, int gx_i
 
 // Full forward pass over N samples already in act[in].
 cudaError_t forward(clbm_net* net, const Plan& P, int N) {
+  if (net->direct) return forward_direct(net, P, N);
   const int L = net->cfg.levels, B = net->cfg.base;
   cudaError_t e;
   int ci = 0;
@@ -954,6 +1247,7 @@ cudaError_t forward(clbm_net* net, const Plan& P, int N) {
 
 // Backward pass; gact[out] holds dloss/dout on entry; writes net->g.
 cudaError_t backward(clbm_net* net, const Plan& P, int N) {
+  if (net->direct) return backward_direct(net, P, N);
   const int L = net->cfg.levels, B = net->cfg.base;
   cudaError_t e;
   // zero all activation gradients except the output's
@@ -1079,6 +1373,68 @@ double u01(uint64_t& s) {
   return (double)(z >> 11) * (1.0 / 9007199254740992.0);
 }
 
+// Whether every inner convolution of a network can read operand tensors: widths that are
+// multiples of eight, tiles that fit shared memory.
+bool direct_fits(const std::vector<Conv>& convs, const clbm_net_config& c) {
+  if (c.base % 8 != 0 || c.in_ch > 8 || c.out_ch > 8) return false;
+  for (const Conv& cv : convs) {
+    const int taps = cv.ks * cv.ks;
+    if (cv.ci % 8 == 0 && !conv_stages(cv.ci, taps, cv.W, tc::tile_n(cv.co))) return false;
+    if (cv.co % 8 == 0 && !conv_stages(cv.co, taps, cv.W, tc::tile_n(cv.ci))) return false;
+    conv::Op x{};
+    x.C = (cv.ci + 7) / 8 * 8;
+    x.H = x.W = cv.H;
+    if (dw_shape(152, x, (cv.co + 7) / 8, taps, 1).smem > kMaxSmem) return false;
+    if ((long long)c.max_batch * x.Pn() >= (1LL << 31) - 65536) return false;
+  }
+  return true;
+}
+
+// The operand tensors, zeroed once: borders and guards stay zero.
+cudaError_t make_operands(clbm_net* n) {
+  const Plan& P = n->plan;
+  const int L = n->cfg.levels;
+  n->aop.assign(n->act_c.size(), conv::Op{});
+  n->gop.assign(n->act_c.size(), conv::Op{});
+  auto make = [&](conv::Op& o, int C, int hw) {
+    o.C = (C + 7) / 8 * 8;
+    o.H = o.W = hw;
+    // guards: a tile reads Wp + 1 positions before position 0 and past its 128 positions
+    const long long front = o.Wp() + 8, tail = o.Wp() + 8 + tc::kBM;
+    o.pst = front + (long long)n->cfg.max_batch * o.Pn() + tail;
+    const size_t bytes = (size_t)(o.C / 8) * o.pst * 16;
+    void* m = nullptr;
+    cudaError_t e = cudaMalloc(&m, bytes);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e;
+    }
+    n->op_mem.push_back(m);
+    o.base = static_cast<__nv_bfloat16*>(m) + front * 8;
+    return cudaMemsetAsync(m, 0, bytes, n->stream);
+  };
+  cudaError_t e = cudaSuccess;
+  auto both = [&](int id) {
+    if (!e) e = make(n->aop[id], n->act_c[id], n->act_hw[id]);
+    if (!e) e = make(n->gop[id], n->act_c[id], n->act_hw[id]);
+  };
+  if (!e) e = make(n->aop[P.in], n->act_c[P.in], n->act_hw[P.in]);
+  if (!e) e = make(n->gop[P.out], n->act_c[P.out], n->act_hw[P.out]);
+  for (int l = 0; l < L - 1; ++l) {
+    both(P.a1[l]);
+    both(P.d1[l]);
+    both(P.d2[l]);
+    if (!e) e = make(n->aop[P.pool[l]], n->act_c[P.pool[l]], n->act_hw[P.pool[l]]);
+    if (!e) e = make(n->aop[P.cat[l]], n->act_c[P.cat[l]], n->act_hw[P.cat[l]]);
+    if (!e) e = make(n->gop[P.cat[l]], n->cfg.base << l, n->act_hw[P.cat[l]]);  // the skip part
+  }
+  both(P.b1);
+  both(P.b2);
+  if (!e) e = cudaFuncSetAttribute(conv::conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  if (!e) e = cudaFuncSetAttribute(conv::dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  return e;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1096,6 +1452,7 @@ clbm_status clbm_net_destroy(clbm_net* n) {
   cudaFree(n->pt);
   for (float* a : n->act) cudaFree(a);
   for (float* a : n->gact) cudaFree(a);
+  for (void* a : n->op_mem) cudaFree(a);
   cudaFree(n->part);
   cudaFree(n->loss_part);
   if (n->grad_pass.exec) cudaGraphExecDestroy(n->grad_pass.exec);
@@ -1171,6 +1528,7 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
   cudaMemset(n->v, 0, off * sizeof(float));
   cudaMemset(n->g, 0, off * sizeof(float));
   to_bf16_kernel<<<grid1(off), 256, 0, n->stream>>>(n->p, n->pb, off);
+  n->direct = c.math == CLBM_NET_TENSOR && direct_fits(n->convs, c);
   if (c.math == CLBM_NET_TENSOR) {
     long long total = 0;
     for (const Conv& cv : n->convs)
@@ -1186,6 +1544,8 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
         d.K = (tr ? cv.co : cv.ci) * d.kk;
         d.bn = tc::tile_n(d.N);
         d.slices = (d.K + tc::kBK - 1) / tc::kBK;
+        // operand-layout convolutions read K in their own chunk order
+        d.groups = n->direct && (tr ? cv.co : cv.ci) % 8 == 0 ? (tr ? cv.co : cv.ci) / 8 : 0;
         d.size = (long long)((d.N + d.bn - 1) / d.bn) * d.slices * d.bn * tc::kBK;
         total += (d.size + 63) / 64 * 64;  // keep every layer's tiles 128-byte aligned
         n->packed_max = std::max(n->packed_max, d.size);
@@ -1202,13 +1562,18 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
   for (size_t id = 0; id < n->act_c.size(); ++id) {
     const long long e = (long long)c.max_batch * n->act_c[id] * n->act_hw[id] * n->act_hw[id];
     float *a = nullptr, *ga = nullptr;
-    if (cudaMalloc(&a, e * sizeof(float)) || cudaMalloc(&ga, e * sizeof(float))) {
+    // operand-layout networks keep FP32 activations of the input, the skip connections and the output only
+    const std::vector<int> cats(n->plan.cat, n->plan.cat + L - 1);
+    const bool keep = !n->direct || (int)id == n->plan.in || (int)id == n->plan.out ||
+                      std::find(cats.begin(), cats.end(), (int)id) != cats.end();
+    if ((keep && cudaMalloc(&a, e * sizeof(float))) || cudaMalloc(&ga, e * sizeof(float))) {
       cudaFree(a);
       return bail(CLBM_ENOMEM);
     }
     n->act.push_back(a);
     n->gact.push_back(ga);
   }
+  if (n->direct && make_operands(n) != cudaSuccess) return bail(CLBM_ENOMEM);
   {  // one wave of CTAs is sized from the device's multiprocessor count
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -1224,6 +1589,16 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
       const long long kper = dw_kper(n->sms, c.math == CLBM_NET_TENSOR, Np, Kd, cv.co);
       cap = std::max(cap, ((Np + kper - 1) / kper) * cv.co * Kd);
       cap = std::max(cap, ((Np + kBiasChunk - 1) / kBiasChunk) * cv.co);  // bias chunk sums
+      if (n->direct) {
+        conv::Op x{};
+        x.C = (cv.ci + 7) / 8 * 8;
+        x.H = x.W = cv.H;
+        const DwShape s = dw_shape(n->sms, x, (cv.co + 7) / 8, cv.ks * cv.ks, (int)nb);
+        cap = std::max(cap, (long long)s.ranges * cv.co * Kd);
+        const long long Mst = split_stride(x, (int)nb);
+        cap = std::max(cap, conv_ranges(n->sms, (int)Np, cv.co, Kd).splits * Mst * cv.co);
+        cap = std::max(cap, conv_ranges(n->sms, (int)Np, cv.ci, cv.co * cv.ks * cv.ks).splits * Mst * cv.ci);
+      }
       if (c.math == CLBM_NET_TENSOR) {  // split-K forward and input-gradient GEMMs
         cap = std::max(cap, (long long)conv_splits(n->sms, (int)Np, cv.co, Kd) * Np * cv.co);
         cap = std::max(cap, (long long)conv_splits(n->sms, (int)Np, cv.ci, cv.co * cv.ks * cv.ks) * Np * cv.ci);

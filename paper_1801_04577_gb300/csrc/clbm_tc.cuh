@@ -210,7 +210,8 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 
 // D tile (blockIdx.x over M in 128-row tiles, blockIdx.y over N in bn-column
 // tiles, blockIdx.z over K in kper-long ranges, kper a multiple of 64 when
-// there is more than one range); st(m, n, value, split).  A is gathered by all
+// there is more than one range); st(m, n, value, split), or st.row(m, n,
+// sixteen values) where ST::kRow.  A is gathered by all
 // threads; B is gathered too, or (GB::kBulk) bulk-copied by thread 0 from a
 // Packed buffer into the stage, completing on the stage's load barrier.
 // Launch with kThreads threads and smem_bytes(bn) bytes of dynamic shared memory.
@@ -301,9 +302,13 @@ __global__ void __launch_bounds__(kThreads) gemm_kernel(GA ga, GB gb, ST st, int
         for (int j = 0; j < 16; ++j) v[j] = 0.0f;
       }
       if (r < mvalid) {
+        if constexpr (ST::kRow) {
+          st.row(m, n0 + c0, v);
+        } else {
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (c0 + j < nvalid) st(m, n0 + c0 + j, v[j], (int)blockIdx.z);
+          for (int j = 0; j < 16; ++j)
+            if (c0 + j < nvalid) st(m, n0 + c0 + j, v[j], (int)blockIdx.z);
+        }
       }
     }
   }
