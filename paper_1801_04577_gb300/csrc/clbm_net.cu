@@ -763,6 +763,13 @@ struct clbm_net {
   bool direct = false;
   std::vector<conv::Op> aop, gop;
   std::vector<void*> op_mem;
+  // Weight gradients run beside the chain of input gradients on streams of their own (branches of
+  // the captured graph), each layer with its own partial sums.
+  static constexpr int kSides = 3;
+  cudaStream_t side[kSides] = {};
+  std::vector<cudaEvent_t> events;
+  std::vector<long long> dw_off, bias_off;  // per layer, in dw_part
+  float* dw_part = nullptr;
   double* h_loss = nullptr;  // page-locked copy of the loss partials and mask sums
   float *tgt = nullptr, *msk = nullptr;  // the caller's target and mask, copied in before a pass
 };
@@ -955,7 +962,7 @@ DwShape dw_shape(int sms, const conv::Op& x, int co_groups, int taps, int N) {
     if (s.group_set == 1 || conv::dw_smem(std::min(16, co_groups), s.group_set, taps, x.W + 2, 2) <= kMaxSmem) break;
   }
   const int cols = conv::dw_cols(s.group_set);
-  s.tap_set = std::min(taps, 512 / cols);
+  s.tap_set = std::min(taps, 256 / cols);  // half of the tensor memory: two blocks, or a convolution beside
   s.tap_sets = (taps + s.tap_set - 1) / s.tap_set;
   s.tap_set = (taps + s.tap_sets - 1) / s.tap_sets;
   s.mtiles = (co_groups + 15) / 16;
@@ -964,9 +971,9 @@ DwShape dw_shape(int sms, const conv::Op& x, int co_groups, int taps, int N) {
     s.smem = conv::dw_smem(gg, s.group_set, taps, x.W + 2, s.stages);
     if (s.smem <= kMaxSmem / 2 || (s.stages == 2 && s.smem <= kMaxSmem)) break;
   }
-  // about one block per multiprocessor, at least two stages of positions each
+  // about two blocks per multiprocessor, at least two stages of positions each
   const long long K = (long long)N * x.Pn(), per_range = (long long)s.group_sets * s.tap_sets * s.mtiles;
-  const long long want = std::max<long long>(1, (sms + per_range - 1) / per_range);
+  const long long want = std::max<long long>(1, (2LL * sms + per_range - 1) / per_range);
   const long long most = std::max<long long>(1, K / (2 * conv::kKP));
   const long long r = std::min(want, most);
   s.kper = (int)(((K + r - 1) / r + conv::kKP - 1) / conv::kKP * conv::kKP);
@@ -974,10 +981,14 @@ DwShape dw_shape(int sms, const conv::Op& x, int co_groups, int taps, int N) {
   return s;
 }
 
-// dW, db of a layer from its input operand x and output gradient operand g (and FP32 view gy).
-cudaError_t dw_direct(clbm_net* net, const Conv& cv, const conv::Op& x, const conv::Op& g, Act gy, int N) {
+// dW, db of a layer from its input operand x and output gradient operand g (and FP32 view gy), on
+// stream st.
+cudaError_t dw_direct(clbm_net* net, const Conv& cv, const conv::Op& x, const conv::Op& g, Act gy, int N,
+                      cudaStream_t st) {
   const int taps = cv.ks * cv.ks;
   const DwShape s = dw_shape(net->sms, x, g.C / 8, taps, N);
+  float* part = net->dw_part + net->dw_off[cv.index];
+  float* bpart = net->dw_part + net->bias_off[cv.index];
   conv::DwArgs a{};
   a.x = x;
   a.g = g;
@@ -990,22 +1001,19 @@ cudaError_t dw_direct(clbm_net* net, const Conv& cv, const conv::Op& x, const co
   a.stages = s.stages;
   a.ci = cv.ci;
   a.co = cv.co;
-  a.part = net->part;
+  a.part = part;
   a.err = net->d_tflag;
   const long long n = (long long)taps * cv.ci * cv.co;
-  if (s.ranges * n > net->part_cap) return cudaErrorInvalidValue;
   conv::dw_kernel<<<dim3((unsigned)s.ranges, (unsigned)(s.tap_sets * s.group_sets), (unsigned)s.mtiles),
-                    conv::kThreads, s.smem, net->stream>>>(a);
+                    conv::kThreads, s.smem, st>>>(a);
   const long long want = std::max<long long>(1, (net->sms * 2048LL) / n);
   int R = 1;
   while (2 * R <= std::min(s.ranges, 32) && 2 * R <= want) R *= 2;
-  conv::dw_sum_kernel<<<(unsigned)std::min<long long>((n + 31) / 32, 65535), dim3(32, R), 0, net->stream>>>(
-      net->part, s.ranges, taps, cv.ci, cv.co, net->g + cv.w_off);
-  // bias: the partial sums are consumed, so part holds the chunk sums next
+  conv::dw_sum_kernel<<<(unsigned)std::min<long long>((n + 31) / 32, 65535), dim3(32, R), 0, st>>>(
+      part, s.ranges, taps, cv.ci, cv.co, net->g + cv.w_off);
   const int Np = N * cv.H * cv.W, chunks = (Np + kBiasChunk - 1) / kBiasChunk;
-  if ((long long)chunks * cv.co > net->part_cap) return cudaErrorInvalidValue;
-  bias_partial_kernel<<<dim3(chunks, cv.co), GT, 0, net->stream>>>(gy, N, net->part);
-  sum_splits(net->part, chunks, cv.co, net->g + cv.b_off, net->sms, net->stream);
+  bias_partial_kernel<<<dim3(chunks, cv.co), GT, 0, st>>>(gy, N, bpart);
+  sum_splits(bpart, chunks, cv.co, net->g + cv.b_off, net->sms, st);
   return cudaGetLastError();
 }
 
@@ -1070,6 +1078,15 @@ cudaError_t backward_direct(clbm_net* net, const Plan& P, int N) {
   const int L = net->cfg.levels, B = net->cfg.base;
   cudaError_t e;
   int li = (int)net->convs.size() - 1;
+  // weight gradients on a side stream, after what net->stream holds by now
+  size_t used = 0;
+  auto weights = [&](const Conv& cv, const conv::Op& x, const conv::Op& g, Act gy) {
+    const cudaStream_t st = net->side[used % clbm_net::kSides];
+    cudaError_t er = cudaEventRecord(net->events[used], net->stream);
+    if (!er) er = cudaStreamWaitEvent(st, net->events[used], 0);
+    ++used;
+    return er ? er : dw_direct(net, cv, x, g, gy, N, st);
+  };
   // the epilogue of a gradient that the ReLU of `id` masks: operand and FP32 copies
   auto masked = [&](int id) {
     conv::Epilogue ep{};
@@ -1097,26 +1114,26 @@ cudaError_t backward_direct(clbm_net* net, const Plan& P, int N) {
     conv::to_op_kernel<<<op_grid((long long)N * o.H * o.W, 1), 128, 0, net->stream>>>(net->act[P.in], net->cfg.in_ch, N, in);
     if ((e = tc_gemm(net, GatherIm2col<1>{grad(P.out)}, packed_of(net, li, 1), TStoreOp{masked(P.d2[0])},
                      N * cv.H * cv.W, cv.ci, cv.co, cv.co))) return e;
-    if ((e = dw_direct(net, cv, net->aop[P.d2[0]], o, grad(P.out), N))) return e;
+    if ((e = weights(cv, net->aop[P.d2[0]], o, grad(P.out)))) return e;
     --li;
   }
   for (int l = 0; l <= L - 2; ++l) {
     const int c2 = li--, c1 = li--;
+    if ((e = weights(net->convs[c2], net->aop[P.d1[l]], net->gop[P.d2[l]], grad(P.d2[l])))) return e;
     if ((e = conv_direct(net, net->gop[P.d2[l]], c2, 1, 9, N, masked(P.d1[l])))) return e;
+    if ((e = weights(net->convs[c1], net->aop[P.cat[l]], net->gop[P.d1[l]], grad(P.d1[l])))) return e;
     if ((e = conv_direct(net, net->gop[P.d1[l]], c1, 1, 9, N, plain(P.cat[l])))) return e;
     const int below = l + 1 <= L - 2 ? P.d2[l + 1] : P.b2;
     const conv::Epilogue ep = masked(below);
     conv::up_back_op_kernel<<<op_grid((long long)N * ep.H * ep.W, ep.channels / 8), 128, 0, net->stream>>>(
         net->gact[P.cat[l]], net->act_c[P.cat[l]], 0, ep);
-    if ((e = dw_direct(net, net->convs[c2], net->aop[P.d1[l]], net->gop[P.d2[l]], grad(P.d2[l]), N))) return e;
-    if ((e = dw_direct(net, net->convs[c1], net->aop[P.cat[l]], net->gop[P.d1[l]], grad(P.d1[l]), N))) return e;
   }
   {  // bottleneck
     const int c2 = li--, c1 = li--;
+    if ((e = weights(net->convs[c2], net->aop[P.b1], net->gop[P.b2], grad(P.b2)))) return e;
     if ((e = conv_direct(net, net->gop[P.b2], c2, 1, 9, N, masked(P.b1)))) return e;
+    if ((e = weights(net->convs[c1], net->aop[P.pool[L - 2]], net->gop[P.b1], grad(P.b1)))) return e;
     if ((e = conv_direct(net, net->gop[P.b1], c1, 1, 9, N, plain(P.pool[L - 2])))) return e;
-    if ((e = dw_direct(net, net->convs[c2], net->aop[P.b1], net->gop[P.b2], grad(P.b2), N))) return e;
-    if ((e = dw_direct(net, net->convs[c1], net->aop[P.pool[L - 2]], net->gop[P.b1], grad(P.b1), N))) return e;
   }
   for (int l = L - 2; l >= 0; --l) {
     const int c = B << l, cup = B << (l + 1), cat = P.cat[l];
@@ -1134,11 +1151,15 @@ cudaError_t backward_direct(clbm_net* net, const Plan& P, int N) {
     ep.channels = c;
     conv::pool_back_op_kernel<<<op_grid((long long)N * ep.H * ep.W, c / 8), 128, 0, net->stream>>>(
         net->gact[cat], cup + c, cup, net->gact[P.pool[l]], c, ep);
+    if ((e = weights(net->convs[c2], net->aop[P.a1[l]], net->gop[cat], view(net, cat, cup, c, true)))) return e;
     if ((e = conv_direct(net, net->gop[cat], c2, 1, 9, N, masked(P.a1[l])))) return e;
+    if ((e = weights(net->convs[c1], net->aop[l > 0 ? P.pool[l - 1] : P.in], net->gop[P.a1[l]], grad(P.a1[l])))) return e;
     if (l > 0)
       if ((e = conv_direct(net, net->gop[P.a1[l]], c1, 1, 9, N, plain(P.pool[l - 1])))) return e;
-    if ((e = dw_direct(net, net->convs[c2], net->aop[P.a1[l]], net->gop[cat], view(net, cat, cup, c, true), N))) return e;
-    if ((e = dw_direct(net, net->convs[c1], net->aop[l > 0 ? P.pool[l - 1] : P.in], net->gop[P.a1[l]], grad(P.a1[l]), N))) return e;
+  }
+  for (int k = 0; k < clbm_net::kSides; ++k) {  // join
+    if ((e = cudaEventRecord(net->events[used + k], net->side[k]))) return e;
+    if ((e = cudaStreamWaitEvent(net->stream, net->events[used + k], 0))) return e;
   }
   return cudaGetLastError();
 }
@@ -1453,6 +1474,13 @@ clbm_status clbm_net_destroy(clbm_net* n) {
   for (float* a : n->act) cudaFree(a);
   for (float* a : n->gact) cudaFree(a);
   for (void* a : n->op_mem) cudaFree(a);
+  cudaFree(n->dw_part);
+  for (cudaEvent_t ev : n->events) cudaEventDestroy(ev);
+  for (cudaStream_t st : n->side)
+    if (st) {
+      cudaStreamSynchronize(st);
+      cudaStreamDestroy(st);
+    }
   cudaFree(n->part);
   cudaFree(n->loss_part);
   if (n->grad_pass.exec) cudaGraphExecDestroy(n->grad_pass.exec);
@@ -1581,9 +1609,10 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
       n->sms = sms;
   }
   // split-K partials: enough for the largest batch (fewer pixels never need more splits)
-  long long cap = 0;
+  long long cap = 0, dw_cap = 0;
   for (const Conv& cv : n->convs) {
     const int Kd = cv.ci * cv.ks * cv.ks;
+    long long dw_need = 0, bias_need = 0;
     for (long long nb = 1; nb <= c.max_batch; ++nb) {
       const long long Np = nb * cv.H * cv.W;
       const long long kper = dw_kper(n->sms, c.math == CLBM_NET_TENSOR, Np, Kd, cv.co);
@@ -1594,7 +1623,8 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
         x.C = (cv.ci + 7) / 8 * 8;
         x.H = x.W = cv.H;
         const DwShape s = dw_shape(n->sms, x, (cv.co + 7) / 8, cv.ks * cv.ks, (int)nb);
-        cap = std::max(cap, (long long)s.ranges * cv.co * Kd);
+        dw_need = std::max(dw_need, (long long)s.ranges * cv.co * Kd);
+        bias_need = std::max(bias_need, ((Np + kBiasChunk - 1) / kBiasChunk) * cv.co);
         const long long Mst = split_stride(x, (int)nb);
         cap = std::max(cap, conv_ranges(n->sms, (int)Np, cv.co, Kd).splits * Mst * cv.co);
         cap = std::max(cap, conv_ranges(n->sms, (int)Np, cv.ci, cv.co * cv.ks * cv.ks).splits * Mst * cv.ci);
@@ -1604,8 +1634,20 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
         cap = std::max(cap, (long long)conv_splits(n->sms, (int)Np, cv.ci, cv.co * cv.ks * cv.ks) * Np * cv.ci);
       }
     }
+    n->dw_off.push_back(dw_cap);
+    dw_cap += (dw_need + 63) / 64 * 64;
+    n->bias_off.push_back(dw_cap);
+    dw_cap += (bias_need + 63) / 64 * 64;
   }
   n->part_cap = cap;
+  if (n->direct) {
+    if (cudaMalloc(&n->dw_part, dw_cap * sizeof(float))) return bail(CLBM_ENOMEM);
+    for (cudaStream_t& st : n->side)
+      if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return bail(CLBM_ECUDA);
+    n->events.resize(n->convs.size() + clbm_net::kSides, nullptr);
+    for (cudaEvent_t& ev : n->events)
+      if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) return bail(CLBM_ECUDA);
+  }
   if (cudaHostAlloc(&n->tflag, sizeof(int), cudaHostAllocMapped) != cudaSuccess) return bail(CLBM_ENOMEM);
   *n->tflag = 0;
   if (cudaHostGetDevicePointer(&n->d_tflag, n->tflag, 0) != cudaSuccess) return bail(CLBM_ECUDA);
