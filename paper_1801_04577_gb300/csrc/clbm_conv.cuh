@@ -107,21 +107,25 @@ struct Epilogue {
 
 struct ConvArgs {
   Op a;              // input operand, channel groups [0, a.C / 8)
-  const bf16* w;     // packed weights: [N tile][slice][bn x 64], chunk order of first_chunk
+  const bf16* w;     // packed weights: [N tile][slice][bn x 64], chunk order of pair_swapped
   int taps, bn, slices;
-  int kper;          // slices per split (blockIdx.z)
+  int kper, ranges;  // slices per range of K, ranges
   int stages;
-  int M;             // positions
-  float* part;       // partial sums [split][channel][Mst] when split, else nullptr
-  long long Mst;
   Epilogue epi;
   int* err;
 };
 
-constexpr int kThreads = 128;
+// Programmatic dependent launch: a kernel of the chain may start while its
+// predecessor runs; pdl_wait() returns when the predecessor's writes are
+// visible, pdl_go() lets the successor start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+constexpr int kMaxBn = 64;         // columns of a tile: a thread keeps its row's sums in registers
+constexpr int kConvThreads = 192;  // four epilogue warps, one for the copies, one for the MMAs
 
 __host__ __device__ constexpr int conv_run(int taps, int Wp) { return tc::kBM + (taps == 9 ? 2 * Wp + 2 : 0); }
-// pairs of K chunks (the MMAs) of one K range, rounded up to whole slices
+// pairs of K chunks (the MMAs), rounded up to whole slices
 __host__ __device__ constexpr int conv_pairs(int C, int taps) { return (taps * C / 8 + 7) / 8 * 4; }
 __host__ __device__ constexpr int conv_smem(int C, int taps, int Wp, int bn, int stages) {
   return (C / 8) * conv_run(taps, Wp) * 16 + stages * bn * 128 + conv_pairs(C, taps) * 8 + bn * 4 + 256;
@@ -136,13 +140,18 @@ __host__ __device__ __forceinline__ bool pair_swapped(int u, int groups, int tot
   return groups > 1 ? u % groups == groups - 1 : u + 1 == total && u > 0;
 }
 
-// Implicit GEMM D[position][channel] of one 128-position tile (blockIdx.x), bn
-// channels (blockIdx.y) and one range of K (blockIdx.z).  Warp 0 issues the
-// copies, warp 1 the MMAs, all four warps the epilogue.  The matrix
-// descriptors are made beforehand by all threads: one thread that divided by
-// the number of channel groups for every MMA took 20 us a tile.  Launch with
-// conv_smem() bytes of dynamic shared memory.
-__global__ void __launch_bounds__(kThreads) conv_kernel(const __grid_constant__ ConvArgs a) {
+// Implicit GEMM D[position][channel] of one 128-position tile (blockIdx.x) and
+// bn channels (blockIdx.y).  Warp 4 issues the copies, warp 5 the MMAs, warps
+// 0-3 the epilogue.  The matrix descriptors are made beforehand by all
+// threads: one thread that divided by the number of channel groups for every
+// MMA took 20 us a tile.
+//
+// K is summed in ranges, each into an accumulator of its own (two, in turn),
+// and the ranges' sums are added in order in registers: the order of a split-K
+// GEMM whose partial sums are added by a second kernel, without that kernel
+// (94 us for the 384 -> 128 convolution at 16^2, 12 us so).
+// Launch with conv_smem() bytes of dynamic shared memory.
+__global__ void __launch_bounds__(kConvThreads) conv_kernel(const __grid_constant__ ConvArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int groups = a.a.C / 8, Wp = a.a.W + 2;
@@ -153,17 +162,20 @@ __global__ void __launch_bounds__(kThreads) conv_kernel(const __grid_constant__ 
   uint64_t* bar_a = desc + conv_pairs(a.a.C, a.taps);
   uint64_t* bar_b = bar_a + 1;         // [stages] weights have arrived
   uint64_t* bar_m = bar_b + a.stages;  // [stages] MMAs that read the stage are done
-  uint64_t* bar_d = bar_m + a.stages;  // all MMAs are done
-  uint32_t* slot = reinterpret_cast<uint32_t*>(bar_d + 1);
+  uint64_t* bar_d = bar_m + a.stages;  // [2] a range is complete in its accumulator
+  uint64_t* bar_f = bar_d + 2;         // [2] ... and has been read
+  uint32_t* slot = reinterpret_cast<uint32_t*>(bar_f + 2);
   float* bias = reinterpret_cast<float*>(slot + 2);  // [bn]
   const int m0 = blockIdx.x * tc::kBM, n0 = blockIdx.y * a.bn;
-  const int s0 = blockIdx.z * a.kper, s1 = min(a.slices, s0 + a.kper), nk = s1 - s0;
-  const uint32_t ncols = tc::tmem_cols(a.bn);
+  const uint32_t ncols = tc::tmem_cols(a.ranges > 1 ? 2 * a.bn : a.bn);
 
   if (warp == 0) tc::tmem_alloc(slot, ncols);
-  if (tid == 0) {
+  if (tid == 32) {
     tc::mbar_init(bar_a, 1);
-    tc::mbar_init(bar_d, 1);
+    for (int k = 0; k < 2; ++k) {
+      tc::mbar_init(&bar_d[k], 1);
+      tc::mbar_init(&bar_f[k], tc::kBM);
+    }
     for (int s = 0; s < a.stages; ++s) {
       tc::mbar_init(&bar_b[s], 1);
       tc::mbar_init(&bar_m[s], 1);
@@ -175,129 +187,129 @@ __global__ void __launch_bounds__(kThreads) conv_kernel(const __grid_constant__ 
     const int t = c / groups, g = c - t * groups;
     return (uint32_t)((g * run + (a.taps == 9 ? (t / 3) * Wp + t % 3 : 0)) * 16);
   };
-  const int pairs = (min(total, s1 * 8) - s0 * 8 + 1) / 2;
-  for (int j = tid; j < pairs; j += kThreads) {
-    const int u = s0 * 8 + 2 * j;
+  const int pairs = (total + 1) / 2;
+  for (int j = tid; j < pairs; j += kConvThreads) {
+    const int u = 2 * j;
     const bool swap = pair_swapped(u, groups, total);
     const uint32_t lo = swap ? (u + 1 < total ? at(u + 1) : at(u - 1)) : at(u);
     const uint32_t hi = swap ? at(u) : (u + 1 < total ? at(u + 1) : at(u));
     desc[j] = tc::smem_desc(tc::smem_u32(A) + lo, hi - lo, 128);
   }
   if (a.epi.bias)
-    for (int k = tid; k < a.bn; k += kThreads) bias[k] = n0 + k < a.epi.channels ? a.epi.bias[n0 + k] : 0.0f;
+    for (int k = tid; k < a.bn; k += kConvThreads) bias[k] = n0 + k < a.epi.channels ? a.epi.bias[n0 + k] : 0.0f;
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
+  pdl_go();
   const uint32_t tmem = *slot;
   bool failed = false;
-  int issued = 0;  // slices whose copies were started (warp 0)
+  float sum[kMaxBn];
+  int pos = 0, n = 0, p = 0;
+  bool inside = false;
 
-  if (warp == 0) {
-    // the channel groups that this range of K reads (all, unless it is shorter than a tap)
-    const int u0 = s0 * 8, u1 = min(total, s1 * 8);
-    const bool every = u1 - u0 >= groups;
-    const int g0 = u0 % groups;
-    auto needed = [&](int g) {
-      const int d = g - g0 < 0 ? g - g0 + groups : g - g0;
-      return every || d < u1 - u0 || (groups > 1 && g == (u1 - 1) % groups - 1);
+  if (warp == 4) {
+    const bf16* w = a.w + (long long)blockIdx.y * a.slices * a.bn * 64;
+    auto weights = [&](int i) {
+      const int s = i % a.stages;
+      tc::mbar_expect_tx(&bar_b[s], (uint32_t)(a.bn * 128));
+      tc::bulk_load(B + s * a.bn * 128, w + (long long)i * a.bn * 64, (uint32_t)(a.bn * 128), &bar_b[s]);
     };
-    if (lane == 0) {
-      int count = 0;
-      for (int g = 0; g < groups; ++g) count += needed(g) ? 1 : 0;
-      tc::mbar_expect_tx(bar_a, (uint32_t)(count * run * 16));
+    const int first = min(a.stages, a.slices);
+    if (lane == 0) {  // the weights are older than the predecessor, the input is its result
+      tc::mbar_expect_tx(bar_a, (uint32_t)(groups * run * 16));
+      for (int i = 0; i < first; ++i) weights(i);
     }
+    pdl_wait();
     __syncwarp();
     for (int g = lane; g < groups; g += 32)
-      if (needed(g))
-        tc::bulk_load(A + g * run * 16, op_at(a.a, g, (long long)m0 - (a.taps == 9 ? Wp + 1 : 0)), (uint32_t)(run * 16),
-                      bar_a);
+      tc::bulk_load(A + g * run * 16, op_at(a.a, g, (long long)m0 - (a.taps == 9 ? Wp + 1 : 0)), (uint32_t)(run * 16),
+                    bar_a);
     if (lane == 0) {
-      const bf16* w = a.w + ((long long)blockIdx.y * a.slices + s0) * a.bn * 64;
-      for (int i = 0; i < nk; ++i) {
-        const int s = i % a.stages;
-        if (i >= a.stages && !tc::mbar_wait(&bar_m[s], (uint32_t)((i / a.stages - 1) & 1))) {
+      int i = first;
+      for (; i < a.slices; ++i) {
+        if (!tc::mbar_wait(&bar_m[i % a.stages], (uint32_t)((i / a.stages - 1) & 1))) {
           failed = true;
           break;
         }
-        tc::mbar_expect_tx(&bar_b[s], (uint32_t)(a.bn * 128));
-        tc::bulk_load(B + s * a.bn * 128, w + (long long)i * a.bn * 64, (uint32_t)(a.bn * 128), &bar_b[s]);
-        issued = i + 1;
+        weights(i);
+      }
+      if (failed) {  // the copies in flight end before the block does (bounded)
+        tc::mbar_wait(bar_a, 0);
+        for (int k = max(0, i - a.stages); k < i; ++k)
+          tc::mbar_wait(&bar_b[k % a.stages], (uint32_t)((k / a.stages) & 1));
       }
     }
-  } else if (tid == 32) {
-    const uint32_t idesc = tc::idesc_bf16_f32(tc::kBM, a.bn);
-    failed = !tc::mbar_wait(bar_a, 0);
-    for (int i = 0; i < nk && !failed; ++i) {
-      const int s = i % a.stages;
-      if (!tc::mbar_wait(&bar_b[s], (uint32_t)((i / a.stages) & 1))) {
+  } else if (warp == 5) {
+    if (lane == 0) {
+      const uint32_t idesc = tc::idesc_bf16_f32(tc::kBM, a.bn);
+      failed = !tc::mbar_wait(bar_a, 0);
+      int i = 0;
+      for (int z = 0; z < a.ranges && !failed; ++z) {
+        const uint32_t acc = tmem + (z & 1) * a.bn;
+        if (z >= 2) {
+          failed = !tc::mbar_wait(&bar_f[z & 1], (uint32_t)((z / 2 - 1) & 1));
+          tc::fence_after();
+        }
+        const int s1 = min(a.slices, (z + 1) * a.kper), s0 = i;
+        for (; i < s1 && !failed; ++i) {
+          const int s = i % a.stages;
+          if (!tc::mbar_wait(&bar_b[s], (uint32_t)((i / a.stages) & 1))) {
+            failed = true;
+            break;
+          }
+          tc::fence_after();
+          const uint64_t bdesc = tc::smem_desc(tc::smem_u32(B) + s * a.bn * 128, 128, 1024);
+          const int m = min(4, pairs - 4 * i);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (j < m) tc::mma_bf16(acc, desc[4 * i + j], bdesc + j * 16, idesc, (i > s0 || j > 0) ? 1u : 0u);
+          tc::mma_commit(&bar_m[s]);
+        }
+        tc::mma_commit(&bar_d[z & 1]);
+      }
+      // after a failure the other warps still wait for every range: let them time out on their own
+    }
+  } else {
+    pos = m0 + tid;
+    inside = a.epi.locate(pos, n, p);
+#pragma unroll
+    for (int c = 0; c < kMaxBn; ++c) sum[c] = 0.0f;
+    for (int z = 0; z < a.ranges; ++z) {
+      if (!tc::mbar_wait(&bar_d[z & 1], (uint32_t)((z / 2) & 1))) {
         failed = true;
         break;
       }
       tc::fence_after();
-      const uint64_t bdesc = tc::smem_desc(tc::smem_u32(B) + s * a.bn * 128, 128, 1024);
-      const int n = min(4, pairs - 4 * i);
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (j < n) tc::mma_bf16(tmem, desc[4 * i + j], bdesc + j * 16, idesc, (i > 0 || j > 0) ? 1u : 0u);
-      tc::mma_commit(&bar_m[s]);
+      for (int c0 = 0; c0 < kMaxBn; c0 += 16) {
+        if (c0 >= a.bn) break;
+        float v[16];
+        tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((z & 1) * a.bn + c0), v);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) sum[c0 + k] += v[k];
+      }
+      tc::fence_before();
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&bar_f[z & 1])) : "memory");
     }
-    tc::mma_commit(bar_d);
   }
-  const bool done = tc::mbar_wait(bar_d, 0);
-  if (__syncthreads_or(failed || !done)) {
-    if (tid == 0) {  // the copies in flight end before the block does (bounded)
-      atomicExch(a.err, 1);
-      tc::mbar_wait(bar_a, 0);
-      for (int i = max(0, issued - a.stages); i < issued; ++i)
-        tc::mbar_wait(&bar_b[i % a.stages], (uint32_t)((i / a.stages) & 1));
-    }
-  } else {
-    tc::fence_after();
-    const int pos = m0 + warp * 32 + lane;
-    int n = 0, p = 0;
-    const bool inside = a.epi.locate(pos, n, p);
-    for (int c0 = 0; c0 < a.bn; c0 += 16) {
-      float v[16];
-      tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-      if (!inside) continue;
+  if (__syncthreads_or(failed)) {
+    if (tid == 0) atomicExch(a.err, 1);
+  } else if (warp < 4) {
+    pdl_wait();
+    if (inside) {
 #pragma unroll
-      for (int h = 0; h < 16; h += 8) {
-        if (n0 + c0 + h >= a.epi.channels) continue;
+      for (int h = 0; h < kMaxBn; h += 8) {
+        if (h >= a.bn || n0 + h >= a.epi.channels) break;
         float x[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] = v[h + k];
-        if (a.part) {
-          float* o = a.part + ((long long)blockIdx.z * a.epi.channels + n0 + c0 + h) * a.Mst + pos;
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            if (n0 + c0 + h + k < a.epi.channels) o[k * a.Mst] = x[k];
-        } else {
-          a.epi.apply(pos, n, p, n0 + c0 + h, x, bias + c0 + h);
-        }
+        for (int k = 0; k < 8; ++k) x[k] = sum[h + k];
+        a.epi.apply(pos, n, p, n0 + h, x, bias + h);
       }
     }
   }
   tc::fence_before();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, ncols);
-}
-
-// The sums of a split convolution in order of the splits, then its epilogue:
-// one thread per position and eight channels.
-__global__ void conv_finish_kernel(const float* __restrict__ part, int splits, int M, long long Mst, Epilogue e) {
-  for (int pos = blockIdx.x * blockDim.x + threadIdx.x; pos < M; pos += gridDim.x * blockDim.x) {
-    int n, p;
-    if (!e.locate(pos, n, p)) continue;
-    const int n0 = blockIdx.y * 8;
-    float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int z = 0; z < splits; ++z) {
-      const float* s = part + ((long long)z * e.channels + n0) * Mst + pos;
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (n0 + k < e.channels) v[k] += s[k * Mst];
-    }
-    e.apply(pos, n, p, n0, v, e.bias + n0);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -310,6 +322,7 @@ __global__ void conv_finish_kernel(const float* __restrict__ part, int splits, i
 // part[range][tap C + c][o].
 // ---------------------------------------------------------------------------
 constexpr int kKP = 128;  // positions per stage
+constexpr int kThreads = 128;
 
 struct DwArgs {
   Op x, g;
@@ -469,7 +482,8 @@ __global__ void dw_sum_kernel(const float* __restrict__ part, int splits, int ta
 
 // ---------------------------------------------------------------------------
 // Element-wise passes in operand layout: one thread per position of the
-// smaller image and eight channels (blockIdx.y = channel group).
+// smaller image and eight channels (blockIdx.y = channel group).  All of the
+// chain are launched as programmatic dependents.
 // ---------------------------------------------------------------------------
 
 // FP32 NCHW (cs channels, C <= 8 of them from coff) -> one channel group, zero beyond C
@@ -486,6 +500,8 @@ __global__ void to_op_kernel(const float* __restrict__ x, int C, int N, Op o) {
 
 // 2x2 average of an FP32 NCHW view into the operand of the next level
 __global__ void pool_op_kernel(const float* __restrict__ in, int cs, int coff, int N, Op o) {
+  pdl_go();
+  pdl_wait();
   const int W2 = o.W * 2, hw2 = 4 * o.H * o.W, hw = o.H * o.W, g = blockIdx.y;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N * hw; i += gridDim.x * blockDim.x) {
     const int n = i / hw, p = i - n * hw, y = p / o.W, x = p - y * o.W;
@@ -503,6 +519,8 @@ __global__ void pool_op_kernel(const float* __restrict__ in, int cs, int coff, i
 
 // nearest 2x upsampling of an operand into channel groups [0, in.C / 8) of another
 __global__ void up_op_kernel(Op in, int N, Op o) {
+  pdl_go();
+  pdl_wait();
   const int hw = in.H * in.W, g = blockIdx.y;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N * hw; i += gridDim.x * blockDim.x) {
     const int n = i / hw, p = i - n * hw, y = p / in.W, x = p - y * in.W;
@@ -518,6 +536,8 @@ __global__ void up_op_kernel(Op in, int N, Op o) {
 // Gradient of the upsampling: the sum of four values of an FP32 NCHW view (in), then the epilogue
 // (ReLU backward, operand and FP32 copies)
 __global__ void up_back_op_kernel(const float* __restrict__ in, int cs, int coff, Epilogue e) {
+  pdl_go();
+  pdl_wait();
   const int W2 = e.W * 2, hw2 = 4 * e.H * e.W, hw = e.H * e.W, g = blockIdx.y;
   const int Wp = e.W + 2, Pn = ((e.H + 2) * Wp + 15) / 16 * 16;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < e.N * hw; i += gridDim.x * blockDim.x) {
@@ -538,6 +558,8 @@ __global__ void up_back_op_kernel(const float* __restrict__ in, int cs, int coff
 // of the larger image
 __global__ void pool_back_op_kernel(const float* __restrict__ in, int cs, int coff, const float* __restrict__ pooled,
                                     int pcs, Epilogue e) {
+  pdl_go();
+  pdl_wait();
   const int hw = e.H * e.W, Wo = e.W / 2, ho = (e.H / 2) * Wo, g = blockIdx.y;
   const int Wp = e.W + 2, Pn = ((e.H + 2) * Wp + 15) / 16 * 16;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < e.N * hw; i += gridDim.x * blockDim.x) {

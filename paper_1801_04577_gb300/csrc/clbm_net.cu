@@ -211,6 +211,41 @@ struct GatherIm2col {
   }
 };
 
+// The same 3x3 gather for C < 8 input channels (the first layer; K = 9 C fits
+// one slice): every tap and channel unrolled, so that all loads of a row are
+// in flight and no index is computed per element.
+template <int C>
+struct GatherFirst {
+  static constexpr bool kBulk = false;
+  Act x;
+  __device__ __forceinline__ void operator()(uint8_t* dst, int row0, int rows_valid, int, int, int) const {
+    static_assert(9 * C <= tc::kBK, "one slice of K");
+    const int r = threadIdx.x, hw = x.H * x.W;
+    const bool rv = r < rows_valid;
+    const int m = rv ? row0 + r : 0;
+    const int nb = m / hw, p = m - nb * hw, yy = p / x.W, xx = p - yy * x.W;
+    const float* src = x.base + (long long)nb * x.cs * hw + p;
+    float v[tc::kBK];
+#pragma unroll
+    for (int k = 0; k < tc::kBK; ++k) v[k] = 0.0f;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      const int dy = t / 3 - 1, dx = t % 3 - 1;
+      const bool ok = rv && yy + dy >= 0 && yy + dy < x.H && xx + dx >= 0 && xx + dx < x.W;
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+        if (ok) v[t * C + c] = __ldg(src + c * hw + dy * x.W + dx);
+    }
+#pragma unroll
+    for (int kc = 0; kc < tc::kBK / 8; ++kc) {
+      float u[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) u[k] = v[8 * kc + k];
+      put_chunk(dst, r, kc, u);
+    }
+  }
+};
+
 // A(m = (channel, tap), k = pixel) = x[channel] at pixel + tap offset: eight
 // consecutive threads gather the 64 pixels of one row, 8 each.
 template <int KS>
@@ -894,6 +929,16 @@ long long dw_kper(int sms, bool tensor, long long Np, int Kd, int co) {
 // ---------------------------------------------------------------------------
 constexpr int kMaxSmem = 232448;  // 227 KB
 
+// Columns of a convolution tile: at most conv::kMaxBn, in as many N tiles as
+// fill the device where a tensor has few positions.
+int direct_bn(int sms, int N, long long positions) {
+  const long long tiles = (positions + tc::kBM - 1) / tc::kBM;
+  int t = (N + conv::kMaxBn - 1) / conv::kMaxBn;
+  auto width = [&](int k) { return ((N + k - 1) / k + 15) / 16 * 16; };
+  while (tiles * t < sms && width(t) > 32) ++t;
+  return width(t);
+}
+
 // Stages of weights beside the input tile (0: the tile does not fit).
 int conv_stages(int C, int taps, int W, int bn) {
   for (int s = 4; s >= 2; --s)
@@ -904,7 +949,7 @@ int conv_stages(int C, int taps, int W, int bn) {
 struct ConvSplit {
   int splits, kper;  // ranges of K, 64-wide slices per range
 };
-// The ranges of the gathering GEMM (the partial sums, and so the results, are the same).
+// The ranges of the gathering GEMM's split K (the sums, and so the results, are the same).
 ConvSplit conv_ranges(int sms, int pixels, int N, int K) {
   const int slices = (K + tc::kBK - 1) / tc::kBK;
   const int s = conv_splits(sms, pixels, N, K);
@@ -914,8 +959,21 @@ ConvSplit conv_ranges(int sms, int pixels, int N, int K) {
 }
 
 long long op_positions(const conv::Op& o, int N) { return (long long)N * o.Pn(); }
-long long split_stride(const conv::Op& o, int N) {
-  return (op_positions(o, N) + tc::kBM - 1) / tc::kBM * tc::kBM;
+
+// A launch that may begin while its predecessor in the stream runs (the kernel waits for it itself).
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 // D = conv(a, packed weights of `layer`) for N samples through the epilogue.
@@ -934,19 +992,13 @@ cudaError_t conv_direct(clbm_net* net, const conv::Op& a, int layer, int transpo
   c.bn = d.bn;
   c.slices = d.slices;
   c.kper = r.kper;
-  c.stages = std::min(conv_stages(a.C, taps, a.W, d.bn), std::max(2, r.kper));
-  c.M = (int)op_positions(a, N);
-  c.Mst = split_stride(a, N);
-  c.part = r.splits > 1 ? net->part : nullptr;
+  c.ranges = r.splits;
+  c.stages = std::min(conv_stages(a.C, taps, a.W, d.bn), std::max(2, d.slices));
   c.epi = e;
   c.err = net->d_tflag;
-  if (r.splits > 1 && (long long)r.splits * d.N * c.Mst > net->part_cap) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)(c.Mst / tc::kBM), (unsigned)((d.N + d.bn - 1) / d.bn), (unsigned)r.splits);
-  conv::conv_kernel<<<grid, conv::kThreads, conv::conv_smem(a.C, taps, a.W + 2, d.bn, c.stages), net->stream>>>(c);
-  if (r.splits > 1)
-    conv::conv_finish_kernel<<<dim3((unsigned)((c.M + 127) / 128), (unsigned)((d.N + 7) / 8)), 128, 0, net->stream>>>(
-        net->part, r.splits, c.M, c.Mst, e);
-  return cudaGetLastError();
+  const dim3 grid((unsigned)((op_positions(a, N) + tc::kBM - 1) / tc::kBM), (unsigned)((d.N + d.bn - 1) / d.bn));
+  return launch_dependent(conv::conv_kernel, grid, conv::kConvThreads,
+                          conv::conv_smem(a.C, taps, a.W + 2, d.bn, c.stages), net->stream, c);
 }
 
 // Launch shape of a weight gradient.
@@ -1048,23 +1100,37 @@ cudaError_t forward_direct(clbm_net* net, const Plan& P, int N) {
       ep.H = ep.W = cv.H;
       ep.N = N;
       ep.channels = cv.co;
-      const int K = cv.ci * 9;
-      if ((e = tc_gemm(net, GatherIm2col<3>{view(net, P.in, 0, cv.ci)}, packed_of(net, 0, 0), TStoreOp{ep},
-                       N * cv.H * cv.W, cv.co, K, K))) return e;
+      const Act x = view(net, P.in, 0, cv.ci);
+      const int K = cv.ci * 9, M = N * cv.H * cv.W;
+      const tc::Packed w = packed_of(net, 0, 0);
+      auto gemm = [&](auto gather) { return tc_gemm(net, gather, w, TStoreOp{ep}, M, cv.co, K, K); };
+      switch (cv.ci) {
+        case 1: e = gemm(GatherFirst<1>{x}); break;
+        case 2: e = gemm(GatherFirst<2>{x}); break;
+        case 3: e = gemm(GatherFirst<3>{x}); break;
+        case 4: e = gemm(GatherFirst<4>{x}); break;
+        case 5: e = gemm(GatherFirst<5>{x}); break;
+        case 6: e = gemm(GatherFirst<6>{x}); break;
+        case 7: e = gemm(GatherFirst<7>{x}); break;
+        default: e = gemm(GatherIm2col<3>{x}); break;
+      }
+      if (e) return e;
       ++li;
     } else {
       if ((e = conv_into(net->aop[P.pool[l - 1]], P.a1[l], 0, 9, 1, nullptr, 0))) return e;
     }
     if ((e = conv_into(net->aop[P.a1[l]], P.cat[l], up, 9, 1, net->act[P.cat[l]], c))) return e;
     const conv::Op& o = net->aop[P.pool[l]];
-    conv::pool_op_kernel<<<op_grid((long long)N * o.H * o.W, c / 8), 128, 0, net->stream>>>(net->act[P.cat[l]], c, 0, N, o);
+    if ((e = launch_dependent(conv::pool_op_kernel, op_grid((long long)N * o.H * o.W, c / 8), 128, 0, net->stream,
+                              net->act[P.cat[l]], c, 0, N, o))) return e;
   }
   if ((e = conv_into(net->aop[P.pool[L - 2]], P.b1, 0, 9, 1, nullptr, 0))) return e;
   if ((e = conv_into(net->aop[P.b1], P.b2, 0, 9, 1, nullptr, 0))) return e;
   int prev = P.b2;
   for (int l = L - 2; l >= 0; --l) {
     const conv::Op& in = net->aop[prev];
-    conv::up_op_kernel<<<op_grid((long long)N * in.H * in.W, in.C / 8), 128, 0, net->stream>>>(in, N, net->aop[P.cat[l]]);
+    if ((e = launch_dependent(conv::up_op_kernel, op_grid((long long)N * in.H * in.W, in.C / 8), 128, 0, net->stream,
+                              in, N, net->aop[P.cat[l]]))) return e;
     if ((e = conv_into(net->aop[P.cat[l]], P.d1[l], 0, 9, 1, nullptr, 0))) return e;
     if ((e = conv_into(net->aop[P.d1[l]], P.d2[l], 0, 9, 1, nullptr, 0))) return e;
     prev = P.d2[l];
@@ -1125,8 +1191,8 @@ cudaError_t backward_direct(clbm_net* net, const Plan& P, int N) {
     if ((e = conv_direct(net, net->gop[P.d1[l]], c1, 1, 9, N, plain(P.cat[l])))) return e;
     const int below = l + 1 <= L - 2 ? P.d2[l + 1] : P.b2;
     const conv::Epilogue ep = masked(below);
-    conv::up_back_op_kernel<<<op_grid((long long)N * ep.H * ep.W, ep.channels / 8), 128, 0, net->stream>>>(
-        net->gact[P.cat[l]], net->act_c[P.cat[l]], 0, ep);
+    if ((e = launch_dependent(conv::up_back_op_kernel, op_grid((long long)N * ep.H * ep.W, ep.channels / 8), 128, 0,
+                              net->stream, net->gact[P.cat[l]], net->act_c[P.cat[l]], 0, ep))) return e;
   }
   {  // bottleneck
     const int c2 = li--, c1 = li--;
@@ -1149,8 +1215,8 @@ cudaError_t backward_direct(clbm_net* net, const Plan& P, int N) {
     ep.H = ep.W = net->act_hw[cat];
     ep.N = N;
     ep.channels = c;
-    conv::pool_back_op_kernel<<<op_grid((long long)N * ep.H * ep.W, c / 8), 128, 0, net->stream>>>(
-        net->gact[cat], cup + c, cup, net->gact[P.pool[l]], c, ep);
+    if ((e = launch_dependent(conv::pool_back_op_kernel, op_grid((long long)N * ep.H * ep.W, c / 8), 128, 0,
+                              net->stream, net->gact[cat], cup + c, cup, net->gact[P.pool[l]], c, ep))) return e;
     if ((e = weights(net->convs[c2], net->aop[P.a1[l]], net->gop[cat], view(net, cat, cup, c, true)))) return e;
     if ((e = conv_direct(net, net->gop[cat], c2, 1, 9, N, masked(P.a1[l])))) return e;
     if ((e = weights(net->convs[c1], net->aop[l > 0 ? P.pool[l - 1] : P.in], net->gop[P.a1[l]], grad(P.a1[l])))) return e;
@@ -1400,8 +1466,8 @@ bool direct_fits(const std::vector<Conv>& convs, const clbm_net_config& c) {
   if (c.base % 8 != 0 || c.in_ch > 8 || c.out_ch > 8) return false;
   for (const Conv& cv : convs) {
     const int taps = cv.ks * cv.ks;
-    if (cv.ci % 8 == 0 && !conv_stages(cv.ci, taps, cv.W, tc::tile_n(cv.co))) return false;
-    if (cv.co % 8 == 0 && !conv_stages(cv.co, taps, cv.W, tc::tile_n(cv.ci))) return false;
+    if (cv.ci % 8 == 0 && !conv_stages(cv.ci, taps, cv.W, conv::kMaxBn)) return false;
+    if (cv.co % 8 == 0 && !conv_stages(cv.co, taps, cv.W, conv::kMaxBn)) return false;
     conv::Op x{};
     x.C = (cv.ci + 7) / 8 * 8;
     x.H = x.W = cv.H;
@@ -1556,6 +1622,12 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
   cudaMemset(n->v, 0, off * sizeof(float));
   cudaMemset(n->g, 0, off * sizeof(float));
   to_bf16_kernel<<<grid1(off), 256, 0, n->stream>>>(n->p, n->pb, off);
+  {  // one wave of CTAs is sized from the device's multiprocessor count
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+      n->sms = sms;
+  }
   n->direct = c.math == CLBM_NET_TENSOR && direct_fits(n->convs, c);
   if (c.math == CLBM_NET_TENSOR) {
     long long total = 0;
@@ -1570,10 +1642,10 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
         d.transpose = tr;
         d.N = tr ? cv.ci : cv.co;
         d.K = (tr ? cv.co : cv.ci) * d.kk;
-        d.bn = tc::tile_n(d.N);
         d.slices = (d.K + tc::kBK - 1) / tc::kBK;
-        // operand-layout convolutions read K in their own chunk order
-        d.groups = n->direct && (tr ? cv.co : cv.ci) % 8 == 0 ? (tr ? cv.co : cv.ci) / 8 : 0;
+        // operand-layout convolutions read K in their own chunk order, in tiles of their own width
+        d.groups = n->direct && (tr ? cv.co : cv.ci) % 8 == 0 && (tr ? cv.ks == 3 : cv.index > 0) ? (tr ? cv.co : cv.ci) / 8 : 0;
+        d.bn = d.groups ? direct_bn(n->sms, d.N, (long long)c.max_batch * cv.H * cv.W) : tc::tile_n(d.N);
         d.size = (long long)((d.N + d.bn - 1) / d.bn) * d.slices * d.bn * tc::kBK;
         total += (d.size + 63) / 64 * 64;  // keep every layer's tiles 128-byte aligned
         n->packed_max = std::max(n->packed_max, d.size);
@@ -1602,12 +1674,6 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
     n->gact.push_back(ga);
   }
   if (n->direct && make_operands(n) != cudaSuccess) return bail(CLBM_ENOMEM);
-  {  // one wave of CTAs is sized from the device's multiprocessor count
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
-      n->sms = sms;
-  }
   // split-K partials: enough for the largest batch (fewer pixels never need more splits)
   long long cap = 0, dw_cap = 0;
   for (const Conv& cv : n->convs) {
@@ -1625,11 +1691,7 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
         const DwShape s = dw_shape(n->sms, x, (cv.co + 7) / 8, cv.ks * cv.ks, (int)nb);
         dw_need = std::max(dw_need, (long long)s.ranges * cv.co * Kd);
         bias_need = std::max(bias_need, ((Np + kBiasChunk - 1) / kBiasChunk) * cv.co);
-        const long long Mst = split_stride(x, (int)nb);
-        cap = std::max(cap, conv_ranges(n->sms, (int)Np, cv.co, Kd).splits * Mst * cv.co);
-        cap = std::max(cap, conv_ranges(n->sms, (int)Np, cv.ci, cv.co * cv.ks * cv.ks).splits * Mst * cv.ci);
-      }
-      if (c.math == CLBM_NET_TENSOR) {  // split-K forward and input-gradient GEMMs
+      } else if (c.math == CLBM_NET_TENSOR) {  // split-K forward and input-gradient GEMMs
         cap = std::max(cap, (long long)conv_splits(n->sms, (int)Np, cv.co, Kd) * Np * cv.co);
         cap = std::max(cap, (long long)conv_splits(n->sms, (int)Np, cv.ci, cv.co * cv.ks * cv.ks) * Np * cv.ci);
       }
