@@ -122,7 +122,9 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 constexpr int kMaxBn = 64;         // columns of a tile: a thread keeps its row's sums in registers
-constexpr int kConvThreads = 192;  // four epilogue warps, one for the copies, one for the MMAs
+// threads of a block: four epilogue warps; copies and MMAs are issued by two of them, or by two more
+// warps where sums of several ranges are formed while the MMAs go on
+__host__ __device__ constexpr int conv_threads(bool ranges) { return ranges ? 192 : 128; }
 
 __host__ __device__ constexpr int conv_run(int taps, int Wp) { return tc::kBM + (taps == 9 ? 2 * Wp + 2 : 0); }
 // pairs of K chunks (the MMAs), rounded up to whole slices
@@ -141,17 +143,21 @@ __host__ __device__ __forceinline__ bool pair_swapped(int u, int groups, int tot
 }
 
 // Implicit GEMM D[position][channel] of one 128-position tile (blockIdx.x) and
-// bn channels (blockIdx.y).  Warp 4 issues the copies, warp 5 the MMAs, warps
-// 0-3 the epilogue.  The matrix descriptors are made beforehand by all
+// bn channels (blockIdx.y).  The matrix descriptors are made beforehand by all
 // threads: one thread that divided by the number of channel groups for every
 // MMA took 20 us a tile.
 //
-// K is summed in ranges, each into an accumulator of its own (two, in turn),
-// and the ranges' sums are added in order in registers: the order of a split-K
-// GEMM whose partial sums are added by a second kernel, without that kernel
-// (94 us for the 384 -> 128 convolution at 16^2, 12 us so).
+// RANGES: K is summed in ranges, each into an accumulator of its own (two, in
+// turn), and the ranges' sums are added in order in registers: the order of a
+// split-K GEMM whose partial sums are added by a second kernel, without that
+// kernel (94 us for the 384 -> 128 convolution at 16^2).  One range needs
+// neither the registers nor the extra warps (three blocks per multiprocessor
+// instead of seven doubled its time).
 // Launch with conv_smem() bytes of dynamic shared memory.
-__global__ void __launch_bounds__(kConvThreads) conv_kernel(const __grid_constant__ ConvArgs a) {
+template <bool RANGES>
+__global__ void __launch_bounds__(conv_threads(RANGES)) conv_kernel(const __grid_constant__ ConvArgs a) {
+  constexpr int kConvThreads = conv_threads(RANGES);
+  constexpr int kCopyWarp = RANGES ? 4 : 0, kMmaWarp = RANGES ? 5 : 1;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int groups = a.a.C / 8, Wp = a.a.W + 2;
@@ -167,7 +173,7 @@ __global__ void __launch_bounds__(kConvThreads) conv_kernel(const __grid_constan
   uint32_t* slot = reinterpret_cast<uint32_t*>(bar_f + 2);
   float* bias = reinterpret_cast<float*>(slot + 2);  // [bn]
   const int m0 = blockIdx.x * tc::kBM, n0 = blockIdx.y * a.bn;
-  const uint32_t ncols = tc::tmem_cols(a.ranges > 1 ? 2 * a.bn : a.bn);
+  const uint32_t ncols = tc::tmem_cols(RANGES ? 2 * a.bn : a.bn);
 
   if (warp == 0) tc::tmem_alloc(slot, ncols);
   if (tid == 32) {
@@ -203,11 +209,12 @@ __global__ void __launch_bounds__(kConvThreads) conv_kernel(const __grid_constan
   pdl_go();
   const uint32_t tmem = *slot;
   bool failed = false;
-  float sum[kMaxBn];
-  int pos = 0, n = 0, p = 0;
-  bool inside = false;
+  float sum[RANGES ? kMaxBn : 1];
+  const int pos = m0 + tid;
+  int n = 0, p = 0;
+  const bool inside = tid < tc::kBM && a.epi.locate(pos, n, p);
 
-  if (warp == 4) {
+  if (warp == kCopyWarp) {
     const bf16* w = a.w + (long long)blockIdx.y * a.slices * a.bn * 64;
     auto weights = [&](int i) {
       const int s = i % a.stages;
@@ -239,12 +246,12 @@ __global__ void __launch_bounds__(kConvThreads) conv_kernel(const __grid_constan
           tc::mbar_wait(&bar_b[k % a.stages], (uint32_t)((k / a.stages) & 1));
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == kMmaWarp) {
     if (lane == 0) {
       const uint32_t idesc = tc::idesc_bf16_f32(tc::kBM, a.bn);
       failed = !tc::mbar_wait(bar_a, 0);
       int i = 0;
-      for (int z = 0; z < a.ranges && !failed; ++z) {
+      for (int z = 0; z < (RANGES ? a.ranges : 1) && !failed; ++z) {
         const uint32_t acc = tmem + (z & 1) * a.bn;
         if (z >= 2) {
           failed = !tc::mbar_wait(&bar_f[z & 1], (uint32_t)((z / 2 - 1) & 1));
@@ -269,41 +276,56 @@ __global__ void __launch_bounds__(kConvThreads) conv_kernel(const __grid_constan
       }
       // after a failure the other warps still wait for every range: let them time out on their own
     }
-  } else {
-    pos = m0 + tid;
-    inside = a.epi.locate(pos, n, p);
+  }
+  if constexpr (RANGES) {
+    if (warp < 4) {
 #pragma unroll
-    for (int c = 0; c < kMaxBn; ++c) sum[c] = 0.0f;
-    for (int z = 0; z < a.ranges; ++z) {
-      if (!tc::mbar_wait(&bar_d[z & 1], (uint32_t)((z / 2) & 1))) {
-        failed = true;
-        break;
+      for (int c = 0; c < kMaxBn; ++c) sum[c] = 0.0f;
+      for (int z = 0; z < a.ranges; ++z) {
+        if (!tc::mbar_wait(&bar_d[z & 1], (uint32_t)((z / 2) & 1))) {
+          failed = true;
+          break;
+        }
+        tc::fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < kMaxBn; c0 += 16) {
+          if (c0 >= a.bn) break;
+          float v[16];
+          tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((z & 1) * a.bn + c0), v);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) sum[c0 + k] += v[k];
+        }
+        tc::fence_before();
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&bar_f[z & 1])) : "memory");
       }
-      tc::fence_after();
-#pragma unroll
-      for (int c0 = 0; c0 < kMaxBn; c0 += 16) {
-        if (c0 >= a.bn) break;
-        float v[16];
-        tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((z & 1) * a.bn + c0), v);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) sum[c0 + k] += v[k];
-      }
-      tc::fence_before();
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&bar_f[z & 1])) : "memory");
     }
+  } else {
+    __syncwarp();
+    if (!tc::mbar_wait(&bar_d[0], 0)) failed = true;
   }
   if (__syncthreads_or(failed)) {
     if (tid == 0) atomicExch(a.err, 1);
   } else if (warp < 4) {
     pdl_wait();
-    if (inside) {
+    tc::fence_after();
 #pragma unroll
-      for (int h = 0; h < kMaxBn; h += 8) {
-        if (h >= a.bn || n0 + h >= a.epi.channels) break;
+    for (int c0 = 0; c0 < kMaxBn; c0 += 16) {
+      if (c0 >= a.bn) break;
+      float v[16];
+      if constexpr (RANGES) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = sum[c0 + k];
+      } else {
+        tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      }
+      if (!inside) continue;
+#pragma unroll
+      for (int h = 0; h < 16; h += 8) {
+        if (n0 + c0 + h >= a.epi.channels) break;
         float x[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] = sum[h + k];
-        a.epi.apply(pos, n, p, n0 + h, x, bias + h);
+        for (int k = 0; k < 8; ++k) x[k] = v[h + k];
+        a.epi.apply(pos, n, p, n0 + c0 + h, x, bias + c0 + h);
       }
     }
   }

@@ -679,10 +679,13 @@ __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict
                             const float* __restrict__ mask, const double* __restrict__ mpart, int N,
                             int C, int HW, float* __restrict__ g, double* __restrict__ part) {
   __shared__ double inv_norm;
+  __shared__ double ms[GT];
+  if (mask && threadIdx.x < N) ms[threadIdx.x] = mpart[threadIdx.x];  // fetched together, added in order
+  __syncthreads();
   if (threadIdx.x == 0) {
     double m = 0.0;
     if (mask) {
-      for (int i = 0; i < N; ++i) m += mpart[i];
+      for (int i = 0; i < N; ++i) m += i < GT ? ms[i] : mpart[i];
     } else {
       m = (double)N * HW;
     }
@@ -997,8 +1000,8 @@ cudaError_t conv_direct(clbm_net* net, const conv::Op& a, int layer, int transpo
   c.epi = e;
   c.err = net->d_tflag;
   const dim3 grid((unsigned)((op_positions(a, N) + tc::kBM - 1) / tc::kBM), (unsigned)((d.N + d.bn - 1) / d.bn));
-  return launch_dependent(conv::conv_kernel, grid, conv::kConvThreads,
-                          conv::conv_smem(a.C, taps, a.W + 2, d.bn, c.stages), net->stream, c);
+  return launch_dependent(r.splits > 1 ? conv::conv_kernel<true> : conv::conv_kernel<false>, grid,
+                          conv::conv_threads(r.splits > 1), conv::conv_smem(a.C, taps, a.W + 2, d.bn, c.stages), net->stream, c);
 }
 
 // Launch shape of a weight gradient.
@@ -1517,7 +1520,8 @@ cudaError_t make_operands(clbm_net* n) {
   }
   both(P.b1);
   both(P.b2);
-  if (!e) e = cudaFuncSetAttribute(conv::conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  if (!e) e = cudaFuncSetAttribute(conv::conv_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  if (!e) e = cudaFuncSetAttribute(conv::conv_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (!e) e = cudaFuncSetAttribute(conv::dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   return e;
 }
@@ -1706,7 +1710,7 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
     if (cudaMalloc(&n->dw_part, dw_cap * sizeof(float))) return bail(CLBM_ENOMEM);
     for (cudaStream_t& st : n->side)
       if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return bail(CLBM_ECUDA);
-    n->events.resize(n->convs.size() + clbm_net::kSides, nullptr);
+    n->events.resize(n->convs.size() + clbm_net::kSides + 2, nullptr);  // the last two: the mask sums
     for (cudaEvent_t& ev : n->events)
       if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) return bail(CLBM_ECUDA);
   }
@@ -1785,11 +1789,19 @@ clbm_status clbm_net_gradients(clbm_net* n, const float* x, const float* target,
   if (!e && mask)
     e = cudaMemcpyAsync(n->msk, mask, (size_t)N * G * G * sizeof(float), cudaMemcpyDeviceToDevice, n->stream);
   if (!e) e = run_captured(n, n->grad_pass, msk, nullptr, nullptr, N, [&]() {
-    cudaError_t e = forward(n, P, N);
-    if (!e && msk) {
-      mask_sum_kernel<<<N, GT, 0, n->stream>>>(msk, G * G, mpart);
-      e = cudaGetLastError();
+    // the mask's sums beside the forward pass where there is a side stream
+    const cudaStream_t ms = n->direct ? n->side[0] : n->stream;
+    cudaEvent_t* const ev = n->direct ? n->events.data() + n->events.size() - 2 : nullptr;
+    cudaError_t e = cudaSuccess;
+    if (msk) {
+      if (ev) e = cudaEventRecord(ev[0], n->stream);
+      if (!e && ev) e = cudaStreamWaitEvent(ms, ev[0], 0);
+      if (!e) mask_sum_kernel<<<N, GT, 0, ms>>>(msk, G * G, mpart);
+      if (!e) e = cudaGetLastError();
+      if (!e && ev) e = cudaEventRecord(ev[1], ms);
     }
+    if (!e) e = forward(n, P, N);
+    if (!e && msk && ev) e = cudaStreamWaitEvent(n->stream, ev[1], 0);
     if (!e) {
       loss_kernel<<<dim3(N, kLossChunks), GT, 0, n->stream>>>(n->act[P.out], n->tgt, msk, mpart, N, C, G * G,
                                                               n->gact[P.out], n->loss_part);
