@@ -1219,11 +1219,12 @@ bool resident_plan(const clbm_ctx* c, int cl, size_t max_smem, int max_threads, 
   if (nx > 65535 || rows + 2 > 65535) return false;  // 16-bit coordinates of the boundary nodes
   const size_t smem = c->L->resident_smem(nx, rows, most, c->p.viscous_heating);
   if (smem > max_smem) return false;
-  const int items = (most + 31) / 32 * 32 + rows * nx;
-  // whole passes over the items: as few threads as take the same number of passes
-  const int passes = (items + max_threads - 1) / max_threads;
+  // a thread per boundary node (at most half of them), the others in whole passes over the
+  // interior: as few as take the same number of passes
+  const int bt = std::min((most + 31) / 32 * 32, max_threads / 2), nodes = rows * nx;
+  const int passes = (nodes + (max_threads - bt) - 1) / (max_threads - bt);
   plan->cl = cl;
-  plan->threads = std::max(64, ((items + passes - 1) / passes + 31) / 32 * 32);
+  plan->threads = std::min(max_threads, std::max(64, bt + ((nodes + passes - 1) / passes + 31) / 32 * 32));
   plan->smem = smem;
   if (lat) {
     const ViewInfo w = describe_view(c);

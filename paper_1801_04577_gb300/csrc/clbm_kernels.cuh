@@ -60,10 +60,6 @@ __host__ __device__ constexpr int ey_of(int d) {
 __host__ __device__ constexpr int opp_of(int d) {
   return d == 0 ? 0 : (d <= 4 ? ((d + 1) % 4) + 1 : ((d - 5 + 2) % 4) + 5);
 }
-// box side crossed by the pull source of D2Q5 direction j: 1 -> x0, 2 -> y0, 3 -> x1, 4 -> y1
-__host__ __device__ constexpr int side_of(int j) {
-  return j == 1 ? 0 : (j == 2 ? 2 : (j == 3 ? 1 : 3));
-}
 
 // ---------------------------------------------------------------------------
 // Storage formats
@@ -477,6 +473,7 @@ __host__ __device__ __forceinline__ void equilibrium(const Co<R>& c, R rho, R ux
 template <typename S>
 struct PlaneSrc {
   using Idx = long long;
+  static constexpr bool kShared = false;
   const S* __restrict__ p;
   long long plane;
   __device__ __forceinline__ S at(int q, long long i) const { return p[q * plane + i]; }
@@ -485,6 +482,7 @@ struct PlaneSrc {
 template <typename S, int ST>
 struct NodeSrc {
   using Idx = int;
+  static constexpr bool kShared = true;
   const S* p;
   __device__ __forceinline__ S at(int q, int i) const { return p[i * ST + q]; }
 };
@@ -581,23 +579,21 @@ __device__ __forceinline__ void node_update(const DevGeom& g, const Co<R>& c, co
   };
   if (wall & 0xFu) {
     const R s1 = node_heat(src, own, c);
-#pragma unroll
-    for (int j = 1; j < 5; ++j) {
-      if (!((wall >> (j - 1)) & 1u)) continue;
-      const int ex = ex_of(j), ey = ey_of(j);
+    // Eq. 26 at the wall of direction j = b + 1
+    auto rule = [&](int b, int ex, int ey) {
       R ka, kb, kc, kd = R(0);
-      if ((box >> (j - 1)) & 1u) {
+      if ((box >> b) & 1u) {
         bool have2;
         if (MASK)
-          have2 = !((fl >> (kFlagSecond + j - 1)) & 1u);
+          have2 = !((fl >> (kFlagSecond + b)) & 1u);
         else
           have2 = ex != 0 ? g.nx > 1 : !(ey > 0 ? (y_hi && g.ywhi) : (y_lo && g.ywlo));
-        const R* k = side_wall<R>(g, side_of(j), have2);
+        const R* k = side_wall<R>(g, ex > 0 ? 0 : (ex < 0 ? 1 : (ey > 0 ? 2 : 3)), have2);
         ka = k[0];
         kb = k[1];
         kc = k[2];
       } else {
-        const R* k = static_cast<const R*>(g.lk_t) + 16 * slot + 4 * (opp_of(j) - 1);
+        const R* k = static_cast<const R*>(g.lk_t) + 16 * slot + 4 * ((b + 2) & 3);  // link opp(j)
         ka = __ldg(k);
         kb = __ldg(k + 1);
         kc = __ldg(k + 2);
@@ -607,7 +603,23 @@ __device__ __forceinline__ void node_update(const DevGeom& g, const Co<R>& c, co
       if (kd != R(0)) e = fma_(kd, node_heat(src, ahead(ex, ey, 2), c), e);
       if (kb != R(0)) e = fma_(kb, node_heat(src, ahead(ex, ey, 1), c), e);
       if (ka != R(0)) e = fma_(ka, s1, e);
-      h[j] = sub_(e, h[j]);  // Eq. 26
+      return e;
+    };
+    if constexpr (MASK && Src::kShared) {
+      // one pass per wall of the node, whichever its direction, so that nodes with walls in
+      // different directions share it (resident 200 x 100 channel 3.5 -> 2.9 us a step; from planes in
+      // device memory the passes by direction are faster, annulus 1.69 -> 1.62 ms)
+      for (uint32_t m = wall & 0xFu; m; m &= m - 1) {
+        const int b = __ffs((int)m) - 1;
+        const R e = rule(b, (b == 0) - (b == 2), (b == 1) - (b == 3));
+#pragma unroll
+        for (int j = 1; j < 5; ++j)
+          if (j == b + 1) h[j] = sub_(e, h[j]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 1; j < 5; ++j)
+        if ((wall >> (j - 1)) & 1u) h[j] = sub_(rule(j - 1, ex_of(j), ey_of(j)), h[j]);
     }
   }
   if (MASK && (fl & kFlagOffMid)) {  // walls off the link midpoint: interpolated bounce-back

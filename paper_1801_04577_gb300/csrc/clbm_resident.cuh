@@ -14,8 +14,7 @@
 // consecutive nodes fall into different banks): one address and immediate
 // offsets reach all populations of a neighbour, which spares the address
 // arithmetic of 28 planes.  Boundary nodes (the list of the plane kernels)
-// come first in a block's work and fill warps of their own, so that interior
-// warps stay convergent.
+// have warps of their own, so that interior warps stay convergent.
 #pragma once
 
 namespace clbm {
@@ -187,7 +186,9 @@ __global__ void __launch_bounds__(kMaxResidentThreads, 1) resident_kernel(const 
   const int r_lo = rank > 0 ? rank - 1 : cl - 1, r_hi = rank < cl - 1 ? rank + 1 : 0;
   const int rows_lo = band_start(r_lo + 1, cl, ny) - band_start(r_lo, cl, ny);
   const int last = (rows - 1) * nx;
-  const int nbp = (nb + 31) & ~31, total = nbp + rows * nx;
+  // The first bt threads update the boundary nodes, the others the interior: a boundary node takes
+  // about as long as two interior ones, and each band waits for its slowest warp.
+  const int bt = min((nb + 31) & ~31, nt / 2 & ~31), total = rows * nx;
 
   // Store of local node li in column x: locally, and into the ghost rows of the neighbours if it
   // lies on an edge of the band (what streams across; all of it where the neighbour has walls).
@@ -225,10 +226,9 @@ __global__ void __launch_bounds__(kMaxResidentThreads, 1) resident_kernel(const 
       const long long t = t0 + s;
       seed = (uint32_t)(t * 0x9E3779B1ull) ^ (uint32_t)(t >> 32);
     }
-    for (int i = tid; i < total; i += nt) {
-      R d[9], h[5], qv = R(0);
-      if (i < nbp) {
-        if (i >= nb) continue;
+    if (tid < bt) {
+      for (int i = tid; i < nb; i += bt) {
+        R d[9], h[5], qv = R(0);
         const ResNode e = edge[i];
         const NodeSrc<S, ST> ns{src};
         if (masked)
@@ -236,8 +236,11 @@ __global__ void __launch_bounds__(kMaxResidentThreads, 1) resident_kernel(const 
         else
           node_update<NodeSrc<S, ST>, false>(L.L.g, c, ns, e.x, e.y, 0u, 0, d, h, qv);
         store(dst, e.y * nx + e.x, e.x, e.y == 1, e.y == rows, d, h, qv, sr_key(seed, (long long)e.gi - (e.x & 3)));
-      } else {
-        const int n = i - nbp, li = n + nx;
+      }
+    } else {
+      for (int n = tid - bt; n < total; n += nt - bt) {
+        R d[9], h[5], qv = R(0);
+        const int li = n + nx;
         if (kind[li] & 3) continue;
         const S* o = src + li * ST;
 #pragma unroll
