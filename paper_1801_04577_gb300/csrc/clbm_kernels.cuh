@@ -676,6 +676,17 @@ __device__ __forceinline__ void st1(S* p, R v, int stochastic, uint32_t key, int
   *p = from_r<S, R>(v);
 }
 
+// Steps of more than one wave of blocks are launched as programmatic
+// dependents: the next step's first blocks take the places that the last wave
+// leaves, read their arguments, and wait here until the stores of the step
+// before are visible (nothing before touches the state).  Per step: annulus
+// 2048 FP32 79.9 -> 78.9 us, FP16 4096 x 2048 79.1 -> 78.6, 1024 x 512 FP32
+// 8.65 -> 8.44.  In one wave the early blocks would land unevenly beside the
+// running ones (FP64 101^2 9.0 -> 12.6 us): those steps are launched plainly.
+__device__ __forceinline__ void step_wait() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
 // Interior update.  One warp updates the 32 * V nodes x = xw .. xw + 32V - 1
 // of row y (each lane owns V consecutive nodes); all 32 lanes must call it
 // together.  Every node is pulled and collided as if it were an interior
@@ -1027,6 +1038,7 @@ __global__ void __launch_bounds__(kStepThreads, kStepBlocks<S>) step_box_kernel(
   const Co<R> c = make_co<R>(a.c);
   const S* src = static_cast<const S*>(a.src);
   S* dst = static_cast<S*>(a.dst);
+  step_wait();
   const int b = blockIdx.x, row = b / xblocks, xb = b - row * xblocks;
   const int xw = (xb * blockDim.x + (threadIdx.x & ~31)) * V;
   if (xw >= a.g.nx) return;  // whole warps only
@@ -1049,6 +1061,7 @@ __global__ void __launch_bounds__(kStepThreads, kStepBlocks<S>) step_fused_kerne
   using R = typename Traits<S>::R;
   constexpr int V = Traits<S>::V;
   const Co<R> c = make_co<R>(a.c);
+  step_wait();
   if ((int)blockIdx.x < nbb) {
     const int k = blockIdx.x * kStepThreads + threadIdx.x;
     if (k < a.nb)
@@ -1617,11 +1630,23 @@ struct LaunchImpl {
     const int wx = std::min(tiles, kStepThreads / 32), xblocks = wx > 0 ? (tiles + wx - 1) / wx : 0;
     if (xblocks <= 0 || rows <= 0) return cudaSuccess;
     const unsigned nblk = (unsigned)xblocks * (unsigned)rows;
-    if (a.c.vh)
-      step_box_kernel<S, VV, true><<<nblk, 32 * wx, 0, s>>>(a, xblocks, rows);
-    else
-      step_box_kernel<S, VV, false><<<nblk, 32 * wx, 0, s>>>(a, xblocks, rows);
-    return cudaGetLastError();
+    return launch_step(a.c.vh ? step_box_kernel<S, VV, true> : step_box_kernel<S, VV, false>, nblk, 32 * wx, s, a,
+                       xblocks, rows);
+  }
+
+  // a step's launch; of more than one wave it may begin while its predecessor in the stream runs
+  template <class... P, class... A>
+  static cudaError_t launch_step(void (*kernel)(P...), unsigned blocks, int threads, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = (long long)blocks > (long long)sm_count() * kStepBlocks<S> ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
   }
 
   static int sm_count() {
@@ -1654,18 +1679,9 @@ struct LaunchImpl {
     const int nbb = (a.nb + kStepThreads - 1) / kStepThreads;
     const unsigned nblk = (unsigned)nbb + (unsigned)xblocks * (unsigned)rows;
     if (nblk == 0) return cudaSuccess;
-    if (a.g.flags) {
-      if (a.c.vh)
-        step_fused_kernel<S, true, true><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-      else
-        step_fused_kernel<S, false, true><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-    } else {
-      if (a.c.vh)
-        step_fused_kernel<S, true, false><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-      else
-        step_fused_kernel<S, false, false><<<nblk, kStepThreads, 0, s>>>(a, nbb, xblocks, y0, rows);
-    }
-    return cudaGetLastError();
+    auto kernel = a.g.flags ? (a.c.vh ? step_fused_kernel<S, true, true> : step_fused_kernel<S, false, true>)
+                            : (a.c.vh ? step_fused_kernel<S, true, false> : step_fused_kernel<S, false, false>);
+    return launch_step(kernel, nblk, kStepThreads, s, a, nbb, xblocks, y0, rows);
   }
 
   static int blocks_for(long long n, int threads) {
