@@ -23,9 +23,9 @@ using namespace clbm;
 
 namespace {
 
-constexpr int kWidthChoices[kBatchGroups] = {1, 2, 4};  // nodes per lane; a warp covers 32 x this
+constexpr int kWidthChoices[kBatchWidths] = {1, 2, 4};  // nodes per lane; a warp covers 32 x this
 
-int group_id(int v) { return v == 1 ? 0 : (v == 2 ? 1 : 2); }
+int group_id(int v, int masked) { return (v == 1 ? 0 : (v == 2 ? 1 : 2)) + (masked ? kBatchWidths : 0); }
 
 int width_class(int nx) { return nx <= 48 ? 0 : (nx <= 96 ? 1 : (nx <= 192 ? 2 : 3)); }
 
@@ -80,8 +80,7 @@ __global__ void batch_scan_kernel(int n, const int* __restrict__ active,
   ctl->n_active = nact;
 }
 
-// Tiles {lattice, row, first x, 0} of rows y0 .. y0 + rows - 1 (the rows that
-// are not boundary rows) of every active lattice.
+// Tiles {lattice, row, first x, 0} of rows y0 .. y0 + rows - 1 of every active lattice.
 __global__ void batch_tiles_kernel(int n, const int* __restrict__ active,
                                    const long long* __restrict__ offset,
                                    const int* __restrict__ group_of, const int* __restrict__ rows_of,
@@ -154,11 +153,12 @@ static clbm_status bfail(clbm_batch* b, clbm_status s, const std::string& m) {
     if (e_ != cudaSuccess) return bfail((b), CLBM_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-// Rows that get interior tiles: all rows of a periodic y axis, else all but the
-// first and last (boundary rows).
-static int interior_rows(const clbm_batch* b, int i) {
-  if (b->res_cl[i]) return 0;  // no tiles
-  return b->py[i] ? b->ny[i] : std::max(b->ny[i] - 2, 0);
+// Rows that get tiles: all; with a mask and y walls all but the first and last
+// (boundary rows).
+static int first_row(const clbm_batch* b, int i) { return b->masked[i] && !b->py[i] ? 1 : 0; }
+static int tile_rows(const clbm_batch* b, int i) {
+  if (b->res_cl[i]) return 0;
+  return std::max(b->ny[i] - 2 * first_row(b, i), 0);
 }
 
 // Upload the per-lattice launch layout (group, tile counts) for the current widths.
@@ -169,14 +169,14 @@ static clbm_status upload_layout(clbm_batch* b, const std::vector<int>& active) 
   for (int i = 0; i < n; ++i) {
     const int w = 32 * b->width[i];
     const int tpr = (b->nx[i] + w - 1) / w;
-    const int rows = interior_rows(b, i);
-    b->group[i] = group_id(b->width[i]);
+    const int rows = tile_rows(b, i);
+    b->group[i] = group_id(b->width[i], b->masked[i]);
     ints[i] = b->group[i];
     ints[n + i] = rows * tpr;
     ints[2 * n + i] = rows;
     ints[3 * n + i] = tpr;
     ints[4 * n + i] = w;
-    ints[5 * n + i] = b->py[i] ? 0 : 1;
+    ints[5 * n + i] = first_row(b, i);
     gcap[b->group[i]] += (long long)rows * tpr;
   }
   std::vector<int4*> bases(kBatchGroups);
@@ -206,8 +206,8 @@ static clbm_status build_tiles(clbm_batch* b) {
 }
 
 // One step of every active lattice; parity = which buffer holds the current state.
-// Interior tiles first (one launch per tile-width group), then the boundary nodes
-// (which, next to solids, replace the provisional values the tiles wrote).
+// Tiles first (one launch per tile width, without and with a mask), then the boundary nodes of
+// the masked lattices (which, next to solids, replace the provisional values the tiles wrote).
 static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
   std::vector<int> used(kBatchGroups, 0);
   for (int i = 0; i < b->n; ++i)
@@ -215,9 +215,9 @@ static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
   const std::vector<long long>& base = b->group_base;  // as in upload_layout
   for (int g = 0; g < kBatchGroups; ++g) {
     if (!used[g]) continue;
-    const int v = kWidthChoices[g];
+    const int v = kWidthChoices[g % kBatchWidths];
     if (b->grid[g] <= 0) return bfail(b, CLBM_ECUDA, "no occupancy for the batched step kernel");
-    BCUDA(b, b->L->batch_step(v, b->d_lats, b->d_tiles + base[g], &b->d_ctl->count[g], parity,
+    BCUDA(b, b->L->batch_step(v, g >= kBatchWidths, b->d_lats, b->d_tiles + base[g], &b->d_ctl->count[g], parity,
                               &b->d_ctl->t, tstep, b->rounding, b->grid[g], b->stream));
   }
   BCUDA(b, b->L->batch_boundary(b->d_lats, b->d_bent, b->nbent, b->d_active, parity, &b->d_ctl->t,
@@ -477,7 +477,7 @@ clbm_status clbm_batch_create(const clbm_batch_item* items, int32_t n, int32_t a
     lats[i].snap = b->d_snap + snap_off;
     snap_off += 3 * b->nodes[i];
     b->masked[i] = v.g.flags != nullptr;
-    for (int k = 0; k < v.nb && !b->res_cl[i]; ++k) bent.push_back(make_int2(i, v.bnodes_host[k]));
+    for (int k = 0; k < v.nb && b->masked[i] && !b->res_cl[i]; ++k) bent.push_back(make_int2(i, v.bnodes_host[k]));
   }
   b->nbent = (int)bent.size();
   if (!bent.empty()) {
@@ -514,7 +514,9 @@ clbm_status clbm_batch_create(const clbm_batch_item* items, int32_t n, int32_t a
       cudaMemset(b->d_ctl, 0, sizeof(BatchCtl)) != cudaSuccess)
     return bail(CLBM_ECUDA);
   for (int g = 0; g < kBatchGroups; ++g)
-    b->grid[g] = kWidthChoices[g] > L->vec ? 0 : L->batch_grid(kWidthChoices[g]);
+    b->grid[g] = kWidthChoices[g % kBatchWidths] > L->vec
+                     ? 0
+                     : L->batch_grid(kWidthChoices[g % kBatchWidths], g >= kBatchWidths);
   if (autotune_tiles) {
     clbm_status st = autotune(b);
     if (st != CLBM_OK) return bail(st);

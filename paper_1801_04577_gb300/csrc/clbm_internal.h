@@ -173,7 +173,8 @@ struct NuLink {
 // ---------------------------------------------------------------------------
 // Batched solves: many independent lattices advanced by the same launches.
 // ---------------------------------------------------------------------------
-constexpr int kBatchGroups = 3;  // tile width 32, 64, 128 nodes
+constexpr int kBatchWidths = 3;                 // tile width 32, 64, 128 nodes
+constexpr int kBatchGroups = 2 * kBatchWidths;  // without a mask, with one
 
 // One lattice of a batch as the batched kernels see it.
 struct BatchLat {
@@ -233,9 +234,9 @@ struct Launchers {
   cudaError_t (*totals)(const DevGeom& g, const void* buf, double* partials, int nblocks,
                         cudaStream_t s);
   size_t elem_bytes;
-  // batched interior step over a tile list (tile = {lattice, row, first x, 0}; tiles skip the
+  // batched step over a tile list (tile = {lattice, row, first x, 0}; with a mask the tiles skip the
   // first and last column); V = nodes per lane
-  cudaError_t (*batch_step)(int V, const BatchLat* lats, const int4* tiles, const int* count,
+  cudaError_t (*batch_step)(int V, int masked, const BatchLat* lats, const int4* tiles, const int* count,
                             int parity, const long long* t, int tstep, int stochastic, int grid,
                             cudaStream_t s);
   // batched boundary nodes: entries {lattice, node index}, skipped when the lattice is inactive
@@ -243,7 +244,7 @@ struct Launchers {
                                 int parity, const long long* t, int tstep, int stochastic,
                                 cudaStream_t s);
   // persistent grid size (blocks) of the batched interior step for V
-  int (*batch_grid)(int V);
+  int (*batch_grid)(int V, int masked);
   // a <- (a + b) / 2 over n stored values (all planes)
   cudaError_t (*average)(void* a, const void* b, long long n, cudaStream_t s);
 

@@ -1448,16 +1448,25 @@ __global__ void __launch_bounds__(kRedThreads)
 // lattice, row, x), so it stays on one lattice for many tiles; the lattice's
 // descriptor is copied into a per-warp shared-memory slot when it changes and
 // read from there, instead of chasing it through global memory on every tile.
-// Tiles cover only the rows that are not boundary rows and skip the first and
-// last column: those nodes belong to the boundary launch that follows.
-template <typename S, int V, bool VH>
-__global__ void __launch_bounds__(kStepThreads, 4)
+// MASKED: tiles cover only the rows that are not boundary rows and skip the
+// first and last column: those nodes belong to the boundary launch that
+// follows.  Otherwise every node is final (box_tile), and the lattice's
+// constants are read from shared memory where they are used, which leaves
+// registers for five blocks a multiprocessor where the step is not bound by
+// memory alone (64 cavities of 32 .. 512: FP32 202 -> 185 us a step, with five
+// blocks 201; FP16 179 -> 156 us, with four blocks 168).
+template <typename S, int V, bool MASKED>
+constexpr int kBatchBlocks = MASKED || sizeof(S) == 8 || (V == Traits<S>::V && sizeof(S) == 4) ? 4 : 5;
+
+template <typename S, int V, bool MASKED>
+__global__ void __launch_bounds__(kStepThreads, (kBatchBlocks<S, V, MASKED>))
     batch_step_kernel(const BatchLat* __restrict__ lats, const int4* __restrict__ tiles,
                       const int* __restrict__ count, int parity, const long long* __restrict__ tptr,
                       int tstep, int stochastic) {
   using R = typename Traits<S>::R;
   static_assert(sizeof(BatchLat) % 8 == 0, "descriptor is copied in 8-byte words");
   __shared__ BatchLat slot[kStepThreads / 32];
+  __shared__ Co<R> coef[MASKED ? 1 : kStepThreads / 32];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const long long n = *count;
@@ -1482,15 +1491,25 @@ __global__ void __launch_bounds__(kStepThreads, 4)
       for (int k = lane; k < (int)(sizeof(BatchLat) / 8); k += 32) to[k] = from[k];
       __syncwarp();
       cur = tl.x;
-      c = make_co<R>(L.c);
+      if constexpr (MASKED) {
+        c = make_co<R>(L.c);
+      } else {
+        if (lane == 0) coef[wib] = make_co<R>(L.c);
+        __syncwarp();
+      }
     }
-    step_tile<S, V, true, VH>(L.g, c, static_cast<const S*>(L.buf[parity]),
-                              static_cast<S*>(L.buf[parity ^ 1]), tl.y, tl.z, lane, seed,
-                              stochastic);
+    const S* src = static_cast<const S*>(L.buf[parity]);
+    S* dst = static_cast<S*>(L.buf[parity ^ 1]);
+    if constexpr (MASKED) {
+      step_tile<S, V, true, false>(L.g, c, src, dst, tl.y, tl.z, lane, seed, stochastic);
+    } else {
+      // one copy of the tile: rows of a few hundred nodes are mostly edge tiles anyway
+      box_tile<S, V, false, true, true>(L.g, coef[wib], src, dst, tl.y, tl.z, lane, seed, stochastic);
+    }
   }
 }
 
-// Boundary nodes of every active lattice of a batch: entries {lattice, node}.
+// Boundary nodes of every active lattice of a batch that has a mask: entries {lattice, node}.
 template <typename S>
 __global__ void __launch_bounds__(kRedThreads)
     batch_boundary_kernel(const BatchLat* __restrict__ lats, const int2* __restrict__ entries,
@@ -1509,10 +1528,7 @@ __global__ void __launch_bounds__(kRedThreads)
     const Co<R> c = make_co<R>(L->c);
     const S* src = static_cast<const S*>(L->buf[parity]);
     S* dst = static_cast<S*>(L->buf[parity ^ 1]);
-    if (L->g.flags)
-      step_node<S, true>(L->g, c, src, dst, e.y, seed, stochastic);
-    else
-      step_node<S, false>(L->g, c, src, dst, e.y, seed, stochastic);
+    step_node<S, true>(L->g, c, src, dst, e.y, seed, stochastic);
   }
 }
 
@@ -1730,25 +1746,27 @@ struct LaunchImpl {
     return cudaGetLastError();
   }
 
+  // batches run without the viscous source (clbm_batch_create rejects it)
   template <int VV>
-  static cudaError_t batch_launch(const BatchLat* lats, const int4* tiles, const int* count,
-                                  int parity, const long long* t, int tstep, int stochastic, int grid,
-                                  cudaStream_t s) {
-    // batches run without the viscous source (clbm_batch_create rejects it)
-    batch_step_kernel<S, VV, false><<<grid, kStepThreads, 0, s>>>(lats, tiles, count, parity, t,
-                                                                   tstep, stochastic);
-    return cudaGetLastError();
+  static const void* batch_kernel(int masked) {
+    return masked ? (const void*)batch_step_kernel<S, VV, true> : (const void*)batch_step_kernel<S, VV, false>;
+  }
+  static const void* batch_kernel_of(int v, int masked) {
+    if (v == 1) return batch_kernel<1>(masked);
+    if (v == 2) return batch_kernel<2>(masked);
+    if constexpr (V >= 4) {
+      if (v == 4) return batch_kernel<4>(masked);
+    }
+    return nullptr;
   }
 
-  static cudaError_t batch_step(int v, const BatchLat* lats, const int4* tiles, const int* count,
+  static cudaError_t batch_step(int v, int masked, const BatchLat* lats, const int4* tiles, const int* count,
                                 int parity, const long long* t, int tstep, int stochastic, int grid,
                                 cudaStream_t s) {
-    if (v == 1) return batch_launch<1>(lats, tiles, count, parity, t, tstep, stochastic, grid, s);
-    if (v == 2) return batch_launch<2>(lats, tiles, count, parity, t, tstep, stochastic, grid, s);
-    if constexpr (V >= 4) {
-      if (v == 4) return batch_launch<4>(lats, tiles, count, parity, t, tstep, stochastic, grid, s);
-    }
-    return cudaErrorInvalidValue;
+    const void* k = batch_kernel_of(v, masked);
+    if (!k) return cudaErrorInvalidValue;
+    void* args[] = {&lats, &tiles, &count, &parity, &t, &tstep, &stochastic};
+    return cudaLaunchKernel(k, dim3(grid), dim3(kStepThreads), args, 0, s);
   }
 
   static cudaError_t batch_boundary(const BatchLat* lats, const int2* entries, int n,
@@ -1762,24 +1780,12 @@ struct LaunchImpl {
     return cudaGetLastError();
   }
 
-  template <int VV>
-  static int grid_of() {
-    int per_sm = 0, dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_step_kernel<S, VV, false>,
-                                                      kStepThreads, 0) != cudaSuccess)
-      return 0;
-    return sms * (per_sm > 0 ? per_sm : 1);
-  }
-
-  static int batch_grid(int v) {
-    if (v == 1) return grid_of<1>();
-    if (v == 2) return grid_of<2>();
-    if constexpr (V >= 4) {
-      if (v == 4) return grid_of<4>();
-    }
-    return 0;
+  static int batch_grid(int v, int masked) {
+    int per_sm = 0;
+    const void* k = batch_kernel_of(v, masked);
+    if (!k) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kStepThreads, 0) != cudaSuccess) return 0;
+    return sm_count() * (per_sm > 0 ? per_sm : 1);
   }
 
   static cudaError_t batch_residual(const BatchLat* lats, const int* active, int* snap_valid,
