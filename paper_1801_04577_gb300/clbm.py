@@ -210,15 +210,16 @@ def clbm_field_shape(ctx):
 def _check_fields(ctx, bufs, on_device, what):
     """Every field array (not a raw address) must hold nx * rows FP64 values on
     the side `on_device` names: the library reads or writes all of them."""
-    if all(b is None or isinstance(b, int) for b in bufs):
-        return
-    nx, rows = clbm_field_shape(ctx)
+    nx = rows = 0
     for b in bufs:
         if b is None or isinstance(b, int):
             continue
+        if not rows:
+            nx, rows = clbm_field_shape(ctx)
         if hasattr(b, "data_ptr"):
-            ok = (b.numel() == nx * rows and str(b.dtype) == "torch.float64" and b.is_contiguous()
-                  and bool(b.is_cuda) == bool(on_device))
+            # (of torch's 8-byte types only float64 is floating point)
+            ok = (b.numel() == nx * rows and b.element_size() == 8 and b.dtype.is_floating_point
+                  and b.is_contiguous() and bool(b.is_cuda) == bool(on_device))
         else:
             ok = (not on_device and isinstance(b, np.ndarray) and b.size == nx * rows
                   and b.dtype == np.float64 and b.flags["C_CONTIGUOUS"])

@@ -110,6 +110,7 @@ struct ConvArgs {
   const bf16* w;     // packed weights: [N tile][slice][bn x 64], chunk order of pair_swapped
   int taps, bn, slices;
   int kper, ranges;  // slices per range of K, ranges
+  int mt;            // 128-position tiles of a block
   int stages;
   Epilogue epi;
   int* err;
@@ -126,11 +127,16 @@ constexpr int kMaxBn = 64;         // columns of a tile: a thread keeps its row'
 // warps where sums of several ranges are formed while the MMAs go on
 __host__ __device__ constexpr int conv_threads(bool ranges) { return ranges ? 192 : 128; }
 
-__host__ __device__ constexpr int conv_run(int taps, int Wp) { return tc::kBM + (taps == 9 ? 2 * Wp + 2 : 0); }
+constexpr int kMaxMt = 4;
+// positions of a block's input: its mt tiles and the rows above and below
+__host__ __device__ constexpr int conv_run(int taps, int Wp, int mt) {
+  return mt * tc::kBM + (taps == 9 ? 2 * Wp + 2 : 0);
+}
 // pairs of K chunks (the MMAs), rounded up to whole slices
 __host__ __device__ constexpr int conv_pairs(int C, int taps) { return (taps * C / 8 + 7) / 8 * 4; }
-__host__ __device__ constexpr int conv_smem(int C, int taps, int Wp, int bn, int stages) {
-  return (C / 8) * conv_run(taps, Wp) * 16 + stages * bn * 128 + conv_pairs(C, taps) * 8 + bn * 4 + 256;
+__host__ __device__ constexpr int conv_smem(int C, int taps, int Wp, int bn, int stages, int mt) {
+  return stages * bn * 128 + (C / 8) * conv_run(taps, Wp, mt) * 16 + conv_pairs(C, taps) * 8 +  // B, A, descriptors,
+         (2 * stages + 5) * 8 + 8 + bn * 4 + 64;                                                // barriers, slot, bias
 }
 
 // K chunk (eight channels of one tap) u = tap * groups + group; an MMA takes a
@@ -142,8 +148,9 @@ __host__ __device__ __forceinline__ bool pair_swapped(int u, int groups, int tot
   return groups > 1 ? u % groups == groups - 1 : u + 1 == total && u > 0;
 }
 
-// Implicit GEMM D[position][channel] of one 128-position tile (blockIdx.x) and
-// bn channels (blockIdx.y).  The matrix descriptors are made beforehand by all
+// Implicit GEMM D[position][channel] of mt 128-position tiles (blockIdx.x) and
+// bn channels (blockIdx.y).  The tiles of a block share its input (of one tile
+// alone, two thirds is halo at 128^2) and its weights.  The matrix descriptors are made beforehand by all
 // threads: one thread that divided by the number of channel groups for every
 // MMA took 20 us a tile.
 //
@@ -155,13 +162,13 @@ __host__ __device__ __forceinline__ bool pair_swapped(int u, int groups, int tot
 // instead of seven doubled its time).
 // Launch with conv_smem() bytes of dynamic shared memory.
 template <bool RANGES>
-__global__ void __launch_bounds__(conv_threads(RANGES)) conv_kernel(const __grid_constant__ ConvArgs a) {
+__global__ void __launch_bounds__(conv_threads(RANGES), RANGES ? 1 : 8) conv_kernel(const __grid_constant__ ConvArgs a) {
   constexpr int kConvThreads = conv_threads(RANGES);
   constexpr int kCopyWarp = RANGES ? 4 : 0, kMmaWarp = RANGES ? 5 : 1;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int groups = a.a.C / 8, Wp = a.a.W + 2;
-  const int run = conv_run(a.taps, Wp), total = a.taps * groups;
+  const int run = conv_run(a.taps, Wp, RANGES ? 1 : a.mt), total = a.taps * groups;
   uint8_t* B = smem;
   uint8_t* A = smem + a.stages * a.bn * 128;
   uint64_t* desc = reinterpret_cast<uint64_t*>(A + groups * run * 16);
@@ -172,8 +179,9 @@ __global__ void __launch_bounds__(conv_threads(RANGES)) conv_kernel(const __grid
   uint64_t* bar_f = bar_d + 2;         // [2] ... and has been read
   uint32_t* slot = reinterpret_cast<uint32_t*>(bar_f + 2);
   float* bias = reinterpret_cast<float*>(slot + 2);  // [bn]
-  const int m0 = blockIdx.x * tc::kBM, n0 = blockIdx.y * a.bn;
-  const uint32_t ncols = tc::tmem_cols(RANGES ? 2 * a.bn : a.bn);
+  const int mt = RANGES ? 1 : a.mt;
+  const int m0 = blockIdx.x * mt * tc::kBM, n0 = blockIdx.y * a.bn;
+  const uint32_t ncols = tc::tmem_cols(RANGES ? 2 * a.bn : mt * a.bn);
 
   if (warp == 0) tc::tmem_alloc(slot, ncols);
   if (tid == 32) {
@@ -210,9 +218,6 @@ __global__ void __launch_bounds__(conv_threads(RANGES)) conv_kernel(const __grid
   const uint32_t tmem = *slot;
   bool failed = false;
   float sum[RANGES ? kMaxBn : 1];
-  const int pos = m0 + tid;
-  int n = 0, p = 0;
-  const bool inside = tid < tc::kBM && a.epi.locate(pos, n, p);
 
   if (warp == kCopyWarp) {
     const bf16* w = a.w + (long long)blockIdx.y * a.slices * a.bn * 64;
@@ -267,9 +272,13 @@ __global__ void __launch_bounds__(conv_threads(RANGES)) conv_kernel(const __grid
           tc::fence_after();
           const uint64_t bdesc = tc::smem_desc(tc::smem_u32(B) + s * a.bn * 128, 128, 1024);
           const int m = min(4, pairs - 4 * i);
+#pragma unroll 1
+          for (int u = 0; u < mt; ++u)  // tile u lies 128 positions further (in units of 16 bytes)
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (j < m) tc::mma_bf16(acc, desc[4 * i + j], bdesc + j * 16, idesc, (i > s0 || j > 0) ? 1u : 0u);
+            for (int j = 0; j < 4; ++j)
+              if (j < m)
+                tc::mma_bf16(acc + u * a.bn, desc[4 * i + j] + u * tc::kBM, bdesc + j * 16, idesc,
+                             (i > s0 || j > 0) ? 1u : 0u);
           tc::mma_commit(&bar_m[s]);
         }
         tc::mma_commit(&bar_d[z & 1]);
@@ -308,24 +317,30 @@ __global__ void __launch_bounds__(conv_threads(RANGES)) conv_kernel(const __grid
   } else if (warp < 4) {
     pdl_wait();
     tc::fence_after();
+#pragma unroll 1
+    for (int u = 0; u < mt; ++u) {
+      const int pos = m0 + u * tc::kBM + tid;
+      int n, p;
+      const bool inside = a.epi.locate(pos, n, p);
 #pragma unroll
-    for (int c0 = 0; c0 < kMaxBn; c0 += 16) {
-      if (c0 >= a.bn) break;
-      float v[16];
-      if constexpr (RANGES) {
+      for (int c0 = 0; c0 < kMaxBn; c0 += 16) {
+        if (c0 >= a.bn) break;
+        float v[16];
+        if constexpr (RANGES) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = sum[c0 + k];
-      } else {
-        tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-      }
-      if (!inside) continue;
+          for (int k = 0; k < 16; ++k) v[k] = sum[c0 + k];
+        } else {
+          tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(u * a.bn + c0), v);
+        }
+        if (!inside) continue;
 #pragma unroll
-      for (int h = 0; h < 16; h += 8) {
-        if (n0 + c0 + h >= a.epi.channels) break;
-        float x[8];
+        for (int h = 0; h < 16; h += 8) {
+          if (n0 + c0 + h >= a.epi.channels) break;
+          float x[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] = v[h + k];
-        a.epi.apply(pos, n, p, n0 + c0 + h, x, bias + c0 + h);
+          for (int k = 0; k < 8; ++k) x[k] = v[h + k];
+          a.epi.apply(pos, n, p, n0 + c0 + h, x, bias + c0 + h);
+        }
       }
     }
   }

@@ -800,7 +800,7 @@ struct clbm_net {
   // of eight.  Operands of the activations and of their gradients, per buffer (base nullptr: none).
   bool direct = false;
   std::vector<conv::Op> aop, gop;
-  std::vector<void*> op_mem;
+  void* op_mem = nullptr;
   // Weight gradients run beside the chain of input gradients on streams of their own (branches of
   // the captured graph), each layer with its own partial sums.
   static constexpr int kSides = 3;
@@ -942,11 +942,14 @@ int direct_bn(int sms, int N, long long positions) {
   return width(t);
 }
 
-// Stages of weights beside the input tile (0: the tile does not fit).
-int conv_stages(int C, int taps, int W, int bn) {
-  for (int s = 4; s >= 2; --s)
-    if (conv::conv_smem(C, taps, W + 2, bn, s) <= kMaxSmem) return s;
-  return 0;
+// Whether a tile of a convolution and two stages of its weights fit shared memory.
+bool conv_fits(int C, int taps, int W, int bn) { return conv::conv_smem(C, taps, W + 2, bn, 2, 1) <= kMaxSmem; }
+
+// Stages of weights beside the input tile (16 stages measured no faster than 4).
+int conv_stages(int C, int taps, int W, int bn, int slices, int mt) {
+  for (int s = std::max(2, std::min(slices, 4)); s > 2; --s)
+    if (conv::conv_smem(C, taps, W + 2, bn, s, mt) <= kMaxSmem) return s;
+  return 2;
 }
 
 struct ConvSplit {
@@ -996,12 +999,18 @@ cudaError_t conv_direct(clbm_net* net, const conv::Op& a, int layer, int transpo
   c.slices = d.slices;
   c.kper = r.kper;
   c.ranges = r.splits;
-  c.stages = std::min(conv_stages(a.C, taps, a.W, d.bn), std::max(2, d.slices));
+  const int tiles = (int)((op_positions(a, N) + tc::kBM - 1) / tc::kBM), ntiles = (d.N + d.bn - 1) / d.bn;
+  // as many tiles a block as leave three blocks to a multiprocessor, in number and in memory
+  c.mt = 1;
+  while (r.splits == 1 && 2 * c.mt <= conv::kMaxMt && tiles * ntiles >= 6 * c.mt * net->sms &&
+         2 * c.mt * d.bn <= 128 && conv::conv_smem(a.C, taps, a.W + 2, d.bn, 4, 2 * c.mt) <= kMaxSmem / 3)
+    c.mt *= 2;
+  c.stages = conv_stages(a.C, taps, a.W, d.bn, d.slices, c.mt);
   c.epi = e;
   c.err = net->d_tflag;
-  const dim3 grid((unsigned)((op_positions(a, N) + tc::kBM - 1) / tc::kBM), (unsigned)((d.N + d.bn - 1) / d.bn));
+  const dim3 grid((unsigned)((tiles + c.mt - 1) / c.mt), (unsigned)ntiles);
   return launch_dependent(r.splits > 1 ? conv::conv_kernel<true> : conv::conv_kernel<false>, grid,
-                          conv::conv_threads(r.splits > 1), conv::conv_smem(a.C, taps, a.W + 2, d.bn, c.stages), net->stream, c);
+                          conv::conv_threads(r.splits > 1), conv::conv_smem(a.C, taps, a.W + 2, d.bn, c.stages, c.mt), net->stream, c);
 }
 
 // Launch shape of a weight gradient.
@@ -1469,8 +1478,8 @@ bool direct_fits(const std::vector<Conv>& convs, const clbm_net_config& c) {
   if (c.base % 8 != 0 || c.in_ch > 8 || c.out_ch > 8) return false;
   for (const Conv& cv : convs) {
     const int taps = cv.ks * cv.ks;
-    if (cv.ci % 8 == 0 && !conv_stages(cv.ci, taps, cv.W, conv::kMaxBn)) return false;
-    if (cv.co % 8 == 0 && !conv_stages(cv.co, taps, cv.W, conv::kMaxBn)) return false;
+    if (cv.ci % 8 == 0 && !conv_fits(cv.ci, taps, cv.W, conv::kMaxBn)) return false;
+    if (cv.co % 8 == 0 && !conv_fits(cv.co, taps, cv.W, conv::kMaxBn)) return false;
     conv::Op x{};
     x.C = (cv.ci + 7) / 8 * 8;
     x.H = x.W = cv.H;
@@ -1486,40 +1495,41 @@ cudaError_t make_operands(clbm_net* n) {
   const int L = n->cfg.levels;
   n->aop.assign(n->act_c.size(), conv::Op{});
   n->gop.assign(n->act_c.size(), conv::Op{});
+  size_t total = 0;
+  std::vector<std::pair<conv::Op*, size_t>> all;  // tensors and their offsets in one allocation
   auto make = [&](conv::Op& o, int C, int hw) {
     o.C = (C + 7) / 8 * 8;
     o.H = o.W = hw;
-    // guards: a tile reads Wp + 1 positions before position 0 and past its 128 positions
-    const long long front = o.Wp() + 8, tail = o.Wp() + 8 + tc::kBM;
+    // guards: a block reads Wp + 1 positions before position 0 and past its last tile
+    const long long front = o.Wp() + 8, tail = o.Wp() + 8 + conv::kMaxMt * tc::kBM;
     o.pst = front + (long long)n->cfg.max_batch * o.Pn() + tail;
-    const size_t bytes = (size_t)(o.C / 8) * o.pst * 16;
-    void* m = nullptr;
-    cudaError_t e = cudaMalloc(&m, bytes);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return e;
-    }
-    n->op_mem.push_back(m);
-    o.base = static_cast<__nv_bfloat16*>(m) + front * 8;
-    return cudaMemsetAsync(m, 0, bytes, n->stream);
+    all.emplace_back(&o, total + front * 16);
+    total += ((size_t)(o.C / 8) * o.pst * 16 + 255) / 256 * 256;
   };
-  cudaError_t e = cudaSuccess;
   auto both = [&](int id) {
-    if (!e) e = make(n->aop[id], n->act_c[id], n->act_hw[id]);
-    if (!e) e = make(n->gop[id], n->act_c[id], n->act_hw[id]);
+    make(n->aop[id], n->act_c[id], n->act_hw[id]);
+    make(n->gop[id], n->act_c[id], n->act_hw[id]);
   };
-  if (!e) e = make(n->aop[P.in], n->act_c[P.in], n->act_hw[P.in]);
-  if (!e) e = make(n->gop[P.out], n->act_c[P.out], n->act_hw[P.out]);
+  make(n->aop[P.in], n->act_c[P.in], n->act_hw[P.in]);
+  make(n->gop[P.out], n->act_c[P.out], n->act_hw[P.out]);
   for (int l = 0; l < L - 1; ++l) {
     both(P.a1[l]);
     both(P.d1[l]);
     both(P.d2[l]);
-    if (!e) e = make(n->aop[P.pool[l]], n->act_c[P.pool[l]], n->act_hw[P.pool[l]]);
-    if (!e) e = make(n->aop[P.cat[l]], n->act_c[P.cat[l]], n->act_hw[P.cat[l]]);
-    if (!e) e = make(n->gop[P.cat[l]], n->cfg.base << l, n->act_hw[P.cat[l]]);  // the skip part
+    make(n->aop[P.pool[l]], n->act_c[P.pool[l]], n->act_hw[P.pool[l]]);
+    make(n->aop[P.cat[l]], n->act_c[P.cat[l]], n->act_hw[P.cat[l]]);
+    make(n->gop[P.cat[l]], n->cfg.base << l, n->act_hw[P.cat[l]]);  // the skip part
   }
   both(P.b1);
   both(P.b2);
+  cudaError_t e = cudaMalloc(&n->op_mem, total);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    n->op_mem = nullptr;
+    return e;
+  }
+  for (auto& t : all) t.first->base = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(n->op_mem) + t.second);
+  e = cudaMemsetAsync(n->op_mem, 0, total, n->stream);
   if (!e) e = cudaFuncSetAttribute(conv::conv_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (!e) e = cudaFuncSetAttribute(conv::conv_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (!e) e = cudaFuncSetAttribute(conv::dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
@@ -1543,7 +1553,7 @@ clbm_status clbm_net_destroy(clbm_net* n) {
   cudaFree(n->pt);
   for (float* a : n->act) cudaFree(a);
   for (float* a : n->gact) cudaFree(a);
-  for (void* a : n->op_mem) cudaFree(a);
+  cudaFree(n->op_mem);
   cudaFree(n->dw_part);
   for (cudaEvent_t ev : n->events) cudaEventDestroy(ev);
   for (cudaStream_t st : n->side)
