@@ -721,7 +721,21 @@ __device__ __forceinline__ void step_tile(const DevGeom& g, const Co<typename Tr
   // belongs to the last column, which the boundary update recomputes.  (The
   // 16-bit single-lattice kernels leave it off: the extra live state costs
   // them register spills, more than the padding they would skip.)
-  const bool live = !SKIP_DEAD || x0 < g.nx;
+  uint16_t fl[V];  // flags of the lane's nodes in a tile that holds flagged ones
+#pragma unroll
+  for (int k = 0; k < V; ++k) fl[k] = 0;
+  bool solid = false;  // ... all of them solid: such a lane, too, neither loads nor stores
+  if constexpr (MASKSTORE) {
+    if (mixed) {
+      using Raw = typename RawOf<2 * V>::T;
+      const Raw r = *reinterpret_cast<const Raw*>(g.flags + (long long)y * g.pitch + x0);
+      memcpy(fl, &r, sizeof(Raw));
+      solid = true;
+#pragma unroll
+      for (int k = 0; k < V; ++k) solid = solid && (fl[k] & kFlagSolid);
+    }
+  }
+  const bool live = !SKIP_DEAD || (x0 < g.nx && !solid);
 
   R v[14][V];
 #pragma unroll
@@ -776,12 +790,11 @@ __device__ __forceinline__ void step_tile(const DevGeom& g, const Co<typename Tr
     // a tile holding flagged nodes (solid, or fluid next to a wall) leaves them,
     // and the edge columns, to the boundary update of the same launch
     if (mixed) {
-      const uint16_t* fp = g.flags + (long long)y * g.pitch + x0;
       uint32_t skip = 0;
 #pragma unroll
       for (int k = 0; k < V; ++k) {
         const int x = x0 + k;
-        if (fp[k] != 0 || x == 0 || x == g.nx - 1) skip |= 1u << k;
+        if (fl[k] != 0 || x == 0 || x == g.nx - 1) skip |= 1u << k;
       }
       if (skip) {
 #pragma unroll

@@ -5,20 +5,19 @@ namespace clbm {
 
 const Launchers kLaunchF64 = LaunchImpl<double>::table();
 
-// One block adds nblocks rows of `width` partials in index order, so a
-// reduction gives the same bits on every run.
+// One block adds nblocks rows of W partials in index order, so a reduction
+// gives the same bits on every run.  All sums in one pass: one after another
+// they took the latency of W reductions (8 us of a small lattice's residual).
+template <int W>
 __global__ void __launch_bounds__(kRedThreads)
-    reduce_partials_kernel(const double* __restrict__ partials, int nblocks, int width,
-                           double* __restrict__ out) {
-  for (int k = 0; k < width; ++k) {
-    double acc[1] = {0.0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) acc[0] += partials[(long long)b * width + k];
-    __shared__ double tmp[1];
-    block_sum_store<1>(acc, tmp);
-    __syncthreads();
-    if (threadIdx.x == 0) out[k] = tmp[0];
-    __syncthreads();
-  }
+    reduce_partials_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
+  double acc[W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) acc[k] = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
+#pragma unroll
+    for (int k = 0; k < W; ++k) acc[k] += partials[(long long)b * W + k];
+  block_sum_store<W>(acc, out);
 }
 
 __global__ void advance_kernel(long long* t, int k) { *t += k; }
@@ -57,7 +56,12 @@ cudaError_t launch_halo(const HaloTable& t, cudaStream_t s) {
 
 cudaError_t launch_reduce_partials(const double* partials, int nblocks, int width, double* out,
                                    cudaStream_t s) {
-  reduce_partials_kernel<<<1, kRedThreads, 0, s>>>(partials, nblocks, width, out);
+  if (width == 8)
+    reduce_partials_kernel<8><<<1, kRedThreads, 0, s>>>(partials, nblocks, out);
+  else if (width == 2)
+    reduce_partials_kernel<2><<<1, kRedThreads, 0, s>>>(partials, nblocks, out);
+  else
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
