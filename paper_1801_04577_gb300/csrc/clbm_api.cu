@@ -707,18 +707,32 @@ static clbm_status capture_steps(clbm_ctx* c, int cur, int par, int len, cudaGra
 // Steps of one resident launch (about 4 ms).
 constexpr int kResidentSteps = 4096;
 
+// Whether a single lattice is faster in shared memory than in planes, with `nodes` nodes in each of
+// its bands (measured, us a step, resident / planes):
+//   FP64: an FP64 instruction takes a warp's quarter of the multiprocessor 64 cycles, so the work
+//         belongs on every multiprocessor: 32^2 (64 nodes a band) 7.0 / 8.1, 36^2 9.4 / 7.9
+//   with a mask the plane steps end in a tail of boundary nodes: 64^2 FP32 2.5 / 4.4, 200 x 100 2.9 /
+//         4.7, FP16 stochastic 4.9 / 6.0
+//   FP32: 32^2 1.5 / 3.3, 150^2 2.7 / 3.2
+//   16 bit: 64^2 2.2 / 2.9, 150^2 2.9 / 2.9, stochastic 110^2 3.0 / 3.4, 128^2 3.5 / 3.4; wide rows
+//         are stored into two bands a value at a time, 512 x 32 5.1 / 2.5
+static bool resident_pays(const clbm_ctx* c, int nodes) {
+  if (c->p.precision == CLBM_F64) return nodes <= 64;
+  if (c->d_flags) return c->p.nx <= 400;
+  if (c->p.precision == CLBM_F32) return c->p.nx <= 256;
+  return c->p.nx <= 160 && nodes <= (c->p.rounding ? 900 : 1400);
+}
+
 // Plan the resident steps of a single lattice: the most blocks a cluster can
 // have, so that each has the fewest nodes (a step's time is a block's latency).
-// FP64 stays with the plane kernels beyond 128 nodes a block: its arithmetic
-// needs the FP64 pipes of every multiprocessor.
 static bool resident_ready(clbm_ctx* c) {
   if (c->res.cl < 0) {
     ResPlan best;
     best.cl = 0;
     for (int cl = kMaxCluster; cl >= 1 && best.cl == 0; cl /= 2) {
-      if (c->p.precision == CLBM_F64 && (long long)c->p.nx * c->p.ny > 128LL * cl) break;
       ResPlan p;
-      if (resident_plan(c, cl, kMaxResidentSmem, kMaxResidentThreads, &p, nullptr) &&
+      if (resident_pays(c, (c->p.ny + cl - 1) / cl * c->p.nx) &&
+          resident_plan(c, cl, kMaxResidentSmem, kMaxResidentThreads, &p, nullptr) &&
           c->L->resident_clusters(cl, p.threads, p.smem, c->p.viscous_heating) > 0)
         best = p;
     }

@@ -105,6 +105,7 @@ struct clbm_batch {
   bool own_stream = false;
   void* arena[2] = {nullptr, nullptr};
   std::vector<clbm_ctx*> views;
+  std::vector<clbm_params> params;
   std::vector<int> nx, ny, py, masked, width, group;
   std::vector<long long> nodes;
   std::vector<int> grid;  // per group
@@ -242,7 +243,12 @@ static clbm_status launch_resident(clbm_batch* b, int K) {
 
 // Which lattices take their steps in shared memory.  A cluster per lattice, as
 // few blocks as leave two blocks to a multiprocessor (their barriers then
-// overlap); more blocks while the batch does not fill the device.
+// overlap); more blocks while the batch does not fill the device; lattices
+// that need a multiprocessor's whole memory for a block take sixteen such.
+// Measured, us a step, resident / tiles: 4 obstacle cavities of 64^2 FP32 2.7 /
+// 17, 64 of them 6.4 / 22, 256 of them 22 / 50; 256 plain ones 22 / 30; only
+// plain lattices with stochastic rounding and more than 900 nodes a band are
+// slower (64 of 128^2: 32 / 24).
 static clbm_status plan_resident(clbm_batch* b) {
   const int n = b->n;
   b->res_cl.assign(n, 0);
@@ -250,53 +256,61 @@ static clbm_status plan_resident(clbm_batch* b) {
   int dev = 0, sms = 0;
   BCUDA(b, cudaGetDevice(&dev));
   BCUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  std::vector<int> cl(n, 0);
+  constexpr size_t smem_of[2] = {kMaxResidentSmem / 2 - 1024, kMaxResidentSmem};  // per block: half, all
+  constexpr int threads_of[2] = {kMaxResidentThreads / 2, kMaxResidentThreads};
+  std::vector<int> cl(n, 0), whole(n, 0);
   long long blocks = 0;
+  auto fits = [&](int i, int c, int w) {
+    const clbm_params& p = b->params[i];
+    const ViewInfo v = describe_view(b->views[i]);
+    if (b->rounding && b->precision != CLBM_F32 && !v.g.flags && (p.ny + c - 1) / c * p.nx > 900) return false;
+    ResPlan r;
+    return resident_plan(b->views[i], c, smem_of[w], threads_of[w], &r, nullptr);
+  };
   for (int i = 0; i < n; ++i) {
-    for (int c = 1; c <= kMaxCluster && !cl[i]; c *= 2) {
-      ResPlan p;
-      if (resident_plan(b->views[i], c, kMaxResidentSmem / 2 - 1024, kMaxResidentThreads / 2, &p, nullptr)) cl[i] = c;
+    for (int c = 1; c <= kMaxCluster && !cl[i]; c *= 2)
+      if (fits(i, c, 0)) cl[i] = c;
+    if (!cl[i] && fits(i, kMaxCluster, 1)) {
+      cl[i] = kMaxCluster;
+      whole[i] = 1;
     }
-    blocks += cl[i];
+    blocks += cl[i] * (1 + whole[i]);
   }
   if (blocks == 0) return CLBM_OK;
   for (bool grown = true; grown;) {  // double the bands while every block still has its own slot
     grown = false;
-    for (int i = 0; i < n; ++i) {
-      ResPlan p;
-      if (cl[i] && cl[i] < kMaxCluster && blocks + cl[i] <= 2 * sms &&
-          resident_plan(b->views[i], 2 * cl[i], kMaxResidentSmem / 2 - 1024, kMaxResidentThreads / 2, &p, nullptr)) {
+    for (int i = 0; i < n; ++i)
+      if (cl[i] && !whole[i] && cl[i] < kMaxCluster && blocks + cl[i] <= 2 * sms && fits(i, 2 * cl[i], 0)) {
         blocks += cl[i];
         cl[i] *= 2;
         grown = true;
       }
-    }
   }
-  for (int c = 1; c <= kMaxCluster; c *= 2) {
-    clbm_batch::Resident r;
-    std::vector<ResLat> lats;
-    for (int i = 0; i < n; ++i) {
-      if (cl[i] != c) continue;
-      ResPlan p;
-      ResLat l;
-      resident_plan(b->views[i], c, kMaxResidentSmem / 2 - 1024, kMaxResidentThreads / 2, &p, &l);
-      l.L.snap = nullptr;
-      l.lat = i;
-      lats.push_back(l);
-      r.plan.cl = c;
-      r.plan.threads = std::max(r.plan.threads, p.threads);
-      r.plan.smem = std::max(r.plan.smem, p.smem);
+  for (int w = 0; w < 2; ++w)
+    for (int c = 1; c <= kMaxCluster; c *= 2) {
+      clbm_batch::Resident r;
+      std::vector<ResLat> lats;
+      for (int i = 0; i < n; ++i) {
+        if (cl[i] != c || whole[i] != w) continue;
+        ResPlan p;
+        ResLat l;
+        resident_plan(b->views[i], c, smem_of[w], threads_of[w], &p, &l);
+        l.lat = i;
+        lats.push_back(l);
+        r.plan.cl = c;
+        r.plan.threads = std::max(r.plan.threads, p.threads);
+        r.plan.smem = std::max(r.plan.smem, p.smem);
+      }
+      if (lats.empty() || b->L->resident_clusters(c, r.plan.threads, r.plan.smem, 0) < 1) continue;
+      r.n = (int)lats.size();
+      if (cudaMalloc(&r.d_lats, lats.size() * sizeof(ResLat)) != cudaSuccess) {
+        cudaGetLastError();
+        return CLBM_ENOMEM;
+      }
+      b->resident.push_back(r);
+      BCUDA(b, cudaMemcpy(r.d_lats, lats.data(), lats.size() * sizeof(ResLat), cudaMemcpyHostToDevice));
+      for (const ResLat& l : lats) b->res_cl[l.lat] = c;
     }
-    if (lats.empty() || b->L->resident_clusters(c, r.plan.threads, r.plan.smem, 0) < 1) continue;
-    r.n = (int)lats.size();
-    if (cudaMalloc(&r.d_lats, lats.size() * sizeof(ResLat)) != cudaSuccess) {
-      cudaGetLastError();
-      return CLBM_ENOMEM;
-    }
-    b->resident.push_back(r);
-    BCUDA(b, cudaMemcpy(r.d_lats, lats.data(), lats.size() * sizeof(ResLat), cudaMemcpyHostToDevice));
-    for (const ResLat& l : lats) b->res_cl[l.lat] = c;
-  }
   b->tiled = std::count(b->res_cl.begin(), b->res_cl.end(), 0) > 0;
   return CLBM_OK;
 }
@@ -445,6 +459,7 @@ clbm_status clbm_batch_create(const clbm_batch_item* items, int32_t n, int32_t a
     if (st != CLBM_OK) return bail(st);
     st = clbm_set_boundaries(b->views[i], it.solid, it.tbc, it.n_tbc, it.side_tbc, it.links, it.n_links);
     if (st != CLBM_OK) return bail(st);
+    b->params.push_back(it.params);
     b->nx.push_back(it.params.nx);
     b->ny.push_back(it.params.ny);
     b->py.push_back(it.params.periodic_y ? 1 : 0);
