@@ -520,7 +520,8 @@ __global__ void dw_sum_kernel(const float* __restrict__ part, int splits, int ta
 // ---------------------------------------------------------------------------
 // Element-wise passes in operand layout: one thread per position of the
 // smaller image and eight channels (blockIdx.y = channel group).  All of the
-// chain are launched as programmatic dependents.
+// chain are launched as programmatic dependents (all of the forward pass's
+// launches without their work 127 of 411 us at 128^2).
 // ---------------------------------------------------------------------------
 
 // FP32 NCHW (cs channels, C <= 8 of them from coff) -> one channel group, zero beyond C

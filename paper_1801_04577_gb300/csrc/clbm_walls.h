@@ -115,7 +115,12 @@ inline void link_heat(double b1, double b2, double b3, double ne, double q, bool
     return mid ? w : midpoint_temperature_q(q, w, T1, T2, have2, T3, have3, dirichlet);
   };
   const double w = weight(1, 0, 0, 0);  // of T_w
-  const double a = w * wall(0.0, 1, 0) + weight(0, 1, 0, 0);
+  // The weight on T1 is w b1 (...) + 3 (2q - 1) / 4q, two terms of order 1 / q whose
+  // difference stays bounded as q -> 0: in closed form off the half-way wall.
+  const double flux = b2 * ne, D = b1 * (1 + 2 * q) + flux * q * (1 + q);
+  const double a = mid || (dirichlet && q < 0.5) ? w * wall(0.0, 1, 0) + weight(0, 1, 0, 0)
+                   : have2 ? 0.75 * (b1 * (4 * q + 1) + (2 * q - 1) * (1 + q) * flux) / D
+                           : (b1 + (q - 0.5) * flux) / (b1 + flux * q);
   const double b = have2 ? w * wall(0.0, 0, 1) + weight(0, 0, 1, 0) : 0.0;
   const double d = have3 ? weight(0, 0, 0, 1) : 0.0;
   k[0] = cT2 * a;
