@@ -246,9 +246,10 @@ static clbm_status launch_resident(clbm_batch* b, int K) {
 // overlap); more blocks while the batch does not fill the device; lattices
 // that need a multiprocessor's whole memory for a block take sixteen such.
 // Measured, us a step, resident / tiles: 4 obstacle cavities of 64^2 FP32 2.7 /
-// 17, 64 of them 6.4 / 22, 256 of them 22 / 50; 256 plain ones 22 / 30; only
-// plain lattices with stochastic rounding and more than 900 nodes a band are
-// slower (64 of 128^2: 32 / 24).
+// 17, 64 of them 6.4 / 22, 256 of them 22 / 50; 256 plain ones 22 / 30.  Only
+// with stochastic rounding, no mask and rows that fill a tile are tiles faster,
+// once every multiprocessor has work (64 of 128^2 32 / 24, 16 of them 11.4 /
+// 10.4, 4 of them 5.3 / 6.4; 64 of 96^2 15.8 / 21.9, 256 of 64^2 23.8 / 27.0).
 static clbm_status plan_resident(clbm_batch* b) {
   const int n = b->n;
   b->res_cl.assign(n, 0);
@@ -259,11 +260,12 @@ static clbm_status plan_resident(clbm_batch* b) {
   constexpr size_t smem_of[2] = {kMaxResidentSmem / 2 - 1024, kMaxResidentSmem};  // per block: half, all
   constexpr int threads_of[2] = {kMaxResidentThreads / 2, kMaxResidentThreads};
   std::vector<int> cl(n, 0), whole(n, 0);
-  long long blocks = 0;
+  long long blocks = 0, total = 0;
+  for (const long long k : b->nodes) total += k;
   auto fits = [&](int i, int c, int w) {
     const clbm_params& p = b->params[i];
     const ViewInfo v = describe_view(b->views[i]);
-    if (b->rounding && b->precision != CLBM_F32 && !v.g.flags && (p.ny + c - 1) / c * p.nx > 900) return false;
+    if (b->rounding && b->precision != CLBM_F32 && !v.g.flags && p.nx > 112 && total > 1024LL * sms) return false;
     ResPlan r;
     return resident_plan(b->views[i], c, smem_of[w], threads_of[w], &r, nullptr);
   };
