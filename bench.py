@@ -39,10 +39,10 @@ from paper_1801_04577_gb300 import inputs as I  # noqa: E402
 
 HBM_FALLBACK_GBS = 6800.0
 # FP64 storage and collision are bound by the FP64 pipe, not by HBM.  FP64 operations per
-# lattice update of step_fused_kernel<double>, counted with ncu on the 2048 x 1024
-# Rayleigh-Benard lattice (sm__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on: 165.9 M
-# DFMA, 140.7 M DADD, 51.5 M DMUL per launch of 2,097,152 nodes; an FMA counts two): 249.8.
-FP64_FLOP_PER_LU = 249.8
+# lattice update of step_box_kernel<double>, counted with ncu on the 2048 x 1024
+# Rayleigh-Benard lattice (sm__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on: 178.3 M
+# DFMA, 104.9 M DADD, 45.1 M DMUL per launch of 2,097,152 nodes; an FMA counts two): 241.5.
+FP64_FLOP_PER_LU = 241.5
 # FP64 peak of the GB300: 152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07 GHz
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.07
 ELEM_BYTES = {"f64": 8, "f32": 4, "f16": 2, "bf16": 2}
@@ -53,11 +53,11 @@ DTYPE = {"f64": "f64", "f32": "f32", "f16": "f16-storage/f32-compute", "bf16": "
 # workload, valid only for the kernel source whose SHA-256 prefix is stored.
 NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum (1 pass) on the full 4096 x 2048
-    # lattice, three launches of step_fused_kernel each: FP32 479.30-479.34 MB read + 415.3-418.8 MB
-    # written; FP16 243.0-243.1 MB read + 189.3-191.8 MB written (the rest of the written lines
+    # lattice, three launches of step_box_kernel each: FP32 469.82-469.83 MB read + 413.8-417.5 MB
+    # written; FP16 234.9-235.0 MB read + 182.6-185.6 MB written (the rest of the written lines
     # is still dirty in L2 when the launch ends).
-    "f32:rb4096": {"bytes_per_launch": 896.1e6, "kernel_hash": "fc7666131524faae"},
-    "f16:rb4096": {"bytes_per_launch": 433.4e6, "kernel_hash": "fc7666131524faae"},
+    "f32:rb4096": {"bytes_per_launch": 885.3e6, "kernel_hash": "79600232252cd837"},
+    "f16:rb4096": {"bytes_per_launch": 418.6e6, "kernel_hash": "79600232252cd837"},
 }
 
 
@@ -273,21 +273,33 @@ def box_lattice(w) -> bool:
 
 
 def step_kernel_name(w) -> str:
-    """Box and masked lattices alike take one fused launch per step: the
-    listed boundary nodes in the first blocks, the interior warp tiles in the
-    rest (masked lattices skip tiles without fluid and leave flagged nodes to
-    the boundary blocks)."""
+    """One launch per step: box lattices in tiles that take walls and seams
+    themselves, masked ones with the listed boundary nodes in the first blocks
+    and the interior warp tiles in the rest (tiles without fluid are skipped,
+    flagged nodes left to the boundary blocks).  Small lattices stay in shared
+    memory for up to 4096 steps a launch."""
+    if resident_lattice(w):
+        return "resident_kernel (many steps a launch); FP64: step_box_kernel, one launch per step"
     if box_lattice(w):
-        return "step_fused_kernel (interior tiles + boundary nodes, one launch per step)"
+        return "step_box_kernel (tiles with walls inline, one launch per step)"
     return "step_fused_kernel<masked> (tile classes + listed boundary nodes, one launch per step)"
 
 
-def step_launches(w, steps: int, graph_levels: int = 5) -> int:
-    """Kernels that clbm_step(steps) launches: one fused launch per step.  A
+def resident_lattice(w) -> bool:
+    """Lattices that a cluster of blocks holds in shared memory, below FP64
+    (of the workloads here: the 64 x 64 cavity)."""
+    return w.params.nx * w.params.ny <= 64 * 64
+
+
+def step_launches(w, steps: int, graph_levels: int = 5, precision: str = "f32") -> int:
+    """Kernels that clbm_step(steps) launches: one launch per step, or one per
+    4096 steps of a lattice in shared memory.  A
     run of two or more steps replays captured graphs of 32, 16, ..., 2 steps
     (the binary digits of `steps`; a last odd step is launched on its own),
     each ending with one step-counter kernel, after one kernel that sets the
     counter."""
+    if steps >= 2 and resident_lattice(w) and precision != "f64":
+        return -(-steps // 4096)
     n = steps
     if steps >= 2:
         top = 1 << graph_levels
@@ -457,7 +469,7 @@ def run_native(args):
                           "peak_kind": peak_kind,
                           "algorithmic_bytes_per_launch": bytes_lu * nodes}),
             # slabs: one step launch per slab per step, plus (one process) one halo-copy launch
-            "gpu_launches": step_launches(w, args.steps) if mode == "single" else args.steps * (
+            "gpu_launches": step_launches(w, args.steps, precision=args.precision) if mode == "single" else args.steps * (
                 args.slabs + 1 if mode == "group" else 1),
             "residual_after": res}
     if e2e is not None:
@@ -508,9 +520,9 @@ def run_batch(args):
     widths = [b.tile_width(i) for i in range(len(ws))]
     K = (args.check_every + 1) // 2 * 2
     replays = -(-int(steps) // K)
-    # per step: one interior launch per tile-width group + the boundary launch;
-    # per replay: residual (2), update, scan, tile rebuild
-    launches = int(steps) * (len(set(widths)) + 1) + replays * 5
+    # per step: one launch per tile-width group; per replay: the lattices that stay in shared
+    # memory (all their steps), residual (2), update, scan, tile rebuild
+    launches = int(steps) * len(set(widths)) + replays * 6
     line = {"metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": 1,
             "steps": int(steps), "warmup": int(warm_steps), "ms_per_step": el / max(steps, 1) * 1e3,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
