@@ -681,7 +681,7 @@ def run_unet(args):
             # the activations' DRAM bytes; the tensor-core rate is reported beside it
             "roofline": {"bound": "hbm", "achieved": nbytes / (ms * 1e-3) / 1e9, "peak": hbm,
                          "unit": "GB/s", "frac": nbytes / (ms * 1e-3) / 1e9 / hbm, "traffic": None,
-                         "kernel": "tc::gemm_kernel (all convolution passes of a training step)",
+                         "kernel": "conv::conv_kernel, conv::dw_kernel (all convolution passes of a training step)",
                          "peak_kind": hbm_kind, "algorithmic_bytes_per_step": nbytes,
                          "roofline_ms": roof_ms, "roofline_time_frac": roof_ms / ms,
                          "tensor_tflops": achieved, "tensor_peak": peak, "tensor_frac": achieved / peak,
