@@ -1222,9 +1222,10 @@ bool resident_plan(const clbm_ctx* c, int cl, size_t max_smem, int max_threads, 
   const int nx = c->p.nx, ny = c->p.ny;
   if (c->slab || (cl > 1 && ny / cl < 2)) return false;
   const int rows = (ny + cl - 1) / cl;
-  if (cl > 1)  // the off-midpoint Dirichlet rule reads two nodes beyond its own: a ghost row holds one
-    for (const clbm_link& k : c->h_links)
-      if (k.dir <= 4 && k.q < 0.5 && c->h_tbc[k.tbc].b1 == 0.0) return false;
+  for (const clbm_link& k : c->h_links)
+    if (k.dir <= 4 && reads_third(k.dir, k.q, c->h_tbc[k.tbc].b1) &&
+        !band_holds_third(k.node / nx, k.dir, ny, cl, c->gpy != 0))
+      return false;
   int off[kMaxCluster + 1], most = 0;
   const std::vector<int32_t>& v = c->h_bnodes;  // ascending
   for (int r = 0; r <= cl; ++r)

@@ -144,4 +144,21 @@ inline void link_bounce(double q, bool have2, double (&k)[3]) {
   }
 }
 
+// The thermal rule of an axis link off the midpoint, q < 1/2, at a Dirichlet
+// wall (b1 = 0) reads the third node x_f - 2 e_i: its row, for the link `dir`
+// (1..4) of a node in row y.
+inline bool reads_third(int dir, double q, double b1) { return dir <= 4 && q < 0.5 && b1 == 0.0; }
+inline int third_row(int y, int dir) { return y - (dir == 2 ? 2 : dir == 4 ? -2 : 0); }
+
+// Whether the resident steps can evaluate that rule.  A band keeps one ghost
+// row on either side, and of it only what streams across is kept up to date
+// away from walls, so the third node must lie among the band's own rows.  Several
+// bands: refused.  One band: all rows are its own, but across the seam of a
+// periodic y axis the node would be a ghost row's or lie beyond it; beyond a wall
+// there is no third node (link_heat's have3).
+inline bool band_holds_third(int y, int dir, int ny, int cl, bool py) {
+  const int y3 = third_row(y, dir);
+  return cl == 1 && (!py || (y3 >= 0 && y3 < ny));
+}
+
 }  // namespace clbm
