@@ -69,6 +69,7 @@ struct clbm_ctx {
   std::vector<clbm_link> h_links;  // links of own-row nodes, node = stored row * nx + x
   int side_tbc[4] = {-1, -1, -1, -1};
   double side_k[4][2][3] = {};  // link_heat of the box sides without / with a second node
+  float side_kf[4][2][3] = {};  // ... rounded to FP32
   double side_u[4][2] = {};  // moving box sides (clbm_set_wall_velocity)
   // scratch
   double* d_fields = nullptr;  // 4 * nx * ny doubles, allocated on first use
@@ -138,9 +139,7 @@ static DevGeom make_geom(const clbm_ctx* c) {
   g.tiles_per_row = c->tiles_per_row;
   g.pad_tiles = 0;
   std::memcpy(g.side_k, c->side_k, sizeof(g.side_k));
-  for (int sd = 0; sd < 4; ++sd)
-    for (int two = 0; two < 2; ++two)
-      for (int m = 0; m < 3; ++m) g.side_kf[sd][two][m] = (float)c->side_k[sd][two][m];
+  std::memcpy(g.side_kf, c->side_kf, sizeof(g.side_kf));
   g.moving = 0;
   g.pad_moving = 0;
   for (int sd = 0; sd < 4; ++sd)
@@ -482,6 +481,7 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
       }
       return !is_solid(x, y);
     };
+    const DevCoef co = make_coef(c);
     std::vector<uint16_t> flags;
     std::vector<int32_t> slot_pitch;
     std::vector<double> lk_t(lk_tbc.size() * 4, 0.0), lk_f(lk_tbc.size() * 6, 0.0);
@@ -545,7 +545,16 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
                 double kt[4];
                 link_heat(b.b1, b.b2, b.b3, lk_ne[4 * s + i - 1], q, have2, fluid_at(x + 2 * dx, y + 2 * dy),
                           c->p.T0, 0.5 * c->p.Q, c->p.cT2, kt);
-                for (int m = 0; m < 4; ++m) lk_t[(size_t)16 * s + 4 * (i - 1) + m] = kt[m];
+                double* const to = &lk_t[(size_t)16 * s + 4 * (i - 1)];
+                auto put = [&](const auto& rates, auto type) {
+                  decltype(type) r[4];
+                  round_heat(kt, b.b2, heat_share(rates), r);
+                  for (int m = 0; m < 4; ++m) to[m] = r[m];
+                };
+                if (c->p.precision == CLBM_F64)
+                  put(co.kd, 0.0);
+                else
+                  put(co.kf, 0.0f);
               }
             }
           }
@@ -588,12 +597,16 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
     for (int s = 0; s < 4; ++s) {
       c->side_tbc[s] = sides[s];
       for (int two = 0; two < 2; ++two) {
-        double k[4] = {0, 0, 0, 0};
+        double k[4] = {0, 0, 0, 0}, kd[4] = {0, 0, 0, 0};
+        float kf[4] = {0, 0, 0, 0};
         if (sides[s] >= 0) {
           const clbm_tbc& b = tbc[sides[s]];
           link_heat(b.b1, b.b2, b.b3, 1.0, 0.5, two != 0, false, c->p.T0, 0.5 * c->p.Q, c->p.cT2, k);
+          round_heat(k, b.b2, heat_share(co.kd), kd);
+          round_heat(k, b.b2, heat_share(co.kf), kf);
         }
-        std::copy(k, k + 3, c->side_k[s][two]);
+        std::copy(kd, kd + 3, c->side_k[s][two]);
+        std::copy(kf, kf + 3, c->side_kf[s][two]);
       }
     }
     c->h_solid = std::move(sol);

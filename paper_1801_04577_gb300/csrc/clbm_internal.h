@@ -79,6 +79,13 @@ struct CollideK {
   T srcq2, srct2, srcQ;      // (1 - l2 / 2) cT2 / 2, l2 cT2 / 2, srcq2 Q
 };
 
+// (h_1 + h_3) / (T - T0) of a uniform state at rest that the collision leaves as it is: G20 =
+// l2m2 (2 G20) + srct2 (T - T0), with the constants as rounded.
+template <typename T>
+inline double heat_share(const CollideK<T>& k) {
+  return 2.0 * (double)k.srct2 / (1.0 - 2.0 * (double)k.l2m2);
+}
+
 struct DevCoef {
   double s_nu, s_b, s3, s4, l0, l1, l2;
   double rho0, T0, gbeta, Fvx, Fvy, Q, cT2;
