@@ -444,14 +444,11 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
       if (solid && solid[k.node]) return fail(c, CLBM_EINVAL, "wall link from a solid node");
       const int y = gy - c->y0 + c->ylo;  // stored row (whole lattices: y0 = ylo = 0)
       if (y < c->ylo || y >= c->yhi) continue;  // another slab's node
-      if (c->slab && axis && k.q < 0.5 && tbc[k.tbc].b1 == 0.0) {
-        // the off-midpoint Dirichlet rule reads T at x_f - 2 e_i: it must be stored
-        const int y3 = y + 2 * kEY[k.dir];
-        const int gy3 = gy + 2 * kEY[k.dir];
-        if ((y3 < 0 || y3 >= ny) && (gpy || (gy3 >= 0 && gy3 < NY)))
-          return fail(c, CLBM_EINVAL, "slab too thin for wall link " + std::to_string(l) +
-                                          ": its third node lies beyond the ghost row");
-      }
+      // the off-midpoint Dirichlet rule reads T at x_f - 2 e_i: it must be stored
+      if (c->slab && axis && reads_third(k.dir, k.q, tbc[k.tbc].b1) &&
+          !slab_holds_third(y, gy, k.dir, ny, NY, gpy))
+        return fail(c, CLBM_EINVAL, "slab too thin for wall link " + std::to_string(l) +
+                                        ": its third node lies beyond the ghost row");
       int32_t& s = slot_of[(size_t)y * nx + x];
       if (s < 0) {
         s = (int32_t)(lk_tbc.size() / 4);

@@ -171,6 +171,13 @@ inline void link_bounce(double q, bool have2, double (&k)[3]) {
 inline bool reads_third(int dir, double q, double b1) { return dir <= 4 && q < 0.5 && b1 == 0.0; }
 inline int third_row(int y, int dir) { return y - (dir == 2 ? 2 : dir == 4 ? -2 : 0); }
 
+// Whether a slab that stores `ny` rows, its row y being row gy of a lattice of NY
+// rows, holds that node's row (its ghost rows are whole copies), or there is none.
+inline bool slab_holds_third(int y, int gy, int dir, int ny, int NY, bool py) {
+  const int y3 = third_row(y, dir), gy3 = third_row(gy, dir);
+  return (y3 >= 0 && y3 < ny) || (!py && (gy3 < 0 || gy3 >= NY));
+}
+
 // Whether the resident steps can evaluate that rule.  A band keeps one ghost
 // row on either side, and of it only what streams across is kept up to date
 // away from walls, so the third node must lie among the band's own rows.  Several

@@ -8,3 +8,6 @@ extern "C" int host_third_row(int y, int dir) { return clbm::third_row(y, dir); 
 extern "C" int host_band_holds_third(int y, int dir, int ny, int cl, int py) {
   return clbm::band_holds_third(y, dir, ny, cl, py != 0);
 }
+extern "C" int host_slab_holds_third(int y, int gy, int dir, int ny, int NY, int py) {
+  return clbm::slab_holds_third(y, gy, dir, ny, NY, py != 0);
+}

@@ -51,3 +51,17 @@ def test_one_band_reads_only_its_own_rows(harness, ny, py):
 def test_several_bands_are_refused(harness):
     assert not any(harness.host_band_holds_third(y, d, 32, cl, py)
                    for y in range(32) for d in (1, 2, 3, 4) for cl in (2, 4, 8, 16) for py in (0, 1))
+
+
+@pytest.mark.parametrize("py", [0, 1])
+@pytest.mark.parametrize("NY,y0,rows", [(9, 0, 9), (9, 0, 1), (9, 0, 2), (9, 3, 1), (9, 3, 2), (9, 3, 3), (9, 7, 2), (2, 1, 1)])
+def test_slabs_hold_the_third_node_or_refuse(harness, NY, y0, rows, py):
+    """A slab stores lattice rows y0 - 1 .. y0 + rows (around the seam of a
+    periodic axis).  The third node of a link lies two rows away from the wall."""
+    stored = range(y0 - 1, y0 + rows + 1)
+    for gy in range(y0, y0 + rows):
+        for d in (1, 2, 3, 4):
+            g3 = gy - 2 * EY[d]
+            none = not py and not 0 <= g3 < NY
+            ok = harness.host_slab_holds_third(gy - y0 + 1, gy, d, rows + 2, NY, py)
+            assert ok == (none or g3 in stored), (gy, d)
