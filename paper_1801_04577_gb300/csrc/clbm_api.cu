@@ -451,16 +451,18 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
                                         ": its third node lies beyond the ghost row");
       int32_t& s = slot_of[(size_t)y * nx + x];
       if (s < 0) {
+        if (lk_tbc.size() / 4 >= (size_t)kMaxLinkSlots)
+          return fail(c, CLBM_EINVAL, "more than 2^29 nodes with wall links");
         s = (int32_t)(lk_tbc.size() / 4);
         lk_ne.insert(lk_ne.end(), 4, 0.0);
         lk_tbc.insert(lk_tbc.end(), 4, -1);
         lk_q.insert(lk_q.end(), 8, 0.5);
       }
       if (axis) {
-        lk_ne[4 * s + k.dir - 1] = k.n_dot_e;
-        lk_tbc[4 * s + k.dir - 1] = k.tbc;
+        lk_ne[4LL * s + k.dir - 1] = k.n_dot_e;
+        lk_tbc[4LL * s + k.dir - 1] = k.tbc;
       }
-      lk_q[8 * s + k.dir - 1] = k.q;
+      lk_q[8LL * s + k.dir - 1] = k.q;
       clbm_link kk = k;
       kk.node = y * nx + x;
       kept.push_back(kk);
@@ -513,7 +515,7 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
               // a D2Q5 link into a solid needs a listed condition: link dir i = opp(j)
               if (j <= 4) {
                 const int s = slot_of[(size_t)y * nx + x];
-                if (s < 0 || lk_tbc[4 * s + kOpp[j] - 1] < 0)
+                if (s < 0 || lk_tbc[4LL * s + kOpp[j] - 1] < 0)
                   return fail(c, CLBM_EINVAL, "missing wall link at node " +
                                                   std::to_string((long long)grow(y) * nx + x) +
                                                   " dir " + std::to_string(kOpp[j]));
@@ -532,17 +534,17 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
             for (int i = 1; i < 9; ++i) {
               const int dx = -kEX[i], dy = -kEY[i];
               const bool have2 = fluid_at(x + dx, y + dy);
-              const double q = lk_q[8 * s + i - 1];
+              const double q = lk_q[8LL * s + i - 1];
               double kf[3];
               link_bounce(q, have2, kf);
-              for (int m = 0; m < 3; ++m) lk_f[(size_t)24 * s + 3 * (i - 1) + m] = kf[m];
+              for (int m = 0; m < 3; ++m) lk_f[bounce_entry(s, i) + m] = kf[m];
               if (kf[0] != 1.0) f |= kFlagOffMid;
-              if (i <= 4 && lk_tbc[4 * s + i - 1] >= 0) {
-                const clbm_tbc& b = tbc[lk_tbc[4 * s + i - 1]];
+              if (i <= 4 && lk_tbc[4LL * s + i - 1] >= 0) {
+                const clbm_tbc& b = tbc[lk_tbc[4LL * s + i - 1]];
                 double kt[4];
-                link_heat(b.b1, b.b2, b.b3, lk_ne[4 * s + i - 1], q, have2, fluid_at(x + 2 * dx, y + 2 * dy),
+                link_heat(b.b1, b.b2, b.b3, lk_ne[4LL * s + i - 1], q, have2, fluid_at(x + 2 * dx, y + 2 * dy),
                           c->p.T0, 0.5 * c->p.Q, c->p.cT2, kt);
-                double* const to = &lk_t[(size_t)16 * s + 4 * (i - 1)];
+                double* const to = &lk_t[heat_entry(s, i)];
                 auto put = [&](const auto& rates, auto type) {
                   decltype(type) r[4];
                   round_heat(kt, b.b2, heat_share(rates), r);

@@ -601,7 +601,7 @@ __device__ __forceinline__ void node_update(const DevGeom& g, const Co<R>& c, co
         kb = k[1];
         kc = k[2];
       } else {
-        const R* k = static_cast<const R*>(g.lk_t) + 16 * slot + 4 * ((b + 2) & 3);  // link opp(j)
+        const R* k = static_cast<const R*>(g.lk_t) + heat_entry(slot, ((b + 2) & 3) + 1);  // link opp(j)
         ka = __ldg(k);
         kb = __ldg(k + 1);
         kc = __ldg(k + 2);
@@ -635,7 +635,7 @@ __device__ __forceinline__ void node_update(const DevGeom& g, const Co<R>& c, co
     for (int j = 1; j < 9; ++j) {
       if (!(((wall & ~box) >> (j - 1)) & 1u)) continue;
       const int i = opp_of(j);
-      const R* k = static_cast<const R*>(g.lk_f) + 24 * slot + 3 * (i - 1);
+      const R* k = static_cast<const R*>(g.lk_f) + bounce_entry(slot, i);
       const R k0 = __ldg(k), k1 = __ldg(k + 1), k2 = __ldg(k + 2);
       R v = mul_(k2, to_r(src.at(j, own)));
       if (k1 != R(0)) v = fma_(k1, to_r(src.at(i, ahead(ex_of(j), ey_of(j), 1))), v);

@@ -1,5 +1,5 @@
 // Test harness: the host rules for wall links whose third node lies near the
-// edge of a band or slab, compiled for the host.  Not part of the library; built
+// edge of a band or slab, and the places of the link tables' entries, compiled for the host.  Not part of the library; built
 // by tests/test_bands_host.py.
 #include "../paper_1801_04577_gb300/csrc/clbm_walls.h"
 
@@ -11,3 +11,5 @@ extern "C" int host_band_holds_third(int y, int dir, int ny, int cl, int py) {
 extern "C" int host_slab_holds_third(int y, int gy, int dir, int ny, int NY, int py) {
   return clbm::slab_holds_third(y, gy, dir, ny, NY, py != 0);
 }
+extern "C" long long host_heat_entry(int slot, int dir) { return clbm::heat_entry(slot, dir); }
+extern "C" long long host_bounce_entry(int slot, int dir) { return clbm::bounce_entry(slot, dir); }

@@ -23,6 +23,7 @@ def harness(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     L = C.CDLL(out)
     L.host_reads_third.argtypes = [C.c_int, C.c_double, C.c_double]
+    L.host_heat_entry.restype = L.host_bounce_entry.restype = C.c_longlong
     return L
 
 
@@ -65,3 +66,12 @@ def test_slabs_hold_the_third_node_or_refuse(harness, NY, y0, rows, py):
             none = not py and not 0 <= g3 < NY
             ok = harness.host_slab_holds_third(gy - y0 + 1, gy, d, rows + 2, NY, py)
             assert ok == (none or g3 in stored), (gy, d)
+
+
+def test_link_table_entries_of_large_lattices(harness):
+    """Every entry its own place, also beyond 2^31 coefficients."""
+    for slot in (0, 1, 89478486, 134217728, 268435456, 2 ** 29 - 2):
+        heat = [harness.host_heat_entry(s, d) for s in (slot, slot + 1) for d in (1, 2, 3, 4)]
+        assert heat == list(range(16 * slot, 16 * (slot + 2), 4))
+        bounce = [harness.host_bounce_entry(s, d) for s in (slot, slot + 1) for d in range(1, 9)]
+        assert bounce == list(range(24 * slot, 24 * (slot + 2), 3))
