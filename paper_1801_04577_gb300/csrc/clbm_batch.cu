@@ -4,7 +4,8 @@
 // an ordinary clbm_ctx "view" over its slice of the arena, so boundaries,
 // initialisation, moments and Nusselt numbers reuse the single-lattice code.
 // A solve replays one CUDA graph per K steps: K launches (per launch group)
-// of the tile-list step kernel, the per-lattice residual, and three small
+// of the tile-list step kernel, beside them (branches) the launches of the
+// lattices that stay in shared memory, the per-lattice residual, and three small
 // kernels that retire converged lattices and rebuild the tile lists on the
 // device.  The host only reads back the active count after each replay.
 #include <cuda_runtime.h>
@@ -115,7 +116,10 @@ struct clbm_batch {
     ResPlan plan;
     int n = 0;
     ResLat* d_lats = nullptr;
+    cudaStream_t side = nullptr;  // the launch's branch of the captured solve
+    cudaEvent_t done = nullptr;
   };
+  cudaEvent_t fork = nullptr;  // where the branches begin (nullptr: one launch and nothing beside it)
   std::vector<Resident> resident;
   std::vector<int> res_cl;
   bool tiled = true;  // some lattice takes the tile kernels
@@ -226,8 +230,16 @@ static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
   return CLBM_OK;
 }
 
-// K steps of the resident lattices, from buffer 0 (K even: back to it).
+// K steps of the resident lattices, from buffer 0 (K even: back to it).  The
+// launches (up to ten, by cluster size) and the tiles' steps touch different
+// lattices, and each launch takes K times the latency of a step however few
+// lattices it holds, so they are branches that join before the residual.  One after
+// another they lost what they gain: us a step before, with branches, all lattices in
+// tiles: 64 uneven cavities of 32 .. 100, FP16 stochastic 31.1 / 16.4 / 16.7; of 32
+// .. 200, FP16, 20 steps between checks 65.4 / 43.7 / 47.1; of 32 .. 512, FP32
+// 189.7 / 185.4 / 195.2; two obstacle cavities of 128^2 beside a 512^2 one 10.9 / 8.8 / 19.5.
 static clbm_status launch_resident(clbm_batch* b, int K) {
+  if (b->fork) BCUDA(b, cudaEventRecord(b->fork, b->stream));
   for (const clbm_batch::Resident& r : b->resident) {
     ResArgs a{};
     a.lats = r.d_lats;
@@ -236,8 +248,17 @@ static clbm_status launch_resident(clbm_batch* b, int K) {
     a.cl = r.plan.cl;
     a.steps = K;
     a.stochastic = b->rounding;
-    BCUDA(b, b->L->resident_step(a, r.n, r.plan.threads, r.plan.smem, 0, b->stream));
+    const cudaStream_t st = b->fork ? r.side : b->stream;
+    if (b->fork) BCUDA(b, cudaStreamWaitEvent(st, b->fork, 0));
+    BCUDA(b, b->L->resident_step(a, r.n, r.plan.threads, r.plan.smem, 0, st));
+    if (b->fork) BCUDA(b, cudaEventRecord(r.done, st));
   }
+  return CLBM_OK;
+}
+
+static clbm_status join_resident(clbm_batch* b) {
+  if (b->fork)
+    for (const clbm_batch::Resident& r : b->resident) BCUDA(b, cudaStreamWaitEvent(b->stream, r.done, 0));
   return CLBM_OK;
 }
 
@@ -314,6 +335,13 @@ static clbm_status plan_resident(clbm_batch* b) {
       for (const ResLat& l : lats) b->res_cl[l.lat] = c;
     }
   b->tiled = std::count(b->res_cl.begin(), b->res_cl.end(), 0) > 0;
+  if (b->resident.size() + (b->tiled ? 1 : 0) > 1 && !b->resident.empty()) {
+    for (clbm_batch::Resident& r : b->resident) {
+      BCUDA(b, cudaStreamCreateWithFlags(&r.side, cudaStreamNonBlocking));
+      BCUDA(b, cudaEventCreateWithFlags(&r.done, cudaEventDisableTiming));
+    }
+    BCUDA(b, cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+  }
   return CLBM_OK;
 }
 
@@ -337,7 +365,12 @@ static void release(clbm_batch* b) {
   cudaFree(b->d_rpart);
   cudaFree(b->d_snap);
   cudaFree(b->d_snap_valid);
-  for (auto& r : b->resident) cudaFree(r.d_lats);
+  for (auto& r : b->resident) {
+    cudaFree(r.d_lats);
+    if (r.done) cudaEventDestroy(r.done);
+    if (r.side) cudaStreamDestroy(r.side);
+  }
+  if (b->fork) cudaEventDestroy(b->fork);
   if (b->h_ctl) cudaFreeHost(b->h_ctl);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
 }
@@ -592,6 +625,7 @@ clbm_status clbm_batch_solve(clbm_batch* b, double tol, int64_t max_steps, int32
     BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     clbm_status cst = launch_resident(b, K);
     for (int j = 0; j < K && cst == CLBM_OK && b->tiled; ++j) cst = launch_steps(b, j & 1, j);
+    if (cst == CLBM_OK) cst = join_resident(b);
     if (cst == CLBM_OK && b->L->batch_residual(b->d_lats, b->d_active, b->d_snap_valid, b->d_res, n, K,
                                                b->d_rpart, b->res_chunks, b->stream) != cudaSuccess)
       cst = CLBM_ECUDA;
