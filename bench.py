@@ -272,34 +272,26 @@ def box_lattice(w) -> bool:
     return w.geom.solid is None and len(w.geom.link_node) == 0
 
 
-def step_kernel_name(w) -> str:
+def step_kernel_name(w, resident: bool = False) -> str:
     """One launch per step: box lattices in tiles that take walls and seams
     themselves, masked ones with the listed boundary nodes in the first blocks
     and the interior warp tiles in the rest (tiles without fluid are skipped,
     flagged nodes left to the boundary blocks).  Small lattices stay in shared
-    memory for up to 4096 steps a launch."""
-    if resident_lattice(w):
-        return "resident_kernel (many steps a launch); FP64: step_box_kernel, one launch per step"
+    memory for up to 4096 steps a launch (`resident`, as the library says)."""
+    if resident:
+        return "resident_kernel (many steps a launch)"
     if box_lattice(w):
         return "step_box_kernel (tiles with walls inline, one launch per step)"
     return "step_fused_kernel<masked> (tile classes + listed boundary nodes, one launch per step)"
 
 
-def resident_lattice(w) -> bool:
-    """Lattices that a cluster of blocks holds in shared memory, below FP64
-    (of the workloads here: the 64 x 64 cavity)."""
-    return w.params.nx * w.params.ny <= 64 * 64
-
-
-def step_launches(w, steps: int, graph_levels: int = 5, precision: str = "f32") -> int:
-    """Kernels that clbm_step(steps) launches: one launch per step, or one per
-    4096 steps of a lattice in shared memory.  A
+def step_launches(w, steps: int, graph_levels: int = 5) -> int:
+    """Kernels that clbm_step(steps) launches with one launch per step (the
+    library's clbm_step_launches says which route a lattice takes).  A
     run of two or more steps replays captured graphs of 32, 16, ..., 2 steps
     (the binary digits of `steps`; a last odd step is launched on its own),
     each ending with one step-counter kernel, after one kernel that sets the
     counter."""
-    if steps >= 2 and resident_lattice(w) and precision != "f64":
-        return -(-steps // 4096)
     n = steps
     if steps >= 2:
         top = 1 << graph_levels
@@ -447,6 +439,8 @@ def run_native(args):
     rec = NCU_TRAFFIC.get(key)
     if rec and rec["kernel_hash"] == kernel_source_hash():
         traffic = rec["bytes_per_launch"]
+    launches = s.step_launches(args.steps) if mode == "single" else 0
+    resident = mode == "single" and 2 <= args.steps and launches < args.steps
     line = {"metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": el_ms / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -458,18 +452,18 @@ def run_native(args):
             "roofline": ({"bound": "alu", "achieved": FP64_FLOP_PER_LU * nodes / per_launch_s / 1e9,
                           "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
                           "frac": FP64_FLOP_PER_LU * nodes / per_launch_s / 1e9 / FP64_PEAK_GFLOPS,
-                          "traffic": traffic, "kernel": step_kernel_name(w),
+                          "traffic": traffic, "kernel": step_kernel_name(w, resident),
                           "peak_kind": "derived: 152 SMs x 2 FP64 FMA/clock x 2 x 2.07 GHz",
                           "flop_per_lattice_update": FP64_FLOP_PER_LU,
                           "hbm_frac": achieved / peak}
                          if args.precision == "f64" else
                          {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                           "frac": achieved / peak, "traffic": traffic,
-                          "kernel": step_kernel_name(w),
+                          "kernel": step_kernel_name(w, resident),
                           "peak_kind": peak_kind,
                           "algorithmic_bytes_per_launch": bytes_lu * nodes}),
             # slabs: one step launch per slab per step, plus (one process) one halo-copy launch
-            "gpu_launches": step_launches(w, args.steps, precision=args.precision) if mode == "single" else args.steps * (
+            "gpu_launches": launches if mode == "single" else args.steps * (
                 args.slabs + 1 if mode == "group" else 1),
             "residual_after": res}
     if e2e is not None:
@@ -520,9 +514,11 @@ def run_batch(args):
     widths = [b.tile_width(i) for i in range(len(ws))]
     K = (args.check_every + 1) // 2 * 2
     replays = -(-int(steps) // K)
-    # per step: one launch per tile-width group; per replay: the lattices that stay in shared
-    # memory (all their steps), residual (2), update, scan, tile rebuild
-    launches = int(steps) * len(set(widths)) + replays * 6
+    # per replay: the lattices that stay in shared memory (all their steps) and the residual and lists;
+    # per step: the tiles of the others
+    resident, per_step, per_check = b.launches()
+    launches = int(steps) * per_step + replays * (resident + per_check)
+    kernels = ["clbm::resident_kernel"] * (resident > 0) + ["clbm::batch_step_kernel"] * (per_step > 0)
     line = {"metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": 1,
             "steps": int(steps), "warmup": int(warm_steps), "ms_per_step": el / max(steps, 1) * 1e3,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -533,7 +529,7 @@ def run_batch(args):
                        "check_every": args.check_every, "rounding": args.rounding},
             "roofline": {"bound": "hbm", "achieved": bytes_lu * updates / el / 1e9, "peak": peak,
                          "unit": "GB/s", "frac": bytes_lu * updates / el / 1e9 / peak,
-                         "traffic": None, "kernel": "clbm::batch_step_kernel (whole solve)",
+                         "traffic": None, "kernel": " and ".join(kernels) + " (whole solve)",
                          "peak_kind": peak_kind},
             "batch": {"converged": int((conv > 0).sum()), "converged_fraction": float((conv > 0).mean()),
                       "diverged": int((conv == -2).sum()),

@@ -176,6 +176,12 @@ clbm_status clbm_init_fields(clbm_ctx* ctx, const double* rho, const double* ux,
  * CLBM_ECUDA reports a launch failure. */
 clbm_status clbm_step(clbm_ctx* ctx, int64_t nsteps);
 
+/* Kernels that clbm_step(nsteps) launches at this point: one for up to 4096
+ * steps where the lattice is small enough to take them in shared memory, else
+ * one a step and, from two steps on, one that sets the step counter and one for
+ * each captured graph of 2, 4, ..., 32 steps.  Errors: CLBM_EINVAL as clbm_step. */
+clbm_status clbm_step_launches(clbm_ctx* ctx, int64_t nsteps, int64_t* launches);
+
 /* Macroscopic fields at the current time: rho = sum f (Eq. 12),
  * u = (sum f e + F/2)/rho (Eq. 12), T = sum g + Q/2 (Eq. 25), as FP64
  * [ny][nx] arrays; solid nodes report 0.  Any pointer may be NULL.
@@ -384,6 +390,13 @@ clbm_status clbm_batch_lattice(clbm_batch* b, int32_t i, clbm_ctx** view);
 
 /* Nodes per warp tile chosen for lattice i (32, 64 or 128). */
 clbm_status clbm_batch_tile_width(const clbm_batch* b, int32_t i, int32_t* nodes_per_warp);
+
+/* Kernels that clbm_batch_solve launches: `resident` once per check interval
+ * for lattices that take its steps in shared memory (one for each cluster size),
+ * `per_step` every step for the others (one for each tile width without and with
+ * a mask, and one for the boundary nodes of masked lattices; 0 when there are no
+ * others), `per_check` once per check interval (residual and work lists). */
+clbm_status clbm_batch_launches(const clbm_batch* b, int32_t* resident, int32_t* per_step, int32_t* per_check);
 
 /* Free the batch, its views and its arena (NULL is allowed). */
 clbm_status clbm_batch_destroy(clbm_batch* b);

@@ -48,9 +48,11 @@ class clbm_batch_item(C.Structure):
                 ("uy", C.c_void_p), ("T", C.c_void_p)]
 
 
-EXPORTS = ["clbm_create", "clbm_set_boundaries", "clbm_init_fields", "clbm_step", "clbm_moments",
+EXPORTS = ["clbm_create", "clbm_set_boundaries", "clbm_init_fields", "clbm_step", "clbm_step_launches",
+           "clbm_moments",
            "clbm_nusselt", "clbm_residual", "clbm_totals", "clbm_residual_fields_noalloc", "clbm_batch_create",
-           "clbm_batch_solve", "clbm_batch_lattice", "clbm_batch_tile_width", "clbm_batch_destroy",
+           "clbm_batch_solve", "clbm_batch_lattice", "clbm_batch_tile_width", "clbm_batch_launches",
+           "clbm_batch_destroy",
            "clbm_damp_period2", "clbm_batch_damp_period2",
            "clbm_set_wall_velocity", "clbm_create_slab", "clbm_halo_bytes", "clbm_halo_pack", "clbm_halo_unpack", "clbm_halo_copy",
            "clbm_slabs_exchange", "clbm_slabs_step", "clbm_reduce_sums", "clbm_finish_sums",
@@ -84,6 +86,7 @@ def load(path: Optional[str] = None):
                                       C.POINTER(clbm_link), C.c_int32]
     L.clbm_init_fields.argtypes = [vp, vp, vp, vp, vp, C.c_int32]
     L.clbm_step.argtypes = [vp, C.c_int64]
+    L.clbm_step_launches.argtypes = [vp, C.c_int64, C.POINTER(C.c_int64)]
     L.clbm_moments.argtypes = [vp, vp, vp, vp, vp, C.c_int32]
     L.clbm_nusselt.argtypes = [vp, C.c_int32, C.c_double, C.c_double, dp]
     L.clbm_residual.argtypes = [vp, dp]
@@ -101,6 +104,7 @@ def load(path: Optional[str] = None):
                                    C.POINTER(C.c_int64)]
     L.clbm_batch_lattice.argtypes = [vp, C.c_int32, C.POINTER(vp)]
     L.clbm_batch_tile_width.argtypes = [vp, C.c_int32, C.POINTER(C.c_int32)]
+    L.clbm_batch_launches.argtypes = [vp] + [C.POINTER(C.c_int32)] * 3
     L.clbm_batch_destroy.argtypes = [vp]
     L.clbm_damp_period2.argtypes = [vp]
     L.clbm_batch_damp_period2.argtypes = [vp]
@@ -240,6 +244,13 @@ def clbm_init_fields(ctx, rho=None, ux=None, uy=None, T=None, on_device: bool = 
 
 def clbm_step(ctx, nsteps: int):
     _check(load().clbm_step(ctx, int(nsteps)), ctx, "clbm_step")
+
+
+def clbm_step_launches(ctx, nsteps: int) -> int:
+    """Kernels that clbm_step(nsteps) would launch now."""
+    out = C.c_int64()
+    _check(load().clbm_step_launches(ctx, int(nsteps), C.byref(out)), ctx, "clbm_step_launches")
+    return out.value
 
 
 def clbm_moments(ctx, rho=None, ux=None, uy=None, T=None, on_device: bool = False):
@@ -432,6 +443,9 @@ class Solver:
     def step(self, n: int = 1):
         clbm_step(self.ctx, n)
 
+    def step_launches(self, n: int) -> int:
+        return clbm_step_launches(self.ctx, n)
+
     def moments(self):
         shape = (self.ny, self.nx)
         out = [np.empty(shape) for _ in range(4)]
@@ -534,6 +548,13 @@ def clbm_batch_tile_width(b, i: int) -> int:
     return w.value
 
 
+def clbm_batch_launches(b):
+    """(resident launches a check interval, launches a step, other launches a check interval)."""
+    v = [C.c_int32() for _ in range(3)]
+    _batch_check(load().clbm_batch_launches(b, *[C.byref(x) for x in v]), b, "clbm_batch_launches")
+    return tuple(x.value for x in v)
+
+
 def clbm_batch_destroy(b):
     if b is not None and b.value:
         load().clbm_batch_destroy(b)
@@ -600,6 +621,9 @@ class Batch:
 
     def nusselt(self, i: int, which: int, length: float, dT: float) -> float:
         return clbm_nusselt(self.view(i), which, length, dT)
+
+    def launches(self):
+        return clbm_batch_launches(self.b)
 
     def tile_width(self, i: int) -> int:
         return clbm_batch_tile_width(self.b, i)

@@ -753,10 +753,30 @@ static bool resident_ready(clbm_ctx* c) {
   return c->res.cl > 0;
 }
 
+// Whether a call of clbm_step takes its steps in shared memory.
+static bool resident_call(clbm_ctx* c, int64_t nsteps) {
+  return nsteps >= 2 && resident_ready(c);
+}
+
+clbm_status clbm_step_launches(clbm_ctx* c, int64_t nsteps, int64_t* launches) {
+  if (!c || nsteps < 0 || !launches) return fail(c, CLBM_EINVAL, "bad step count");
+  if (!c->have_walls) return fail(c, CLBM_EINVAL, "non-periodic lattice: call clbm_set_boundaries first");
+  if (resident_call(c, nsteps)) {
+    *launches = (nsteps + kResidentSteps - 1) / kResidentSteps;
+    return CLBM_OK;
+  }
+  *launches = nsteps;
+  if (nsteps >= 2) {
+    *launches += 1 + nsteps / kGraphSteps;
+    for (int l = 0; l < kGraphLevels - 1; ++l) *launches += (nsteps >> (l + 1)) & 1;
+  }
+  return CLBM_OK;
+}
+
 clbm_status clbm_step(clbm_ctx* c, int64_t nsteps) {
   if (!c || nsteps < 0) return fail(c, CLBM_EINVAL, "bad step count");
   if (!c->have_walls) return fail(c, CLBM_EINVAL, "non-periodic lattice: call clbm_set_boundaries first");
-  if (nsteps >= 2 && resident_ready(c)) {
+  if (resident_call(c, nsteps)) {
     ResArgs a{};
     resident_plan(c, c->res.cl, kMaxResidentSmem, kMaxResidentThreads, &c->res, &a.one);
     a.cl = c->res.cl;

@@ -601,6 +601,17 @@ clbm_status clbm_batch_lattice(clbm_batch* b, int32_t i, clbm_ctx** view) {
   return CLBM_OK;
 }
 
+clbm_status clbm_batch_launches(const clbm_batch* b, int32_t* resident, int32_t* per_step, int32_t* per_check) {
+  if (!b || !resident || !per_step || !per_check) return CLBM_EINVAL;
+  int used[kBatchGroups] = {};
+  for (int i = 0; i < b->n; ++i)
+    if (!b->res_cl[i]) used[b->group[i]] = 1;
+  *resident = (int32_t)b->resident.size();
+  *per_step = (int32_t)std::count(used, used + kBatchGroups, 1) + (b->nbent > 0 ? 1 : 0);
+  *per_check = 5;  // residual (two stages), retire, scan, tiles
+  return CLBM_OK;
+}
+
 clbm_status clbm_batch_solve(clbm_batch* b, double tol, int64_t max_steps, int32_t check_every,
                              int64_t* conv_steps, double* residuals, int64_t* steps_run) {
   if (!b || max_steps < 1 || check_every < 1 || !(tol >= 0)) return bfail(b, CLBM_EINVAL, "bad solve arguments");

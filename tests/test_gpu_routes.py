@@ -1,0 +1,63 @@
+"""Which steps a lattice takes in shared memory, as the library reports it, at
+the ends of the rule's ranges; every route gives single steps bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1801_04577_gb300 import clbm
+from paper_1801_04577_gb300 import inputs as I
+
+from test_gpu_resident_seams import cylinder
+
+pytestmark = pytest.mark.gpu
+
+
+def plane_launches(n):
+    """One a step, the counter, and the graphs of 32, 16, ..., 2 steps."""
+    return n if n < 2 else n + 1 + n // 32 + bin((n % 32) >> 1).count("1")
+
+
+CASES = [
+    # lattice, precision, rounding, steps, resident
+    (lambda: I.natural_convection_cavity(32, 1e4), "f64", 0, 5, True),    # 64 nodes a band
+    (lambda: I.natural_convection_cavity(33, 1e4), "f64", 0, 5, False),
+    (lambda: I.annulus(20, 2.6, Ra=1e4), "f64", 0, 7, True),              # a mask, eight bands of up to 60 nodes
+    (lambda: I.annulus(24, 2.6, Ra=1e4), "f64", 0, 7, False),             # ... of 72
+    (lambda: I.obstacle_channel(16, 61), "f64", 0, 7, True),
+    (lambda: I.annulus(24, 2.6, Ra=1e4, interpolated=True), "f32", 0, 9, True),  # off the midpoint: one band
+    (lambda: I.annulus(32, 2.6, Ra=1e4, interpolated=True), "f32", 0, 9, True),
+    (lambda: I.annulus(48, 2.6, Ra=1e4, interpolated=True), "f32", 0, 40, False),  # beyond a block's memory
+    (lambda: cylinder(13.0), "f32", 0, 11, True),
+    (lambda: cylinder(4.6), "f32", 0, 11, False),   # a third node across the seam
+    (lambda: cylinder(19.4), "bf16", 0, 11, False),
+]
+
+
+@pytest.mark.parametrize("k", range(len(CASES)))
+def test_route_and_result(k):
+    make, precision, rounding, n, resident = CASES[k]
+    w = make()
+    a, b = (clbm.from_workload(w, precision, rounding=rounding) for _ in range(2))
+    assert a.step_launches(n) == (1 if resident else plane_launches(n))
+    assert a.step_launches(1) == 1 and a.step_launches(0) == 0
+    if resident:
+        assert a.step_launches(10000) == 3
+    for m in (n, n + 1):
+        a.step(m)
+        for _ in range(m):
+            b.step(1)
+    for x, y in zip(a.moments(), b.moments()):
+        np.testing.assert_array_equal(x, y)
+    assert a.residual() == b.residual()
+    a.close()
+    b.close()
+
+
+def test_batch_launches():
+    small, masked, wide = I.natural_convection_cavity(32, 1e4), I.obstacle_channel(500, 120), I.natural_convection_cavity(400, 1e4)
+    for ws, precision, want in (([small] * 4, "f32", (1, 0, 5)),                # one cluster size
+                                ([small] * 4, "f64", (0, 1, 5)),
+                                ([wide, masked], "f32", (0, 3, 5)),             # a width each, boundary nodes
+                                ([small, wide], "f32", (1, 1, 5))):
+        b = clbm.Batch(ws, precision, autotune=False)
+        assert b.launches() == want
+        b.close()
