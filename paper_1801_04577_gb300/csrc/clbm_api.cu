@@ -718,6 +718,14 @@ static clbm_status capture_steps(clbm_ctx* c, int cur, int par, int len, cudaGra
 
 // Steps of one resident launch (about 4 ms).
 constexpr int kResidentSteps = 4096;
+// Steps of a call from which on it is resident.  The launch loads and stores two states, 7 us and 9 us
+// per 1000 nodes of a band, before it gains 0.3 .. 0.9 us a step, or with a mask, where the plane steps
+// end in a tail of boundary nodes, 1.5 .. 2 (with stochastic rounding 0.5 .. 1.5).
+// Calls of 2 / 8 / 100 steps, resident / planes, us: cavity 150^2 FP32 (1500 nodes a band) 27 / 43 / 286
+// against 13 / 30 / 315; channel 200 x 100 FP16 stochastic (1400) 33 / 59 / 504 against 17 / 50 / 563;
+// annulus 32^2 FP32 off the midpoint, one band (1024) 29 / 58 / 524 against 18 / 54 / 618.  Of 8 / 16:
+// channel 100^2 FP32 (700) 34 / 53 against 43 / 80, 100 x 400 FP16 (2500) 68 / 103 against 51 / 94.
+static int resident_from(const clbm_ctx* c) { return c->res.nodes / (c->d_flags && !c->p.rounding ? 120 : 80); }
 
 // Whether a single lattice is faster in shared memory than in planes, with `nodes` nodes in each of
 // its bands (measured, us a step, resident / planes):
@@ -755,7 +763,7 @@ static bool resident_ready(clbm_ctx* c) {
 
 // Whether a call of clbm_step takes its steps in shared memory.
 static bool resident_call(clbm_ctx* c, int64_t nsteps) {
-  return nsteps >= 2 && resident_ready(c);
+  return nsteps >= 2 && resident_ready(c) && nsteps >= resident_from(c);
 }
 
 clbm_status clbm_step_launches(clbm_ctx* c, int64_t nsteps, int64_t* launches) {
@@ -1271,6 +1279,7 @@ bool resident_plan(const clbm_ctx* c, int cl, size_t max_smem, int max_threads, 
   const int bt = std::min((most + 31) / 32 * 32, max_threads / 2), nodes = rows * nx;
   const int passes = (nodes + (max_threads - bt) - 1) / (max_threads - bt);
   plan->cl = cl;
+  plan->nodes = nodes;
   plan->threads = std::min(max_threads, std::max(64, bt + ((nodes + passes - 1) / passes + 31) / 32 * 32));
   plan->smem = smem;
   if (lat) {

@@ -18,6 +18,8 @@ def plane_launches(n):
 
 CASES = [
     # lattice, precision, rounding, steps, resident
+    (lambda: I.natural_convection_cavity(64, 1e4), "f32", 0, 2, False),   # 256 nodes a band: from 3 steps on
+    (lambda: I.natural_convection_cavity(64, 1e4), "f32", 0, 3, True),
     (lambda: I.natural_convection_cavity(32, 1e4), "f64", 0, 5, True),    # 64 nodes a band
     (lambda: I.natural_convection_cavity(33, 1e4), "f64", 0, 5, False),
     (lambda: I.annulus(20, 2.6, Ra=1e4), "f64", 0, 7, True),              # a mask, eight bands of up to 60 nodes
@@ -25,6 +27,7 @@ CASES = [
     (lambda: I.obstacle_channel(16, 61), "f64", 0, 7, True),
     (lambda: I.annulus(24, 2.6, Ra=1e4, interpolated=True), "f32", 0, 9, True),  # off the midpoint: one band
     (lambda: I.annulus(32, 2.6, Ra=1e4, interpolated=True), "f32", 0, 9, True),
+    (lambda: I.annulus(32, 2.6, Ra=1e4, interpolated=True), "f32", 0, 7, False),
     (lambda: I.annulus(48, 2.6, Ra=1e4, interpolated=True), "f32", 0, 40, False),  # beyond a block's memory
     (lambda: cylinder(13.0), "f32", 0, 11, True),
     (lambda: cylinder(4.6), "f32", 0, 11, False),   # a third node across the seam
