@@ -727,20 +727,25 @@ constexpr int kResidentSteps = 4096;
 // channel 100^2 FP32 (700) 34 / 53 against 43 / 80, 100 x 400 FP16 (2500) 68 / 103 against 51 / 94.
 static int resident_from(const clbm_ctx* c) { return c->res.nodes / (c->d_flags && !c->p.rounding ? 120 : 80); }
 
-// Whether a single lattice is faster in shared memory than in planes, with `nodes` nodes in each of
-// its bands (measured, us a step, resident / planes):
+// Whether a single lattice is faster in shared memory than in planes with the bands of plan p
+// (measured, us a step, resident / planes):
 //   FP64: an FP64 instruction takes a warp's quarter of the multiprocessor 64 cycles, so the work
 //         belongs on every multiprocessor: 32^2 (64 nodes a band) 7.0 / 8.1, 36^2 9.4 / 7.9
-//   with a mask the plane steps end in a tail of boundary nodes: 64^2 FP32 2.5 / 4.4, 200 x 100 2.9 /
-//         4.7, FP16 stochastic 4.9 / 6.0
-//   FP32: 32^2 1.5 / 3.3, 150^2 2.7 / 3.2
-//   16 bit: 64^2 2.2 / 2.9, 150^2 2.9 / 2.9, stochastic 110^2 3.0 / 3.4, 128^2 3.5 / 3.4; wide rows
+//   with a mask the plane steps end in a tail of boundary nodes: 64^2 FP32 2.5 / 4.4, 200 x 100 2.8 /
+//         4.6, FP16 stochastic 4.8 / 5.6; nearest 16-bit pays in bands of up to 3200 nodes (200 x
+//         250 5.6 / 6.1), stochastic up to 1950 (100 x 300, 1900 nodes: 5.7 / 6.0, 200 x 150,
+//         2000: 6.5 / 5.8); one band (walls off the midpoint) while a pass updates all its
+//         boundary nodes (annulus 48^2 FP16, 256 of them: 6.2 / 6.6, 52^2, 280: 8.9 / 7.0)
+//   FP32: 32^2 1.4 / 3.3, 150^2 2.6 / 3.1
+//   16 bit: 64^2 2.1 / 3.0, 150^2 2.9 / 2.9, stochastic 110^2 3.0 / 3.4, 128^2 3.5 / 3.4; wide rows
 //         are stored into two bands a value at a time, 512 x 32 5.1 / 2.5
-static bool resident_pays(const clbm_ctx* c, int nodes) {
-  if (c->p.precision == CLBM_F64) return nodes <= 64;
-  if (c->d_flags) return c->p.nx <= 400;
+static bool resident_pays(const clbm_ctx* c, const ResPlan& p) {
+  if (c->p.precision == CLBM_F64) return p.nodes <= 64;
+  if (c->d_flags)
+    return c->p.nx <= 400 && (!c->p.rounding || p.nodes <= 1950) &&
+           (p.cl > 1 || p.edge <= kMaxResidentThreads / 2);
   if (c->p.precision == CLBM_F32) return c->p.nx <= 256;
-  return c->p.nx <= 160 && nodes <= (c->p.rounding ? 900 : 1400);
+  return c->p.nx <= 160 && p.nodes <= (c->p.rounding ? 900 : 1400);
 }
 
 // Plan the resident steps of a single lattice: the most blocks a cluster can
@@ -751,8 +756,7 @@ static bool resident_ready(clbm_ctx* c) {
     best.cl = 0;
     for (int cl = kMaxCluster; cl >= 1 && best.cl == 0; cl /= 2) {
       ResPlan p;
-      if (resident_pays(c, (c->p.ny + cl - 1) / cl * c->p.nx) &&
-          resident_plan(c, cl, kMaxResidentSmem, kMaxResidentThreads, &p, nullptr) &&
+      if (resident_plan(c, cl, kMaxResidentSmem, kMaxResidentThreads, &p, nullptr) && resident_pays(c, p) &&
           c->L->resident_clusters(cl, p.threads, p.smem, c->p.viscous_heating) > 0)
         best = p;
     }
@@ -1280,6 +1284,7 @@ bool resident_plan(const clbm_ctx* c, int cl, size_t max_smem, int max_threads, 
   const int passes = (nodes + (max_threads - bt) - 1) / (max_threads - bt);
   plan->cl = cl;
   plan->nodes = nodes;
+  plan->edge = most;
   plan->threads = std::min(max_threads, std::max(64, bt + ((nodes + passes - 1) / passes + 31) / 32 * 32));
   plan->smem = smem;
   if (lat) {

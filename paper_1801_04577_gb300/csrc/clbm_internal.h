@@ -295,7 +295,7 @@ void set_view_time(clbm_ctx* c, int64_t t, int cur);
 // A lattice's launch on clusters of `cl` resident blocks: false if its bands do not fit.
 struct ResPlan {
   int cl = -1, threads = 0;  // cl: -1 not planned yet, 0 the lattice is not resident
-  int nodes = 0;             // of a band
+  int nodes = 0, edge = 0;   // of a band, and the most boundary nodes of one
   size_t smem = 0;
 };
 bool resident_plan(const clbm_ctx* c, int cl, size_t max_smem, int max_threads, ResPlan* plan, ResLat* lat);

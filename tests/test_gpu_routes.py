@@ -29,6 +29,12 @@ CASES = [
     (lambda: I.annulus(32, 2.6, Ra=1e4, interpolated=True), "f32", 0, 9, True),
     (lambda: I.annulus(32, 2.6, Ra=1e4, interpolated=True), "f32", 0, 7, False),
     (lambda: I.annulus(48, 2.6, Ra=1e4, interpolated=True), "f32", 0, 40, False),  # beyond a block's memory
+    (lambda: I.annulus(48, 2.6, Ra=1e4, interpolated=True), "f16", 0, 19, True),   # 256 boundary nodes
+    (lambda: I.annulus(52, 2.6, Ra=1e4, interpolated=True), "bf16", 0, 40, False),
+    (lambda: I.annulus(44, 2.6, Ra=1e4, interpolated=True), "f16", 1, 25, True),
+    (lambda: I.annulus(48, 2.6, Ra=1e4, interpolated=True), "f16", 1, 40, False),  # stochastic: 1950 nodes
+    (lambda: I.obstacle_channel(200, 150), "f16", 0, 17, True),
+    (lambda: I.obstacle_channel(200, 150), "f16", 1, 40, False),
     (lambda: cylinder(13.0), "f32", 0, 11, True),
     (lambda: cylinder(4.6), "f32", 0, 11, False),   # a third node across the seam
     (lambda: cylinder(19.4), "bf16", 0, 11, False),
