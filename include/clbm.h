@@ -385,7 +385,9 @@ clbm_status clbm_batch_solve(clbm_batch* b, double tol, int64_t max_steps, int32
                              int64_t* conv_steps, double* residuals, int64_t* steps_run);
 
 /* Context view of lattice i (owned by the batch: do not destroy it) for
- * clbm_moments, clbm_nusselt, clbm_residual, clbm_init_fields or clbm_step. */
+ * clbm_moments, clbm_nusselt, clbm_residual, clbm_init_fields or clbm_step.
+ * Walls set on a view later (clbm_set_boundaries) hold for the view's own
+ * steps; clbm_batch_solve keeps those of clbm_batch_create. */
 clbm_status clbm_batch_lattice(clbm_batch* b, int32_t i, clbm_ctx** view);
 
 /* Nodes per warp tile chosen for lattice i (32, 64 or 128). */

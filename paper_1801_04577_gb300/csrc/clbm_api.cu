@@ -60,6 +60,7 @@ struct clbm_ctx {
   int32_t* d_slot = nullptr;
   void* d_lk_t = nullptr;
   void* d_lk_f = nullptr;
+  std::vector<void*> retired;  // a view's earlier tables
   uint8_t* d_tile_fluid = nullptr;  // masked lattices: which interior warp tiles hold fluid
   int tiles_per_row = 0;
   std::vector<int32_t> h_bnodes;  // nodes the boundary kernel recomputes (pitch layout)
@@ -173,14 +174,20 @@ static DevCoef make_coef(const clbm_ctx* c) {
   return k;
 }
 
+// Give up a table of the walls.  A batch's launches hold the tables its views were created with, so a
+// view keeps them until it goes (and the batch goes on with those walls).
+static void drop_table(clbm_ctx* c, void* table) {
+  if (table && c->borrowed)
+    c->retired.push_back(table);
+  else
+    cudaFree(table);
+}
+
 static void free_tables(clbm_ctx* c) {
   c->res = ResPlan{};
-  cudaFree(c->d_flags);
-  cudaFree(c->d_slot);
-  cudaFree(c->d_lk_t);
-  cudaFree(c->d_lk_f);
-  cudaFree(c->d_tile_fluid);
-  cudaFree(c->d_bnodes);
+  for (void* t : {(void*)c->d_flags, (void*)c->d_slot, c->d_lk_t, c->d_lk_f, (void*)c->d_tile_fluid,
+                  (void*)c->d_bnodes})
+    drop_table(c, t);
   c->d_bnodes = nullptr;
   c->d_flags = nullptr;
   c->d_slot = nullptr;
@@ -212,7 +219,7 @@ static cudaError_t upload_boundary_list(clbm_ctx* c, const std::vector<uint16_t>
       if (need) v.push_back((int32_t)ip);
     }
   }
-  cudaFree(c->d_bnodes);
+  drop_table(c, c->d_bnodes);
   c->d_bnodes = nullptr;
   if (v.empty()) return cudaSuccess;
   cudaError_t e = cudaMalloc(&c->d_bnodes, v.size() * sizeof(int32_t));
@@ -252,8 +259,11 @@ clbm_status clbm_destroy(clbm_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   drop_graphs(c);
   cudaFree(c->d_t);
+  const bool view = c->borrowed;
+  c->borrowed = false;  // nothing is launched on the tables any more
   free_tables(c);
-  if (!c->borrowed) {
+  for (void* t : c->retired) cudaFree(t);
+  if (!view) {
     cudaFree(c->buf[0]);
     cudaFree(c->buf[1]);
   }
@@ -563,6 +573,7 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
     // upload
     CLBM_CUDA(c, cudaStreamSynchronize(c->stream));
     drop_graphs(c);  // captured steps hold the old wall description
+    c->retired.reserve(c->retired.size() + 6);
     free_tables(c);
     if (masked) {
       const size_t np = (size_t)ny * c->pitch;
