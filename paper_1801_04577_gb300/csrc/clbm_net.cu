@@ -1684,13 +1684,15 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
   // activations
   n->plan = make_plan(n);
   for (size_t id = 0; id < n->act_c.size(); ++id) {
-    const long long e = (long long)c.max_batch * n->act_c[id] * n->act_hw[id] * n->act_hw[id];
+    const long long image = (long long)c.max_batch * n->act_hw[id] * n->act_hw[id], e = image * n->act_c[id];
     float *a = nullptr, *ga = nullptr;
-    // operand-layout networks keep FP32 activations of the input, the skip connections and the output only
-    const std::vector<int> cats(n->plan.cat, n->plan.cat + L - 1);
-    const bool keep = !n->direct || (int)id == n->plan.in || (int)id == n->plan.out ||
-                      std::find(cats.begin(), cats.end(), (int)id) != cats.end();
-    if ((keep && cudaMalloc(&a, e * sizeof(float))) || cudaMalloc(&ga, e * sizeof(float))) {
+    // operand-layout networks keep FP32 activations of the input, the output and the skip connections
+    // (without the upsampled part beside them) only, and no gradient of the input
+    const int l = (int)(std::find(n->plan.cat, n->plan.cat + L - 1, (int)id) - n->plan.cat);
+    const bool whole = !n->direct || (int)id == n->plan.in || (int)id == n->plan.out;
+    const long long ea = whole ? e : l < L - 1 ? image * (c.base << l) : 0;
+    const bool grad = !n->direct || (int)id != n->plan.in;
+    if ((ea && cudaMalloc(&a, ea * sizeof(float))) || (grad && cudaMalloc(&ga, e * sizeof(float)))) {
       cudaFree(a);
       return bail(CLBM_ENOMEM);
     }
@@ -1705,17 +1707,19 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
     long long dw_need = 0, bias_need = 0;
     for (long long nb = 1; nb <= c.max_batch; ++nb) {
       const long long Np = nb * cv.H * cv.W;
-      const long long kper = dw_kper(n->sms, c.math == CLBM_NET_TENSOR, Np, Kd, cv.co);
-      cap = std::max(cap, ((Np + kper - 1) / kper) * cv.co * Kd);
-      cap = std::max(cap, ((Np + kBiasChunk - 1) / kBiasChunk) * cv.co);  // bias chunk sums
-      if (n->direct) {
+      if (n->direct) {  // partial sums of each layer's own
         conv::Op x{};
         x.C = (cv.ci + 7) / 8 * 8;
         x.H = x.W = cv.H;
         const DwShape s = dw_shape(n->sms, x, (cv.co + 7) / 8, cv.ks * cv.ks, (int)nb);
         dw_need = std::max(dw_need, (long long)s.ranges * cv.co * Kd);
         bias_need = std::max(bias_need, ((Np + kBiasChunk - 1) / kBiasChunk) * cv.co);
-      } else if (c.math == CLBM_NET_TENSOR) {  // split-K forward and input-gradient GEMMs
+        continue;
+      }
+      const long long kper = dw_kper(n->sms, c.math == CLBM_NET_TENSOR, Np, Kd, cv.co);
+      cap = std::max(cap, ((Np + kper - 1) / kper) * cv.co * Kd);
+      cap = std::max(cap, ((Np + kBiasChunk - 1) / kBiasChunk) * cv.co);  // bias chunk sums
+      if (c.math == CLBM_NET_TENSOR) {  // split-K forward and input-gradient GEMMs
         cap = std::max(cap, (long long)conv_splits(n->sms, (int)Np, cv.co, Kd) * Np * cv.co);
         cap = std::max(cap, (long long)conv_splits(n->sms, (int)Np, cv.ci, cv.co * cv.ks * cv.ks) * Np * cv.ci);
       }
@@ -1737,7 +1741,7 @@ clbm_status clbm_net_create(const clbm_net_config* cfg, uint64_t seed, void* str
   if (cudaHostAlloc(&n->tflag, sizeof(int), cudaHostAllocMapped) != cudaSuccess) return bail(CLBM_ENOMEM);
   *n->tflag = 0;
   if (cudaHostGetDevicePointer(&n->d_tflag, n->tflag, 0) != cudaSuccess) return bail(CLBM_ECUDA);
-  if (cudaMalloc(&n->part, cap * sizeof(float)) ||
+  if ((cap && cudaMalloc(&n->part, cap * sizeof(float))) ||
       cudaMalloc(&n->loss_part, (size_t)c.max_batch * (kLossChunks + 1) * sizeof(double)) ||
       cudaHostAlloc(&n->h_loss, (size_t)c.max_batch * (kLossChunks + 1) * sizeof(double), cudaHostAllocDefault) ||
       cudaMalloc(&n->tgt, (size_t)c.max_batch * c.out_ch * c.grid * c.grid * sizeof(float)) ||
