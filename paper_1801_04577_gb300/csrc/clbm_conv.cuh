@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(conv_threads(RANGES), RANGES ? 1 : 8) conv_ker
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
       const uint32_t idesc = tc::idesc_bf16_f32(tc::kBM, a.bn);
+      pdl_wait();  // the waits' limit counts from when the input can come
       failed = !tc::mbar_wait(bar_a, 0);
       int i = 0;
       for (int z = 0; z < (RANGES ? a.ranges : 1) && !failed; ++z) {
@@ -288,6 +289,7 @@ __global__ void __launch_bounds__(conv_threads(RANGES), RANGES ? 1 : 8) conv_ker
   }
   if constexpr (RANGES) {
     if (warp < 4) {
+      pdl_wait();
 #pragma unroll
       for (int c = 0; c < kMaxBn; ++c) sum[c] = 0.0f;
       for (int z = 0; z < a.ranges; ++z) {
@@ -310,12 +312,12 @@ __global__ void __launch_bounds__(conv_threads(RANGES), RANGES ? 1 : 8) conv_ker
     }
   } else {
     __syncwarp();
+    pdl_wait();
     if (!tc::mbar_wait(&bar_d[0], 0)) failed = true;
   }
   if (__syncthreads_or(failed)) {
     if (tid == 0) atomicExch(a.err, 1);
   } else if (warp < 4) {
-    pdl_wait();
     tc::fence_after();
 #pragma unroll 1
     for (int u = 0; u < mt; ++u) {
