@@ -516,7 +516,7 @@ def run_batch(args):
     replays = -(-int(steps) // K)
     # per replay: the lattices that stay in shared memory (all their steps) and the residual and lists;
     # per step: the tiles of the others
-    resident, per_step, per_check = b.launches()
+    resident, per_step, per_check = b.launches(args.check_every)
     launches = int(steps) * per_step + replays * (resident + per_check)
     kernels = ["clbm::resident_kernel"] * (resident > 0) + ["clbm::batch_step_kernel"] * (per_step > 0)
     line = {"metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": 1,

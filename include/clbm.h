@@ -393,12 +393,15 @@ clbm_status clbm_batch_lattice(clbm_batch* b, int32_t i, clbm_ctx** view);
 /* Nodes per warp tile chosen for lattice i (32, 64 or 128). */
 clbm_status clbm_batch_tile_width(const clbm_batch* b, int32_t i, int32_t* nodes_per_warp);
 
-/* Kernels that clbm_batch_solve launches: `resident` once per check interval
- * for lattices that take its steps in shared memory (one for each cluster size),
- * `per_step` every step for the others (one for each tile width without and with
- * a mask, and one for the boundary nodes of masked lattices; 0 when there are no
- * others), `per_check` once per check interval (residual and work lists). */
-clbm_status clbm_batch_launches(const clbm_batch* b, int32_t* resident, int32_t* per_step, int32_t* per_check);
+/* Kernels that clbm_batch_solve launches with this check_every: `resident` once
+ * per check interval for lattices that take its steps in shared memory (one for
+ * each cluster size, without and with a mask), `per_step` every step for the
+ * others (one for each tile width without and with a mask, and one for the
+ * boundary nodes of masked lattices; 0 when there are no others), `per_check`
+ * once per check interval (residual and work lists).  CLBM_EINVAL for
+ * check_every < 1. */
+clbm_status clbm_batch_launches(const clbm_batch* b, int32_t check_every, int32_t* resident, int32_t* per_step,
+                                int32_t* per_check);
 
 /* Free the batch, its views and its arena (NULL is allowed). */
 clbm_status clbm_batch_destroy(clbm_batch* b);

@@ -104,7 +104,7 @@ def load(path: Optional[str] = None):
                                    C.POINTER(C.c_int64)]
     L.clbm_batch_lattice.argtypes = [vp, C.c_int32, C.POINTER(vp)]
     L.clbm_batch_tile_width.argtypes = [vp, C.c_int32, C.POINTER(C.c_int32)]
-    L.clbm_batch_launches.argtypes = [vp] + [C.POINTER(C.c_int32)] * 3
+    L.clbm_batch_launches.argtypes = [vp, C.c_int32] + [C.POINTER(C.c_int32)] * 3
     L.clbm_batch_destroy.argtypes = [vp]
     L.clbm_damp_period2.argtypes = [vp]
     L.clbm_batch_damp_period2.argtypes = [vp]
@@ -548,10 +548,10 @@ def clbm_batch_tile_width(b, i: int) -> int:
     return w.value
 
 
-def clbm_batch_launches(b):
+def clbm_batch_launches(b, check_every: int):
     """(resident launches a check interval, launches a step, other launches a check interval)."""
     v = [C.c_int32() for _ in range(3)]
-    _batch_check(load().clbm_batch_launches(b, *[C.byref(x) for x in v]), b, "clbm_batch_launches")
+    _batch_check(load().clbm_batch_launches(b, int(check_every), *[C.byref(x) for x in v]), b, "clbm_batch_launches")
     return tuple(x.value for x in v)
 
 
@@ -622,8 +622,8 @@ class Batch:
     def nusselt(self, i: int, which: int, length: float, dT: float) -> float:
         return clbm_nusselt(self.view(i), which, length, dT)
 
-    def launches(self):
-        return clbm_batch_launches(self.b)
+    def launches(self, check_every: int = 100):
+        return clbm_batch_launches(self.b, check_every)
 
     def tile_width(self, i: int) -> int:
         return clbm_batch_tile_width(self.b, i)

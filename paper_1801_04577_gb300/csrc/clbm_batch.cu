@@ -114,15 +114,15 @@ struct clbm_batch {
   // cluster size (0: the tile kernels)
   struct Resident {
     ResPlan plan;
-    int n = 0;
+    int n = 0, from = 0;  // lattices; shortest check interval
     ResLat* d_lats = nullptr;
     cudaStream_t side = nullptr;  // the launch's branch of the captured solve
     cudaEvent_t done = nullptr;
   };
-  cudaEvent_t fork = nullptr;  // where the branches begin (nullptr: one launch and nothing beside it)
+  cudaEvent_t fork = nullptr;  // where the branches begin
   std::vector<Resident> resident;
-  std::vector<int> res_cl;
-  bool tiled = true;  // some lattice takes the tile kernels
+  std::vector<int> res_cl, res_from;  // per lattice: cluster size (0: none), shortest check interval
+  int interval = 1 << 30;             // steps between checks that the lists are made for
   std::vector<long long> group_base = std::vector<long long>(kBatchGroups, 0);  // tile-list offsets
   BatchLat* d_lats = nullptr;
   int* d_active = nullptr;
@@ -137,8 +137,8 @@ struct clbm_batch {
   int4** d_group_tiles = nullptr;
   double* d_snap = nullptr;  // convergence snapshots of all lattices
   int* d_snap_valid = nullptr;
-  int2* d_bent = nullptr;  // boundary entries {lattice, node} of all lattices
-  int nbent = 0;
+  int2* d_bent = nullptr;  // boundary entries {lattice, node} of the masked lattices, those resident from the
+  std::vector<std::pair<int, int>> bent;  // shortest intervals last: {from, end of those from there on or never}
   double* d_rpart = nullptr;  // residual chunk sums
   int res_chunks = 1;
   cudaGraphExec_t exec = nullptr;
@@ -158,11 +158,31 @@ static clbm_status bfail(clbm_batch* b, clbm_status s, const std::string& m) {
     if (e_ != cudaSuccess) return bfail((b), CLBM_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
+// Whether lattice i takes the steps of a check interval of K in shared memory.  The launch loads and
+// stores its states before it gains anything: us a step at K = 4 / 8 / 12 / 24, resident / tiles, of
+// 256 cavities of 64^2 FP32 98 / 59 / 46 / 33 against 61 / 44 / 39 / 33, 16 of them 28 / 15 / 12 / 7.6
+// against 24 / 14 / 11 / 8.1, 256 obstacle cavities 99 / 60 / 47 / 33 against 83 / 64 / 58 / 52, 64 of
+// 128^2 (a whole multiprocessor's memory a block) 125 / 75 / 59 / 42 against 83 / 61 / 54 / 46.
+constexpr int kFromMasked = 6, kFromOther = 12;
+static bool resident_at(const clbm_batch* b, int i, int K) { return b->res_cl[i] && K >= b->res_from[i]; }
+static bool tiled_at(const clbm_batch* b, int K) {
+  for (int i = 0; i < b->n; ++i)
+    if (!resident_at(b, i, K)) return true;
+  return false;
+}
+// Boundary entries of the lattices that are tiled at K.
+static int entries_at(const clbm_batch* b, int K) {
+  int n = 0;
+  for (const auto& e : b->bent)
+    if (K < e.first) n = std::max(n, e.second);
+  return n;
+}
+
 // Rows that get tiles: all; with a mask and y walls all but the first and last
 // (boundary rows).
 static int first_row(const clbm_batch* b, int i) { return b->masked[i] && !b->py[i] ? 1 : 0; }
 static int tile_rows(const clbm_batch* b, int i) {
-  if (b->res_cl[i]) return 0;
+  if (resident_at(b, i, b->interval)) return 0;
   return std::max(b->ny[i] - 2 * first_row(b, i), 0);
 }
 
@@ -216,7 +236,7 @@ static clbm_status build_tiles(clbm_batch* b) {
 static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
   std::vector<int> used(kBatchGroups, 0);
   for (int i = 0; i < b->n; ++i)
-    if (!b->res_cl[i]) used[b->group[i]] = 1;
+    if (!resident_at(b, i, b->interval)) used[b->group[i]] = 1;
   const std::vector<long long>& base = b->group_base;  // as in upload_layout
   for (int g = 0; g < kBatchGroups; ++g) {
     if (!used[g]) continue;
@@ -225,13 +245,24 @@ static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
     BCUDA(b, b->L->batch_step(v, g >= kBatchWidths, b->d_lats, b->d_tiles + base[g], &b->d_ctl->count[g], parity,
                               &b->d_ctl->t, tstep, b->rounding, b->grid[g], b->stream));
   }
-  BCUDA(b, b->L->batch_boundary(b->d_lats, b->d_bent, b->nbent, b->d_active, parity, &b->d_ctl->t,
+  BCUDA(b, b->L->batch_boundary(b->d_lats, b->d_bent, entries_at(b, b->interval), b->d_active, parity, &b->d_ctl->t,
                                 tstep, b->rounding, b->stream));
   return CLBM_OK;
 }
 
+// Launches of resident lattices at K, and whether they are branches (not one alone).
+static int launches_at(const clbm_batch* b, int K) {
+  int n = 0;
+  for (const clbm_batch::Resident& r : b->resident) n += K >= r.from;
+  return n;
+}
+static bool branches_at(const clbm_batch* b, int K) {
+  const int n = launches_at(b, K);
+  return n > 0 && n + (tiled_at(b, K) ? 1 : 0) > 1;
+}
+
 // K steps of the resident lattices, from buffer 0 (K even: back to it).  The
-// launches (up to ten, by cluster size) and the tiles' steps touch different
+// launches (by cluster size, without and with a mask) and the tiles' steps touch different
 // lattices, and each launch takes K times the latency of a step however few
 // lattices it holds, so they are branches that join before the residual.  One after
 // another they lost what they gain: us a step before, with branches, all lattices in
@@ -239,8 +270,10 @@ static clbm_status launch_steps(clbm_batch* b, int parity, int tstep) {
 // .. 200, FP16, 20 steps between checks 65.4 / 43.7 / 47.1; of 32 .. 512, FP32
 // 189.7 / 185.4 / 195.2; two obstacle cavities of 128^2 beside a 512^2 one 10.9 / 8.8 / 19.5.
 static clbm_status launch_resident(clbm_batch* b, int K) {
-  if (b->fork) BCUDA(b, cudaEventRecord(b->fork, b->stream));
+  const bool fork = branches_at(b, K);
+  if (fork) BCUDA(b, cudaEventRecord(b->fork, b->stream));
   for (const clbm_batch::Resident& r : b->resident) {
+    if (K < r.from) continue;
     ResArgs a{};
     a.lats = r.d_lats;
     a.active = b->d_active;
@@ -248,17 +281,18 @@ static clbm_status launch_resident(clbm_batch* b, int K) {
     a.cl = r.plan.cl;
     a.steps = K;
     a.stochastic = b->rounding;
-    const cudaStream_t st = b->fork ? r.side : b->stream;
-    if (b->fork) BCUDA(b, cudaStreamWaitEvent(st, b->fork, 0));
+    const cudaStream_t st = fork ? r.side : b->stream;
+    if (fork) BCUDA(b, cudaStreamWaitEvent(st, b->fork, 0));
     BCUDA(b, b->L->resident_step(a, r.n, r.plan.threads, r.plan.smem, 0, st));
-    if (b->fork) BCUDA(b, cudaEventRecord(r.done, st));
+    if (fork) BCUDA(b, cudaEventRecord(r.done, st));
   }
   return CLBM_OK;
 }
 
-static clbm_status join_resident(clbm_batch* b) {
-  if (b->fork)
-    for (const clbm_batch::Resident& r : b->resident) BCUDA(b, cudaStreamWaitEvent(b->stream, r.done, 0));
+static clbm_status join_resident(clbm_batch* b, int K) {
+  if (branches_at(b, K))
+    for (const clbm_batch::Resident& r : b->resident)
+      if (K >= r.from) BCUDA(b, cudaStreamWaitEvent(b->stream, r.done, 0));
   return CLBM_OK;
 }
 
@@ -274,6 +308,7 @@ static clbm_status join_resident(clbm_batch* b) {
 static clbm_status plan_resident(clbm_batch* b) {
   const int n = b->n;
   b->res_cl.assign(n, 0);
+  b->res_from.assign(n, 0);
   if (b->precision == CLBM_F64) return CLBM_OK;  // bound by the FP64 pipes of every multiprocessor
   int dev = 0, sms = 0;
   BCUDA(b, cudaGetDevice(&dev));
@@ -309,33 +344,40 @@ static clbm_status plan_resident(clbm_batch* b) {
         grown = true;
       }
   }
-  for (int w = 0; w < 2; ++w)
-    for (int c = 1; c <= kMaxCluster; c *= 2) {
-      clbm_batch::Resident r;
-      std::vector<ResLat> lats;
-      for (int i = 0; i < n; ++i) {
-        if (cl[i] != c || whole[i] != w) continue;
-        ResPlan p;
-        ResLat l;
-        resident_plan(b->views[i], c, smem_of[w], threads_of[w], &p, &l);
-        l.lat = i;
-        lats.push_back(l);
-        r.plan.cl = c;
-        r.plan.threads = std::max(r.plan.threads, p.threads);
-        r.plan.smem = std::max(r.plan.smem, p.smem);
+  std::vector<int> from(n, kFromOther);
+  for (int i = 0; i < n; ++i)
+    if (!whole[i] && describe_view(b->views[i]).g.flags) from[i] = kFromMasked;
+  for (const int f : {kFromOther, kFromMasked})
+    for (int w = 0; w < 2; ++w)
+      for (int c = 1; c <= kMaxCluster; c *= 2) {
+        clbm_batch::Resident r;
+        r.from = f;
+        std::vector<ResLat> lats;
+        for (int i = 0; i < n; ++i) {
+          if (cl[i] != c || whole[i] != w || from[i] != f) continue;
+          ResPlan p;
+          ResLat l;
+          resident_plan(b->views[i], c, smem_of[w], threads_of[w], &p, &l);
+          l.lat = i;
+          lats.push_back(l);
+          r.plan.cl = c;
+          r.plan.threads = std::max(r.plan.threads, p.threads);
+          r.plan.smem = std::max(r.plan.smem, p.smem);
+        }
+        if (lats.empty() || b->L->resident_clusters(c, r.plan.threads, r.plan.smem, 0) < 1) continue;
+        r.n = (int)lats.size();
+        if (cudaMalloc(&r.d_lats, lats.size() * sizeof(ResLat)) != cudaSuccess) {
+          cudaGetLastError();
+          return CLBM_ENOMEM;
+        }
+        b->resident.push_back(r);
+        BCUDA(b, cudaMemcpy(r.d_lats, lats.data(), lats.size() * sizeof(ResLat), cudaMemcpyHostToDevice));
+        for (const ResLat& l : lats) {
+          b->res_cl[l.lat] = c;
+          b->res_from[l.lat] = f;
+        }
       }
-      if (lats.empty() || b->L->resident_clusters(c, r.plan.threads, r.plan.smem, 0) < 1) continue;
-      r.n = (int)lats.size();
-      if (cudaMalloc(&r.d_lats, lats.size() * sizeof(ResLat)) != cudaSuccess) {
-        cudaGetLastError();
-        return CLBM_ENOMEM;
-      }
-      b->resident.push_back(r);
-      BCUDA(b, cudaMemcpy(r.d_lats, lats.data(), lats.size() * sizeof(ResLat), cudaMemcpyHostToDevice));
-      for (const ResLat& l : lats) b->res_cl[l.lat] = c;
-    }
-  b->tiled = std::count(b->res_cl.begin(), b->res_cl.end(), 0) > 0;
-  if (b->resident.size() + (b->tiled ? 1 : 0) > 1 && !b->resident.empty()) {
+  if (branches_at(b, kFromMasked) || branches_at(b, kFromOther)) {
     for (clbm_batch::Resident& r : b->resident) {
       BCUDA(b, cudaStreamCreateWithFlags(&r.side, cudaStreamNonBlocking));
       BCUDA(b, cudaEventCreateWithFlags(&r.done, cudaEventDisableTiming));
@@ -395,11 +437,15 @@ static clbm_status autotune(clbm_batch* b) {
   for (int cls = 0; cls < 4; ++cls) {
     std::vector<int> active(n, 0);
     long long nodes = 0;
-    for (int i = 0; i < n; ++i)
-      if (width_class(b->nx[i]) == cls && !b->res_cl[i]) {
-        active[i] = 1;
-        nodes += b->nodes[i];
-      }
+    for (const int K : {1 << 30, 2}) {  // the tiled lattices, or if there are none those that short intervals tile
+      b->interval = K;
+      for (int i = 0; i < n; ++i)
+        if (width_class(b->nx[i]) == cls && !resident_at(b, i, K)) {
+          active[i] = 1;
+          nodes += b->nodes[i];
+        }
+      if (nodes > 0) break;
+    }
     if (nodes == 0) continue;
     float best_t = 1e30f;
     for (int c = 0; c < nchoice; ++c) {
@@ -423,6 +469,7 @@ static clbm_status autotune(clbm_batch* b) {
       }
     }
   }
+  b->interval = 1 << 30;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   for (int i = 0; i < n; ++i) b->width[i] = best[width_class(b->nx[i])];
@@ -527,9 +574,15 @@ clbm_status clbm_batch_create(const clbm_batch_item* items, int32_t n, int32_t a
     lats[i].snap = b->d_snap + snap_off;
     snap_off += 3 * b->nodes[i];
     b->masked[i] = v.g.flags != nullptr;
-    for (int k = 0; k < v.nb && b->masked[i] && !b->res_cl[i]; ++k) bent.push_back(make_int2(i, v.bnodes_host[k]));
   }
-  b->nbent = (int)bent.size();
+  for (const int from : {1 << 30, kFromOther, kFromMasked}) {  // the last first: those tiled at any interval
+    for (int i = 0; i < n; ++i) {
+      if (!b->masked[i] || (b->res_cl[i] ? b->res_from[i] : 1 << 30) != from) continue;
+      const ViewInfo v = describe_view(b->views[i]);
+      for (int k = 0; k < v.nb; ++k) bent.push_back(make_int2(i, v.bnodes_host[k]));
+    }
+    b->bent.emplace_back(from, (int)bent.size());
+  }
   if (!bent.empty()) {
     if (cudaMalloc(&b->d_bent, bent.size() * sizeof(int2)) != cudaSuccess ||
         cudaMemcpy(b->d_bent, bent.data(), bent.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -601,13 +654,18 @@ clbm_status clbm_batch_lattice(clbm_batch* b, int32_t i, clbm_ctx** view) {
   return CLBM_OK;
 }
 
-clbm_status clbm_batch_launches(const clbm_batch* b, int32_t* resident, int32_t* per_step, int32_t* per_check) {
-  if (!b || !resident || !per_step || !per_check) return CLBM_EINVAL;
+// Steps between checks: even, so that each replay starts and ends in buffer 0.
+static int interval_of(int32_t check_every) { return (check_every + 1) / 2 * 2; }
+
+clbm_status clbm_batch_launches(const clbm_batch* b, int32_t check_every, int32_t* resident, int32_t* per_step,
+                                int32_t* per_check) {
+  if (!b || check_every < 1 || !resident || !per_step || !per_check) return CLBM_EINVAL;
   int used[kBatchGroups] = {};
+  const int K = interval_of(check_every);
   for (int i = 0; i < b->n; ++i)
-    if (!b->res_cl[i]) used[b->group[i]] = 1;
-  *resident = (int32_t)b->resident.size();
-  *per_step = (int32_t)std::count(used, used + kBatchGroups, 1) + (b->nbent > 0 ? 1 : 0);
+    if (!resident_at(b, i, K)) used[b->group[i]] = 1;
+  *resident = (int32_t)launches_at(b, K);
+  *per_step = (int32_t)std::count(used, used + kBatchGroups, 1) + (entries_at(b, K) > 0 ? 1 : 0);
   *per_check = 5;  // residual (two stages), retire, scan, tiles
   return CLBM_OK;
 }
@@ -616,7 +674,8 @@ clbm_status clbm_batch_solve(clbm_batch* b, double tol, int64_t max_steps, int32
                              int64_t* conv_steps, double* residuals, int64_t* steps_run) {
   if (!b || max_steps < 1 || check_every < 1 || !(tol >= 0)) return bfail(b, CLBM_EINVAL, "bad solve arguments");
   const int n = b->n;
-  const int K = (check_every + 1) / 2 * 2;  // even: each replay starts and ends in buffer 0
+  const int K = interval_of(check_every);
+  b->interval = K;
   // start: every lattice active, counters reset, tile lists rebuilt
   std::vector<int> all(n, 1);
   clbm_status st = upload_layout(b, all);
@@ -635,8 +694,9 @@ clbm_status clbm_batch_solve(clbm_batch* b, double tol, int64_t max_steps, int32
     cudaGraph_t graph;
     BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     clbm_status cst = launch_resident(b, K);
-    for (int j = 0; j < K && cst == CLBM_OK && b->tiled; ++j) cst = launch_steps(b, j & 1, j);
-    if (cst == CLBM_OK) cst = join_resident(b);
+    const bool tiled = tiled_at(b, K);
+    for (int j = 0; j < K && cst == CLBM_OK && tiled; ++j) cst = launch_steps(b, j & 1, j);
+    if (cst == CLBM_OK) cst = join_resident(b, K);
     if (cst == CLBM_OK && b->L->batch_residual(b->d_lats, b->d_active, b->d_snap_valid, b->d_res, n, K,
                                                b->d_rpart, b->res_chunks, b->stream) != cudaSuccess)
       cst = CLBM_ECUDA;

@@ -62,11 +62,40 @@ def test_route_and_result(k):
 
 
 def test_batch_launches():
-    small, masked, wide = I.natural_convection_cavity(32, 1e4), I.obstacle_channel(500, 120), I.natural_convection_cavity(400, 1e4)
-    for ws, precision, want in (([small] * 4, "f32", (1, 0, 5)),                # one cluster size
-                                ([small] * 4, "f64", (0, 1, 5)),
-                                ([wide, masked], "f32", (0, 3, 5)),             # a width each, boundary nodes
-                                ([small, wide], "f32", (1, 1, 5))):
+    C = I.natural_convection_cavity
+    small, masked, wide, obstacle = C(32, 1e4), I.obstacle_channel(500, 120), C(400, 1e4), I.obstacle_cavities(1, 32)[0]
+    for ws, precision, K, want in (([small] * 4, "f32", 12, (1, 0, 5)),        # one cluster size
+                                   ([small] * 4, "f32", 10, (0, 1, 5)),        # from intervals of 12 on,
+                                   ([obstacle] * 4, "f32", 6, (1, 0, 5)),      # with a mask of 6
+                                   ([obstacle] * 4, "f32", 3, (0, 2, 5)),      # tiles and their boundary nodes
+                                   ([small] * 4, "f64", 100, (0, 1, 5)),
+                                   ([wide, masked], "f32", 100, (0, 3, 5)),    # without and with a mask
+                                   ([small, wide], "f32", 100, (1, 1, 5)),
+                                   ([small, wide, obstacle], "f32", 8, (1, 1, 5)),
+                                   ([small, wide, obstacle], "f32", 4, (0, 3, 5)),
+                                   ([small, wide, obstacle], "f32", 12, (2, 1, 5))):
         b = clbm.Batch(ws, precision, autotune=False)
-        assert b.launches() == want
+        assert b.launches(K) == want, (precision, K)
         b.close()
+
+
+@pytest.mark.parametrize("precision,rounding", [("f32", 0), ("f16", 1)])
+def test_check_intervals_do_not_change_results(precision, rounding):
+    """Every kind of lattice by the routes that intervals of 2 .. 24 steps choose."""
+    ws = [I.natural_convection_cavity(32, 1e4), I.obstacle_cavities(1, 32)[0], I.natural_convection_cavity(300, 1e4),
+          I.obstacle_cavities(1, 128)[0], I.obstacle_channel(500, 120)]
+    b = clbm.Batch(ws, precision, rounding=rounding)
+    start = [[np.copy(a) for a in b.moments(i)] for i in range(len(ws))]
+    want = None
+    for K in (24, 12, 8, 6, 4, 2, 24):
+        for i, m in enumerate(start):
+            clbm.clbm_init_fields(b.view(i), *m)
+        conv, _, steps = b.solve(0.0, 24, K)
+        assert steps == 24 and (conv == -1).all()
+        got = [b.moments(i) for i in range(len(ws))]
+        if want is None:
+            want = got
+        for x, y in zip(got, want):
+            for p, q in zip(x, y):
+                np.testing.assert_array_equal(p, q, err_msg=str(K))
+    b.close()
