@@ -28,7 +28,9 @@
 // loads V contiguous values of every plane with one 16-byte (8-byte for
 // 16-bit storage) load.  The x-shift of the pull is done with one warp
 // shuffle per plane; lanes 0 and 31 fetch the single value that crosses the
-// warp boundary.  Nodes on box edges and next to solids take a fix-up path.
+// warp boundary.  Box walls and periodic seams are selects of an address in the
+// tiles (box_tile); nodes next to solids, and the edges of lattices with a mask
+// or moving sides, are updated from a list of their own (node_update).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -434,7 +436,8 @@ __host__ __device__ __forceinline__ void collide(const Co<R>& c, R (&d)[9], R (&
   h[4] = sub_(q02, q01);
 }
 
-// HK is of no effect: every storage type takes the same constants.
+// (HK selects nothing: every storage type takes the same constants.  The host harness of the
+// collision's tests names it.)
 template <typename R, bool HK = true>
 __host__ __device__ __forceinline__ void collide_any(const Co<R>& c, bool vh, R (&d)[9], R (&h)[5],
                                                      R& qv) {
@@ -695,16 +698,17 @@ __device__ __forceinline__ void step_wait() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
 
-// Interior update.  One warp updates the 32 * V nodes x = xw .. xw + 32V - 1
-// of row y (each lane owns V consecutive nodes); all 32 lanes must call it
-// together.  Every node is pulled and collided as if it were an interior
-// fluid node: rows beyond a non-periodic edge are clamped and the ±1 x-shift
-// at the row ends reads a neighbour, so box edges, periodic seams and nodes
-// next to solids come out wrong here and are recomputed afterwards by the
-// boundary kernel from its precomputed node list.  Keeping the walls out of
-// this kernel keeps its warps free of divergent wall code.
-template <typename S, int V, bool SKIP_EDGES = false, bool VH = false, bool SKIP_DEAD = true,
-          bool MASKSTORE = false>
+// Interior update of lattices with a mask or moving sides.  One warp updates
+// the 32 * V nodes x = xw .. xw + 32V - 1 of row y (each lane owns V consecutive
+// nodes); all 32 lanes must call it together.  Every node is pulled and collided
+// as if it were an interior fluid node: rows beyond a non-periodic edge are
+// clamped and the ±1 x-shift at the row ends reads a neighbour, so what comes
+// out for the first and last column (and, next to solids, for flagged nodes) is
+// wrong.  Those nodes are the boundary list's: the tile leaves them out, or
+// (MASKSTORE false) writes the flagged ones provisionally before a boundary
+// launch replaces them.  Keeping the walls out keeps the warps free of divergent
+// wall code.
+template <typename S, int V, bool VH, bool SKIP_DEAD, bool MASKSTORE>
 __device__ __forceinline__ void step_tile(const DevGeom& g, const Co<typename Traits<S>::R>& c,
                                           const S* __restrict__ src, S* __restrict__ dst, int y,
                                           int xw, int lane, uint32_t seed, int stochastic,
@@ -819,29 +823,23 @@ __device__ __forceinline__ void step_tile(const DevGeom& g, const Co<typename Tr
     }
   }
   if constexpr (VH) {  // the viscous source of this step, read back with T (15th plane)
-    if constexpr (SKIP_EDGES) {
 #pragma unroll
-      for (int k = 0; k < V; ++k) {
-        const int x = x0 + k;
-        if (x != 0 && x != g.nx - 1) out[14 * plane + k] = from_r<S, R>(qv[k]);
-      }
-    } else {
-      stv<S, V>(out + 14 * plane, qv);
+    for (int k = 0; k < V; ++k) {
+      const int x = x0 + k;
+      if (x != 0 && x != g.nx - 1) out[14 * plane + k] = from_r<S, R>(qv[k]);
     }
   }
-  if constexpr (SKIP_EDGES) {
-    // leave the first and last column to the boundary update running alongside
-    if (x0 == 0 || (x0 <= g.nx - 1 && g.nx - 1 < x0 + V)) {
+  // leave the first and last column to the boundary update running alongside
+  if (x0 == 0 || (x0 <= g.nx - 1 && g.nx - 1 < x0 + V)) {
 #pragma unroll
-      for (int k = 0; k < V; ++k) {
-        const int x = x0 + k;
-        if (x == 0 || x == g.nx - 1) continue;
-        const uint32_t key = sr_key(seed, (long long)(y + g.yoff) * g.pitch + (x & ~3));
+    for (int k = 0; k < V; ++k) {
+      const int x = x0 + k;
+      if (x == 0 || x == g.nx - 1) continue;
+      const uint32_t key = sr_key(seed, (long long)(y + g.yoff) * g.pitch + (x & ~3));
 #pragma unroll
-        for (int q = 0; q < 14; ++q) st1<S, R>(out + q * plane + k, v[q][k], stochastic, key, q, x & 3);
-      }
-      return;
+      for (int q = 0; q < 14; ++q) st1<S, R>(out + q * plane + k, v[q][k], stochastic, key, q, x & 3);
     }
+    return;
   }
   if constexpr (sizeof(S) == 2) {
     if (stochastic) {
@@ -1104,13 +1102,11 @@ __global__ void __launch_bounds__(kStepThreads, kStepBlocks<S>) step_fused_kerne
   if constexpr (MASKED) {  // tile classes: 0 no fluid, 1 unflagged fluid, 2 holds flagged nodes
     const uint8_t cls = a.g.tile_fluid[(long long)y * a.g.tiles_per_row + warp];
     if (!cls) return;
-    step_tile<S, V, true, VH, sizeof(S) != 2, true>(a.g, c, static_cast<const S*>(a.src),
-                                                    static_cast<S*>(a.dst), y, xw, lane, step_seed(a),
-                                                    a.stochastic, cls == 2);
+    step_tile<S, V, VH, sizeof(S) != 2, true>(a.g, c, static_cast<const S*>(a.src), static_cast<S*>(a.dst), y, xw, lane,
+                                              step_seed(a), a.stochastic, cls == 2);
   } else {
-    step_tile<S, V, true, VH, sizeof(S) != 2>(a.g, c, static_cast<const S*>(a.src),
-                                              static_cast<S*>(a.dst), y, xw, lane, step_seed(a),
-                                              a.stochastic);
+    step_tile<S, V, VH, sizeof(S) != 2, false>(a.g, c, static_cast<const S*>(a.src), static_cast<S*>(a.dst), y, xw, lane,
+                                               step_seed(a), a.stochastic);
   }
 }
 
@@ -1526,7 +1522,7 @@ __global__ void __launch_bounds__(kStepThreads, (kBatchBlocks<S, V, MASKED>))
     const S* src = static_cast<const S*>(L.buf[parity]);
     S* dst = static_cast<S*>(L.buf[parity ^ 1]);
     if constexpr (MASKED) {
-      step_tile<S, V, true, false>(L.g, c, src, dst, tl.y, tl.z, lane, seed, stochastic);
+      step_tile<S, V, false, true, false>(L.g, c, src, dst, tl.y, tl.z, lane, seed, stochastic);
     } else {
       // one copy of the tile: rows of a few hundred nodes are mostly edge tiles anyway
       box_tile<S, V, false, true, true>(L.g, coef[wib], src, dst, tl.y, tl.z, lane, seed, stochastic);

@@ -3,7 +3,7 @@
 // A small lattice advanced by one launch per step is bound by latency: a 64 x
 // 64 step moves 0.9 MB through L2 but takes the launch, the cold start of its
 // blocks and the boundary nodes' chain of loads, 5.0 us (1.9 us here; 128 x
-// 128 FP32 2.3; 64 batched obstacle cavities of 64 x 64 66 -> 27 us).  Here a cluster of up
+// 128 FP32 2.3; 256 batched obstacle cavities of 64 x 64 66 -> 28 us).  Here a cluster of up
 // to sixteen thread blocks holds both states of the lattice in shared memory
 // (each block a band of rows with a ghost row on either side), takes any
 // number of steps with one cluster barrier each, and writes the last two
@@ -19,7 +19,7 @@
 // 3.0 -> 2.3 us).  A step is then as long as the chain load - collide - store
 // - cluster barrier of one block; arriving at the barrier early and waiting
 // late made it longer (2.3 -> 2.65 us), as did fewer threads and more blocks
-// a multiprocessor (64 batched cavities 33 -> 34 .. 47 us).
+// a multiprocessor (256 batched obstacle cavities 33 -> 34 .. 47 us).
 #pragma once
 
 namespace clbm {
