@@ -557,7 +557,7 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
                 double* const to = &lk_t[heat_entry(s, i)];
                 auto put = [&](const auto& rates, auto type) {
                   decltype(type) r[4];
-                  round_heat(kt, b.b2, heat_share(rates), r);
+                  round_heat(kt, b.b2, heat_share(rates, c->p.cT2), r);
                   for (int m = 0; m < 4; ++m) to[m] = r[m];
                 };
                 if (c->p.precision == CLBM_F64)
@@ -612,8 +612,8 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
         if (sides[s] >= 0) {
           const clbm_tbc& b = tbc[sides[s]];
           link_heat(b.b1, b.b2, b.b3, 1.0, 0.5, two != 0, false, c->p.T0, 0.5 * c->p.Q, c->p.cT2, k);
-          round_heat(k, b.b2, heat_share(co.kd), kd);
-          round_heat(k, b.b2, heat_share(co.kf), kf);
+          round_heat(k, b.b2, heat_share(co.kd, c->p.cT2), kd);
+          round_heat(k, b.b2, heat_share(co.kf, c->p.cT2), kf);
         }
         std::copy(kd, kd + 3, c->side_k[s][two]);
         std::copy(kf, kf + 3, c->side_kf[s][two]);

@@ -5,6 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+#include <limits>
+
 #include "../../include/clbm.h"
 
 namespace clbm {
@@ -80,10 +83,12 @@ struct CollideK {
 };
 
 // (h_1 + h_3) / (T - T0) of a uniform state at rest that the collision leaves as it is: G20 =
-// l2m2 (2 G20) + srct2 (T - T0), with the constants as rounded.
+// l2m2 (2 G20) + srct2 (T - T0), with the constants as rounded.  The rounding of l2m2 weighs as 1 / l2 in
+// it: where l2 is so small that it says nothing any more (below 5e-4 in FP32), cT2 itself.
 template <typename T>
-inline double heat_share(const CollideK<T>& k) {
-  return 2.0 * (double)k.srct2 / (1.0 - 2.0 * (double)k.l2m2);
+inline double heat_share(const CollideK<T>& k, double cT2) {
+  const double s = 2.0 * (double)k.srct2 / (1.0 - 2.0 * (double)k.l2m2);
+  return std::fabs(s - cT2) <= 1024.0 * (double)std::numeric_limits<T>::epsilon() * cT2 ? s : cT2;
 }
 
 struct DevCoef {

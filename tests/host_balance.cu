@@ -15,12 +15,12 @@ extern "C" void host_round_heat(double b1, double b2, double b3, double ne, doub
   double k[4], d[4];
   float f[4];
   clbm::link_heat(b1, b2, b3, ne, q, have2 != 0, have3 != 0, 0.5, 1e-5, cT2, k);
-  clbm::round_heat(k, b2, clbm::heat_share(c.kd), d);
-  clbm::round_heat(k, b2, clbm::heat_share(c.kf), f);
+  clbm::round_heat(k, b2, clbm::heat_share(c.kd, cT2), d);
+  clbm::round_heat(k, b2, clbm::heat_share(c.kf, cT2), f);
   for (int i = 0; i < 4; ++i) {
     o[i] = d[i];
     o[5 + i] = f[i];
   }
-  o[4] = clbm::heat_share(c.kd);
-  o[9] = clbm::heat_share(c.kf);
+  o[4] = clbm::heat_share(c.kd, cT2);
+  o[9] = clbm::heat_share(c.kf, cT2);
 }

@@ -59,3 +59,14 @@ def test_other_walls_are_rounded_one_by_one(harness):
         harness.host_round_heat(b1, b2, 0.2, 0.9, q, have2, have3, 1.1, 0.4, k)
         for m in range(4):
             assert np.float32(k[m]) == k[5 + m]
+
+
+@pytest.mark.parametrize("l2", [1e-3, 1e-4, 1e-6, 1e-8, 1e-12, 1e-17])
+def test_small_rates(harness, l2):
+    """The rounded constants of a rate near zero say nothing about the share (1 - l2
+    may round to 1): the weights stay at cT2."""
+    k = (C.c_double * 10)()
+    for q, have2 in itertools.product(FRACTIONS, (0, 1)):
+        harness.host_round_heat(1.0, 0.0, 0.1, 0.9, q, have2, 0, l2, 0.4, k)
+        for off, R in ((0, np.float64), (5, np.float32)):
+            assert abs(k[off] + k[off + 1] - 0.4) <= 1026 * float(np.finfo(R).eps) * 0.4, (q, have2, R)
