@@ -462,7 +462,7 @@ clbm_status clbm_set_boundaries(clbm_ctx* c, const uint8_t* solid, const clbm_tb
       int32_t& s = slot_of[(size_t)y * nx + x];
       if (s < 0) {
         if (lk_tbc.size() / 4 >= (size_t)kMaxLinkSlots)
-          return fail(c, CLBM_EINVAL, "more than 2^29 nodes with wall links");
+          return fail(c, CLBM_EINVAL, "more than 2^28 nodes with wall links");
         s = (int32_t)(lk_tbc.size() / 4);
         lk_ne.insert(lk_ne.end(), 4, 0.0);
         lk_tbc.insert(lk_tbc.end(), 4, -1);

@@ -11,5 +11,5 @@ extern "C" int host_band_holds_third(int y, int dir, int ny, int cl, int py) {
 extern "C" int host_slab_holds_third(int y, int gy, int dir, int ny, int NY, int py) {
   return clbm::slab_holds_third(y, gy, dir, ny, NY, py != 0);
 }
-extern "C" long long host_heat_entry(int slot, int dir) { return clbm::heat_entry(slot, dir); }
+extern "C" long long host_heat_entry(int slot, int dir) { return (long long)clbm::heat_entry(slot, dir); }
 extern "C" long long host_bounce_entry(int slot, int dir) { return clbm::bounce_entry(slot, dir); }
