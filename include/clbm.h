@@ -142,7 +142,8 @@ clbm_status clbm_create(const clbm_params* params, void* stream, clbm_ctx** out)
  *              every D2Q5 link from a fluid node into a solid node must be listed
  * All inputs are copied.  The distribution state is left unchanged.
  * Errors: CLBM_EINVAL for out-of-range indices, a missing link, a fluid node
- * with no fluid neighbour, or a non-periodic side without a condition. */
+ * with no fluid neighbour, a non-periodic side without a condition, or more than
+ * 2^28 nodes with listed links. */
 clbm_status clbm_set_boundaries(clbm_ctx* ctx, const uint8_t* solid, const clbm_tbc* tbc,
                                 int32_t n_tbc, const int32_t* side_tbc, const clbm_link* links,
                                 int32_t n_links);
